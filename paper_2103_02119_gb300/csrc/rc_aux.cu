@@ -94,74 +94,103 @@ __global__ void init_kernel(double* __restrict__ f, const AuxParams p, const dou
 // of rows, keeping the FP32 state (r - rho0, u, v) of the rows y - 1, y,
 // y + 1 and of one column either side in shared memory, so that each cell's
 // FP64 input is converted once rather than once per population.
-constexpr int kInitRows = 16;  // rows of a band (more when ny / 16 > 65535)
+//
+// Bound by the latency of the FP64 reads, then by memory: the row after the
+// next is fetched into registers while a row is written, and a ring of four
+// rows needs one barrier a row (a row's slot is written again two barriers
+// after its last read).  Small lattices take short bands (init_rows), so
+// that a launch is not one block's march.
+constexpr int kInitRows = 16;  // most rows of a band (more when ny / 16 > 65535)
+constexpr int kInitThreads = kThreads + 32;  // one column a thread; a last warp for the two halo columns
 
 template <bool MASK>
-__global__ void __launch_bounds__(kThreads)
-init32_kernel(float* __restrict__ f, const AuxParams p, const double* rho, const double* ux,
-              const double* uy, int rows) {
+__global__ void __launch_bounds__(kInitThreads)
+init32_kernel(float* __restrict__ f, const AuxParams p, const double* __restrict__ rho,
+              const double* __restrict__ ux, const double* __restrict__ uy, int rows) {
     constexpr int SW = kThreads + 2;
-    __shared__ float st[3][3][SW];  // [component][ring row][column x - x0 + 1]
+    __shared__ float st[3][4][SW];  // [component][ring row][column x - x0 + 1]
     const Feq32 feq{(float)p.cs2, (float)p.a, (float)(0.5 / (p.a * p.a)), (float)p.rho0};
     const int tx = threadIdx.x;
     const int x0 = blockIdx.x * kThreads;
     const int w = min(kThreads, p.nx - x0);
     const int y0 = blockIdx.y * rows;
     const int y1 = min(p.ny, y0 + rows);
-    // ring slot of row yy in [y0 - 1, y1]
-    auto slot = [&](int yy) { return (yy - y0 + 1) % 3; };
-    auto load_row = [&](int yy) {
-        const int k = slot(yy);
+    if (w <= 0 || y0 >= p.ny) return;
+    // the ring column this thread fetches (-1: none): its own, or a halo one
+    const int c = tx < w ? tx + 1 : tx == kThreads ? 0 : tx == kThreads + 1 ? w + 1 : -1;
+    int gx = x0 - 1 + c;
+    if (gx < 0) gx = p.px ? gx + p.nx : -1;
+    else if (gx >= p.nx) gx = p.px ? gx - p.nx : -1;
+    if (c < 0) gx = -1;
+    double qr, qu, qv;
+    auto fetch = [&](int yy) {  // outside a wall: the rest state, which nothing reads
         int gy = yy;
         if (gy < 0) gy = p.py ? gy + p.ny : -1;
         else if (gy >= p.ny) gy = p.py ? gy - p.ny : -1;
-        for (int c = tx; c < w + 2; c += kThreads) {
-            int gx = x0 - 1 + c;
-            if (gx < 0) gx = p.px ? gx + p.nx : -1;
-            else if (gx >= p.nx) gx = p.px ? gx - p.nx : -1;
-            float dr = 0.0f, u = 0.0f, v = 0.0f;  // outside a wall: never read
-            if (gx >= 0 && gy >= 0) {
-                const long long t = (long long)gy * p.nx + gx;
-                dr = (float)((rho ? rho[t] : 1.0) - p.rho0);
-                u = ux ? (float)ux[t] : 0.0f;
-                v = uy ? (float)uy[t] : 0.0f;
-            }
-            st[0][k][c] = dr;
-            st[1][k][c] = u;
-            st[2][k][c] = v;
-        }
+        qr = p.rho0;
+        qu = qv = 0.0;
+        if (gx < 0 || gy < 0) return;
+        const long long t = (long long)gy * p.nx + gx;
+        qr = rho ? rho[t] : 1.0;
+        if (ux) qu = ux[t];
+        if (uy) qv = uy[t];
     };
-    if (w <= 0 || y0 >= p.ny) return;
-    load_row(y0 - 1);
-    load_row(y0);
+    auto slot = [&](int yy) { return (yy - y0 + 1) & 3; };
+    auto put = [&](int yy) {
+        if (c < 0) return;
+        const int s = slot(yy);
+        st[0][s][c] = (float)(qr - p.rho0);
+        st[1][s][c] = (float)qu;
+        st[2][s][c] = (float)qv;
+    };
+    fetch(y0 - 1);
+    const double r0 = qr, u0 = qu, v0 = qv;
+    fetch(y0);
+    const double r1 = qr, u1 = qu, v1 = qv;
+    fetch(y0 + 1);
+    const double r2 = qr, u2 = qu, v2 = qv;
+    qr = r0, qu = u0, qv = v0;
+    put(y0 - 1);
+    qr = r1, qu = u1, qv = v1;
+    put(y0);
+    qr = r2, qu = u2, qv = v2;
     for (int y = y0; y < y1; ++y) {
-        load_row(y + 1);
+        put(y + 1);
         __syncthreads();
-        if (tx < w) {
-            const int x = x0 + tx;
-            const long long o = (long long)y * p.rstride + x;
-            const unsigned sb = link_bits<MASK>(p, x, y);
-            if (sb == 0xFFu) {
+        if (y + 1 < y1) fetch(y + 2);
+        if (tx >= w) continue;
+        const int x = x0 + tx;
+        const long long o = (long long)y * p.rstride + x;
+        const unsigned sb = link_bits<MASK>(p, x, y);
+        if (sb == 0xFFu) {
 #pragma unroll
-                for (int i = 0; i < 9; ++i) f[i * p.plane + o] = 0.0f;
-            } else {
-                const int k = slot(y), c = tx + 1;
-#pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    float v;
-                    if (i > 0 && ((sb >> (opp(i) - 1)) & 1u)) {
-                        // pulled back by the cell itself
-                        v = feq(opp(i), st[0][k][c], st[1][k][c], st[2][k][c]);
-                    } else {
-                        const int kk = slot(y + ey(i)), cc = c + ex(i);
-                        v = feq(i, st[0][kk][cc], st[1][kk][cc], st[2][kk][cc]);
-                    }
-                    f[i * p.plane + o] = v;
-                }
-            }
+            for (int i = 0; i < 9; ++i) f[i * p.plane + o] = 0.0f;
+            continue;
         }
-        __syncthreads();  // row y - 1's slot is overwritten next
+        const int k = slot(y);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            float v;
+            if (i > 0 && ((sb >> (opp(i) - 1)) & 1u)) {
+                // pulled back by the cell itself
+                v = feq(opp(i), st[0][k][c], st[1][k][c], st[2][k][c]);
+            } else {
+                const int kk = slot(y + ey(i)), cc = c + ex(i);
+                v = feq(i, st[0][kk][cc], st[1][kk][cc], st[2][kk][cc]);
+            }
+            f[i * p.plane + o] = v;
+        }
     }
+}
+
+// Rows of an init32_kernel band: kInitRows where the blocks then fill the
+// GPU (about eight 256-thread blocks on each of 152 SMs), fewer on smaller
+// lattices, down to one.
+int init_rows(int nx, int ny) {
+    const long long segs = (nx + kThreads - 1) / kThreads;
+    const long long fit = segs * ny / 1216;
+    const int rows = (int)(fit < 1 ? 1 : fit < kInitRows ? fit : kInitRows);
+    return max(rows, (ny + 65534) / 65535);  // grid.y limit
 }
 
 template <typename T, bool MASK>
@@ -588,10 +617,10 @@ template <typename T>
 cudaError_t launch_init(T* f, const AuxParams& p, const double* rho, const double* ux,
                         const double* uy, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
-        const int rows = max(kInitRows, (p.ny + 65534) / 65535);  // grid.y limit
+        const int rows = init_rows(p.nx, p.ny);
         const dim3 g((p.nx + kThreads - 1) / kThreads, (p.ny + rows - 1) / rows);
-        if (p.lmask) init32_kernel<true><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy, rows);
-        else init32_kernel<false><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy, rows);
+        if (p.lmask) init32_kernel<true><<<g, kInitThreads, 0, s>>>(f, p, rho, ux, uy, rows);
+        else init32_kernel<false><<<g, kInitThreads, 0, s>>>(f, p, rho, ux, uy, rows);
     } else {
         const dim3 g = grid2_for(p.nx, p.ny);
         if (p.lmask) init_kernel<true><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
