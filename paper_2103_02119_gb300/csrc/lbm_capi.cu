@@ -277,6 +277,12 @@ AuxParams aux_of(const lbm_params& q, const Geometry& g) {
     a.w3 = q.omega[3];
     a.w4 = q.omega[4];
     a.w5 = q.omega[5];
+    a.a32 = (float)q.a;
+    a.cs232 = (float)q.cs2;
+    a.iah232 = (float)(0.5 / (q.a * q.a));
+    a.rho032 = (float)q.rho0;
+    a.hFx32 = 0.5f * (float)q.Fx;
+    a.hFy32 = 0.5f * (float)q.Fy;
     a.lmask = g.lmask;
     return a;
 }
@@ -717,14 +723,12 @@ lbm_status lbm_stress(lbm_handle* h, double* dxux, double* dyuy, double* sxy, do
     const AuxParams a = aux(h);
     cudaError_t e;
     if (h->p.precision == 64) {
-        e = lbm::launch_moments<double>((const double*)h->f[h->cur], a, rho, nullptr, nullptr,
-                                        h->stream, true);
+        e = lbm::launch_density<double>((const double*)h->f[h->cur], a, rho, h->stream);
         if (e == cudaSuccess)
             e = lbm::launch_stress<double>((const double*)h->f[h->cur], a, rho, d[0], d[1], d[2],
                                            d[3], d[4], d[5], h->stream);
     } else {
-        e = lbm::launch_moments<float>((const float*)h->f[h->cur], a, rho, nullptr, nullptr,
-                                       h->stream, true);
+        e = lbm::launch_density<float>((const float*)h->f[h->cur], a, rho, h->stream);
         if (e == cudaSuccess)
             e = lbm::launch_stress<float>((const float*)h->f[h->cur], a, rho, d[0], d[1], d[2],
                                           d[3], d[4], d[5], h->stream);
@@ -834,18 +838,16 @@ lbm_status lbm_diagnostics(lbm_handle* h, double out[LBM_DIAG_COUNT]) {
     cudaError_t e = h->p.precision == 64
                         ? lbm::launch_diag<double>((const double*)h->f[h->cur], (const double*)prev,
                                                    a, h->uprev, have, h->part, h->diag_blocks,
-                                                   h->stream)
+                                                   h->status, h->stream)
                         : lbm::launch_diag<float>((const float*)h->f[h->cur], (const float*)prev, a,
                                                   h->uprev, have, h->part, h->diag_blocks,
-                                                  h->stream);
+                                                  h->status, h->stream);
     CK(h, e, "diagnostics kernels");
-    DiagPartial r;
+    DiagPartial r;  // with the status word: one copy
     CK(h, cudaMemcpyAsync(&r, h->part + h->diag_blocks, sizeof(r), cudaMemcpyDeviceToHost, h->stream),
        "cudaMemcpyAsync(D2H)");
-    int kstatus = 0;
-    CK(h, cudaMemcpyAsync(&kstatus, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream),
-       "cudaMemcpyAsync(D2H)");
     CK(h, cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    const int kstatus = (int)r.status;
     if (kstatus) return status_error(h, kstatus);
     out[0] = fixed_to_double(r.limb) + (double)h->n_fluid * h->p.rho0;
     out[1] = r.mx;
@@ -979,18 +981,18 @@ extern "C" lbm_status lbm_diagnostics_noalloc(lbm_handle* h, double out[LBM_DIAG
     const void* prev = h->steps >= 1 ? h->f[h->cur ^ 1] : nullptr;
     cudaError_t e = h->p.precision == 64
                         ? lbm::launch_diag<double>((const double*)h->f[h->cur], (const double*)prev,
-                                                   a, uref, have, part, h->diag_blocks, h->stream)
+                                                   a, uref, have, part, h->diag_blocks, h->status,
+                                                   h->stream)
                         : lbm::launch_diag<float>((const float*)h->f[h->cur], (const float*)prev, a,
-                                                  uref, have, part, h->diag_blocks, h->stream);
+                                                  uref, have, part, h->diag_blocks, h->status,
+                                                  h->stream);
     CK(h, e, "diagnostics kernels");
     DiagPartial r;
     CK(h, cudaMemcpyAsync(&r, part + h->diag_blocks, sizeof(r), cudaMemcpyDeviceToHost,
                           h->stream),
        "cudaMemcpyAsync(D2H)");
-    int kstatus = 0;
-    CK(h, cudaMemcpyAsync(&kstatus, h->status, sizeof(int), cudaMemcpyDeviceToHost, h->stream),
-       "cudaMemcpyAsync(D2H)");
     CK(h, cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    const int kstatus = (int)r.status;
     if (kstatus) {
         // the state is not valid: no values, and no residual reference taken
         return status_error(h, kstatus);

@@ -21,7 +21,9 @@ struct DiagPartial {
     double mx, my, en, dres, ures, sres;
     long long nonfinite;
     long long limb[kMassLimbs];
+    long long status;  // final result only: the step kernels' status word
 };
+constexpr int kDiagReals = 6;  // mx .. sres
 
 template <typename T>
 cudaError_t launch_step(const T* fin, T* fout, const KParams<T>& p, int bx, int nbands,
@@ -155,14 +157,16 @@ cudaError_t launch_set_f(T* f, const AuxParams& p, const double* fin, cudaStream
 // post-stream distributions / moments of the state (device outputs)
 template <typename T>
 cudaError_t launch_get_f(const T* f, const AuxParams& p, double* fout, cudaStream_t s);
-// exact64: rho and u in FP64 arithmetic (diagnostics, stress); otherwise FP32
-// storage is read out in FP32 (rho = rho0 + d still in FP64).
+// FP32 storage is read out in FP32 (rho = rho0 + d in FP64).
 template <typename T>
 cudaError_t launch_moments(const T* f, const AuxParams& p, double* rho, double* ux,
-                           double* uy, cudaStream_t s, bool exact64 = false);
+                           double* uy, cudaStream_t s);
+// the density field in FP64 arithmetic (0 in solid cells)
+template <typename T>
+cudaError_t launch_density(const T* f, const AuxParams& p, double* rho, cudaStream_t s);
 // Local strain rates and viscous stress (FP64, nullable outputs of nx*ny
 // doubles) of the state; rho: the density field of the same state (from
-// launch_moments).
+// launch_density).
 template <typename T>
 cudaError_t launch_stress(const T* f, const AuxParams& p, const double* rho, double* dxux,
                           double* dyuy, double* sxy, double* txx, double* tyy, double* txy,
@@ -170,9 +174,11 @@ cudaError_t launch_stress(const T* f, const AuxParams& p, const double* rho, dou
 // diagnostics: per-block partials into `part` (nblocks entries) then a final
 // reduction into part[nblocks]; fprev: the state one step earlier (nullable:
 // the residual then uses u(n) alone); uprev (2*nx*ny doubles) is read (if
-// have_prev) and overwritten with the two-step mean velocity.
+// have_prev) and overwritten with the two-step mean velocity; status: the
+// device word that part[nblocks].status is copied from.
 template <typename T>
 cudaError_t launch_diag(const T* f, const T* fprev, const AuxParams& p, double* uprev,
-                        int have_prev, DiagPartial* part, int nblocks, cudaStream_t s);
+                        int have_prev, DiagPartial* part, int nblocks, const int* status,
+                        cudaStream_t s);
 
 }  // namespace lbm

@@ -15,12 +15,6 @@ namespace {
 
 constexpr int kThreads = 256;
 
-__device__ __forceinline__ double feq_d(int i, double rho, double ux, double uy,
-                                        double cs2, double a) {
-    const double iah2 = 0.5 / (a * a);
-    return rho * phi_x<double>(ex(i), ux, cs2) * phi_y<double>(ey(i), uy, cs2, a, iah2);
-}
-
 // Target cell of direction i from (x, y), wrapped on periodic axes.  Only
 // called when the target is a fluid cell (so inside the domain).
 __device__ __forceinline__ long long target(const AuxParams& p, int x, int y, int i) {
@@ -28,13 +22,6 @@ __device__ __forceinline__ long long target(const AuxParams& p, int x, int y, in
     if (tx < 0) tx += p.nx; else if (tx >= p.nx) tx -= p.nx;
     if (ty < 0) ty += p.ny; else if (ty >= p.ny) ty -= p.ny;
     return (long long)ty * p.nx + tx;
-}
-
-// f_i^eq(r, u, v) - w_i rho0, the stored deviation of an equilibrium.  FP64
-// storage evaluates f^eq in FP64 and subtracts the rest part.
-__device__ __forceinline__ double feq_dev64(int i, double r, double u, double v,
-                                            const AuxParams& p) {
-    return feq_d(i, r, u, v, p.cs2, p.a) - p.wrest[i];
 }
 
 // FP32 storage carries the rest part analytically, as the step does: with
@@ -64,28 +51,203 @@ struct Feq32 {
         for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < (p).nx;                  \
              x += gridDim.x * blockDim.x)
 
+// Cells in tiles of kThreads: one row of 256 columns, or 2, 4, 8 rows of 128,
+// 64, 32 on narrow lattices; a block takes tiles blockIdx.x, + gridDim.x, ...
+// (one division of a tile index, the same for the whole block, instead of
+// one of a cell index per thread).
+struct Tiles {
+    int sh, ntx, n;
+    __host__ __device__ Tiles(int nx, int ny) {
+        sh = nx <= 32 ? 5 : nx <= 64 ? 6 : nx <= 128 ? 7 : 8;
+        ntx = (nx + (1 << sh) - 1) >> sh;
+        const int rows = kThreads >> sh;
+        n = ntx * ((ny + rows - 1) / rows);
+    }
+    __device__ __forceinline__ int y(int t) const {
+        return t / ntx * (kThreads >> sh) + ((int)threadIdx.x >> sh);
+    }
+    __device__ __forceinline__ int x(int t) const {
+        return (t % ntx << sh) + ((int)threadIdx.x & ((1 << sh) - 1));
+    }
+};
+#define LBM_FOR_TILES(p, t)            \
+    const Tiles tiles((p).nx, (p).ny); \
+    for (int t = blockIdx.x; t < tiles.n; t += gridDim.x)
+
+// GB300 has two FP64 lanes per SM (against 128 FP32 and 64 integer ones): the
+// read-out kernels are bound by them, and by conversions, which take the same
+// lanes.  So they spend FP64 on what needs it and the rest on integers.
+// Measured on 2048 x 2047 FP32 cells with obstacles, against sums, conversions
+// and divisions in FP64: lbm_stress 558 against 2085 us, lbm_diagnostics after a
+// step 380 against 1260 us, lbm_get_f 84 against 146 us, lbm_set_f 91 against
+// 143 us, lbm_moments 51 against 68 us; the residual check of a 96-lattice batch
+// 0.75 against 2.56 ms.
+
+// float -> double, exact, on the integer pipe, without a branch (a conversion
+// instruction under a predicate takes its place in the FP64 pipe even where
+// the predicate is false).
+__device__ __forceinline__ double widen(float f) {
+    const bool tiny = (__float_as_uint(f) & 0x7F800000u) == 0u;  // subnormal or zero
+    const unsigned u = __float_as_uint(tiny ? f * 18446744073709551616.0f : f);  // 2^64
+    const unsigned m = u & 0x7FFFFFFFu;
+    unsigned hi = (m >> 3) + (tiny ? 0x38000000u - (64u << 20) : 0x38000000u);
+    if (m >= 0x7F800000u) hi += 0x38000000u;  // Inf, NaN
+    return __hiloint2double((int)((u & 0x80000000u) | (m ? hi : 0u)), (int)(m << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
+// double -> float, rounded to nearest even, on the integer pipe; values that
+// are not normal floats below 2^127 (zero aside) through a call.
+__device__ __noinline__ float narrow_any(double d) { return (float)d; }
+__device__ __forceinline__ float narrow(double d) {
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned m = hi & 0x7FFFFFFFu;
+    unsigned u = ((m - 0x38000000u) << 3) | (lo >> 29);
+    const unsigned rest = lo << 3;
+    u += (rest > 0x80000000u || (rest == 0x80000000u && (u & 1u))) ? 1u : 0u;
+    if (m - 0x38100000u >= 0x47E00000u - 0x38100000u) {
+        if (m | lo) return narrow_any(d);
+        u = 0u;
+    }
+    return __uint_as_float((hi & 0x80000000u) | u);
+}
+
+// 1 / a for normal a away from the ends of the range: the hardware's
+// approximation (about 2^-23) and two Newton steps, four FP64 operations
+// (below 1 ulp; an IEEE division takes two to three times as many).
+__device__ __forceinline__ double rcp64(double a) {
+    double x;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(a));
+    x = fma(x, fma(-a, x, 1.0), x);
+    return fma(x, fma(-a, x, 1.0), x);
+}
+__device__ __forceinline__ bool rcp64_ok(double a) {  // 2^-900 <= |a| < 2^900
+    const unsigned m = (unsigned)__double2hiint(a) & 0x7FFFFFFFu;
+    return m - ((1023u - 900u) << 20) < (1800u << 20);
+}
+
+// Sums of the nine deviations of a cell: d = sum g, jx = sum g e_x, jy = sum
+// g e_y, sxx = sum g e_x^2, syy, sxy likewise (e_y in units of a).
+struct Raw {
+    double d, jx, jy, sxx, syy, sxy;
+};
+template <typename T>
+__device__ __forceinline__ Raw raw_sums64(const T g[9]) {
+    double w[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) w[i] = widen(g[i]);
+    const double se = w[5] + w[8], sw = w[6] + w[7], sm = w[2] + w[4];
+    const double ke = w[1] + se, kw = w[3] + sw;
+    const double de = w[5] - w[8], dw = w[6] - w[7];
+    Raw r;
+    r.sxx = ke + kw;
+    r.d = (w[0] + sm) + r.sxx;
+    r.jx = ke - kw;
+    r.jy = (w[2] - w[4]) + (de + dw);
+    r.syy = sm + (se + sw);
+    r.sxy = de - dw;
+    return r;
+}
+
+// FP32 storage: the deviations as multiples of 2^-kFixedShift in 64-bit
+// integers, where all nine are exact (each zero, or between 2^-35 and 2 in
+// magnitude), so that the sums are exact and cost integer instructions.
+constexpr int kFixedShift = 58;
+__device__ __forceinline__ bool fixed_of(float f, long long& v) {
+    const unsigned u = __float_as_uint(f), m = u & 0x7FFFFFFFu;
+    const int sh = (int)(m >> 23) - (150 - kFixedShift);
+    const unsigned long long a = (unsigned long long)((m & 0x007FFFFFu) | 0x00800000u) << (sh & 63);
+    v = (int)u < 0 ? -(long long)a : (long long)a;
+    if (m == 0u) v = 0;
+    return m == 0u || (sh >= 0 && m < 0x40000000u);
+}
+// a nonzero integer multiple of 2^-kFixedShift as a double (one rounding)
+__device__ __forceinline__ double unfixed(long long v) {
+    const double d = __ll2double_rn(v);
+    const int hi = __double2hiint(d);
+    return __hiloint2double(v ? hi - (kFixedShift << 20) : 0, __double2loint(d));
+}
+// fixed: d in the fixed point (valid when the result is true)
+__device__ __forceinline__ bool raw_sums(const float g[9], Raw& r, long long& fixed) {
+    long long w[9];
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) ok &= fixed_of(g[i], w[i]);
+    fixed = 0;
+    if (!ok) {
+        r = raw_sums64(g);
+        return false;
+    }
+    const long long se = w[5] + w[8], sw = w[6] + w[7], sm = w[2] + w[4];
+    const long long ke = w[1] + se, kw = w[3] + sw;
+    const long long de = w[5] - w[8], dw = w[6] - w[7];
+    fixed = w[0] + sm + ke + kw;
+    r.d = unfixed(fixed);
+    r.jx = unfixed(ke - kw);
+    r.jy = unfixed(w[2] - w[4] + de + dw);
+    r.sxx = unfixed(ke + kw);
+    r.syy = unfixed(sm + se + sw);
+    r.sxy = unfixed(de - dw);
+    return true;
+}
+__device__ __forceinline__ bool raw_sums(const double g[9], Raw& r, long long& fixed) {
+    fixed = 0;
+    r = raw_sums64(g);
+    return false;
+}
+
+// j / rho for both components
+__device__ __forceinline__ void over_rho(double rho, double jx, double jy, double& ux,
+                                         double& uy) {
+    if (rcp64_ok(rho)) {
+        const double ir = rcp64(rho);
+        ux = jx * ir;
+        uy = jy * ir;
+    } else {
+        ux = jx / rho;
+        uy = jy / rho;
+    }
+}
+
+// FP64 storage: a cell's nine equilibria, from three factors along each axis,
+// go to the slots that pull them (slot i of the cell at x - e_i, or the cell's
+// own slot opp(i) where that is a wall or solid), so that each is evaluated
+// once: about 40 FP64 operations a cell.  Evaluated per slot instead, from
+// the neighbour's fields, 1024 x 1024 cells took 234 us (now 74 us).
 template <bool MASK>
-__global__ void init_kernel(double* __restrict__ f, const AuxParams p, const double* rho,
-                            const double* ux, const double* uy) {
-    LBM_FOR_CELLS(p) {
+__global__ void __launch_bounds__(kThreads)
+init_kernel(double* __restrict__ f, const AuxParams p, const double* __restrict__ rho,
+            const double* __restrict__ ux, const double* __restrict__ uy) {
+    const double iah2 = 0.5 / (p.a * p.a);
+    LBM_FOR_TILES(p, t) {
+        const int x = tiles.x(t), y = tiles.y(t);
+        if (x >= p.nx || y >= p.ny) continue;
         const long long c = (long long)y * p.nx + x;
         const long long o = (long long)y * p.rstride + x;
         const unsigned sb = link_bits<MASK>(p, x, y);
         if (sb == 0xFFu) {
+#pragma unroll
             for (int i = 0; i < 9; ++i) f[i * p.plane + o] = 0.0;
             continue;
         }
-        const double r0 = rho ? rho[c] : 1.0, u0 = ux ? ux[c] : 0.0,
-                     v0 = uy ? uy[c] : 0.0;
+        const double r = rho ? rho[c] : 1.0, u = ux ? ux[c] : 0.0, v = uy ? uy[c] : 0.0;
+        double X[3], Y[3];  // e = 0, +1, -1
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            X[k] = r * phi_x<double>(k == 2 ? -1 : k, u, p.cs2);
+            Y[k] = phi_y<double>(k == 2 ? -1 : k, v, p.cs2, p.a, iah2);
+        }
+#pragma unroll
         for (int i = 0; i < 9; ++i) {
-            double v;
-            if (i > 0 && ((sb >> (opp(i) - 1)) & 1u)) {
-                v = feq_dev64(opp(i), r0, u0, v0, p);  // pulled back by c itself
+            const double v9 = X[ex(i) < 0 ? 2 : ex(i)] * Y[ey(i) < 0 ? 2 : ey(i)] - p.wrest[i];
+            if (i > 0 && ((sb >> (i - 1)) & 1u)) {
+                f[opp(i) * p.plane + o] = v9;
             } else {
-                const long long t = i == 0 ? c : target(p, x, y, i);
-                v = feq_dev64(i, rho ? rho[t] : 1.0, ux ? ux[t] : 0.0, uy ? uy[t] : 0.0, p);
+                int tx = x - ex(i), ty = y - ey(i);
+                tx = tx < 0 ? tx + p.nx : tx >= p.nx ? tx - p.nx : tx;
+                ty = ty < 0 ? ty + p.ny : ty >= p.ny ? ty - p.ny : ty;
+                f[i * p.plane + (long long)ty * p.rstride + tx] = v9;
             }
-            f[i * p.plane + o] = v;
         }
     }
 }
@@ -109,7 +271,7 @@ init32_kernel(float* __restrict__ f, const AuxParams p, const double* __restrict
               const double* __restrict__ ux, const double* __restrict__ uy, int rows) {
     constexpr int SW = kThreads + 2;
     __shared__ float st[3][4][SW];  // [component][ring row][column x - x0 + 1]
-    const Feq32 feq{(float)p.cs2, (float)p.a, (float)(0.5 / (p.a * p.a)), (float)p.rho0};
+    const Feq32 feq{p.cs232, p.a32, p.iah232, p.rho032};
     const int tx = threadIdx.x;
     const int x0 = blockIdx.x * kThreads;
     const int w = min(kThreads, p.nx - x0);
@@ -139,9 +301,9 @@ init32_kernel(float* __restrict__ f, const AuxParams p, const double* __restrict
     auto put = [&](int yy) {
         if (c < 0) return;
         const int s = slot(yy);
-        st[0][s][c] = (float)(qr - p.rho0);
-        st[1][s][c] = (float)qu;
-        st[2][s][c] = (float)qv;
+        st[0][s][c] = narrow(qr - p.rho0);
+        st[1][s][c] = narrow(qu);
+        st[2][s][c] = narrow(qv);
     };
     fetch(y0 - 1);
     const double r0 = qr, u0 = qu, v0 = qv;
@@ -193,61 +355,79 @@ int init_rows(int nx, int ny) {
     return max(rows, (ny + 65534) / 65535);  // grid.y limit
 }
 
+template <typename T>
+__device__ __forceinline__ T stored(double v);
+template <>
+__device__ __forceinline__ float stored<float>(double v) { return narrow(v); }
+template <>
+__device__ __forceinline__ double stored<double>(double v) { return v; }
+
 template <typename T, bool MASK>
-__global__ void set_f_kernel(T* __restrict__ f, const AuxParams p,
-                             const double* __restrict__ fin) {
+__global__ void __launch_bounds__(kThreads)
+set_f_kernel(T* __restrict__ f, const AuxParams p, const double* __restrict__ fin) {
     const long long N = (long long)p.nx * p.ny;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(c % p.nx), y = (int)(c / p.nx);
+    LBM_FOR_TILES(p, t) {
+        const int x = tiles.x(t), y = tiles.y(t);
+        if (x >= p.nx || y >= p.ny) continue;
+        const long long c = (long long)y * p.nx + x;
         const long long o = (long long)y * p.rstride + x;
         const unsigned sb = link_bits<MASK>(p, x, y);
         if (sb == 0xFFu) {
+#pragma unroll
             for (int i = 0; i < 9; ++i) f[i * p.plane + o] = T(0);
             continue;
         }
-        for (int i = 0; i < 9; ++i) {
-            double v;
-            if (i > 0 && ((sb >> (opp(i) - 1)) & 1u)) v = fin[opp(i) * N + c];
-            else v = fin[i * N + (i == 0 ? c : target(p, x, y, i))];
-            f[i * p.plane + o] = T(v - p.wrest[i]);
-        }
+        double v[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            v[i] = (i > 0 && ((sb >> (opp(i) - 1)) & 1u))
+                       ? fin[opp(i) * N + c]
+                       : fin[i * N + (i == 0 ? c : target(p, x, y, i))];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f[i * p.plane + o] = stored<T>(v[i] - p.wrest[i]);
     }
 }
 
 template <typename T, bool MASK>
-__global__ void get_f_kernel(const T* __restrict__ f, const AuxParams p,
-                             double* __restrict__ fout) {
+__global__ void __launch_bounds__(kThreads)
+get_f_kernel(const T* __restrict__ f, const AuxParams p, double* __restrict__ fout) {
     const long long N = (long long)p.nx * p.ny;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(c % p.nx), y = (int)(c / p.nx);
+    LBM_FOR_TILES(p, t) {
+        const int x = tiles.x(t), y = tiles.y(t);
+        if (x >= p.nx || y >= p.ny) continue;
+        const long long c = (long long)y * p.nx + x;
         const unsigned sb = link_bits<MASK>(p, x, y);
         if (sb == 0xFFu) {
+#pragma unroll
             for (int i = 0; i < 9; ++i) fout[i * N + c] = 0.0;
             continue;
         }
         T g[9];
         pull(f, p, x, y, sb, g);
-        for (int i = 0; i < 9; ++i) fout[i * N + c] = (double)g[i] + p.wrest[i];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fout[i * N + c] = widen(g[i]) + p.wrest[i];
     }
 }
 
-// rho and u of one fluid cell from its pulled deviations, in FP64.
+// rho, rho u (with half the force) and u of one fluid cell from its pulled
+// deviations, in FP64.  fixed: the density deviation in fixed point, where
+// the result is true.
+struct Macro {
+    double rho, jx, jy, ux, uy;
+};
 template <typename T>
-__device__ __forceinline__ void macro(const AuxParams& p, const T g[9], double& rho,
-                                      double& ux, double& uy) {
-    double d = 0.0, jx = 0.0, jy = 0.0;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const double v = (double)g[i];
-        d += v;
-        jx += ex(i) * v;
-        jy += ey(i) * v;
-    }
-    rho = p.rho0 + d;
-    ux = (jx + 0.5 * p.Fx) / rho;
-    uy = (p.a * jy + 0.5 * p.Fy) / rho;
+__device__ __forceinline__ bool macro(const AuxParams& p, const T g[9], Macro& m,
+                                      long long& fixed) {
+    Raw r;
+    const bool ok = raw_sums(g, r, fixed);
+    m.rho = p.rho0 + r.d;
+    m.jx = r.jx + 0.5 * p.Fx;
+    m.jy = fma(p.a, r.jy, 0.5 * p.Fy);
+    over_rho(m.rho, m.jx, m.jy, m.ux, m.uy);
+    return ok;
+}
+__device__ __forceinline__ bool finite64(double v) {
+    return ((unsigned)__double2hiint(v) & 0x7FF00000u) != 0x7FF00000u;
 }
 
 // The read-out of FP32 storage (lbm_moments): the nine deviations summed in
@@ -263,17 +443,22 @@ __device__ __forceinline__ void macro_out(const AuxParams& p, const float g[9], 
         if (ex(i) != 0) jx += ex(i) > 0 ? g[i] : -g[i];
         if (ey(i) != 0) jy += ey(i) > 0 ? g[i] : -g[i];
     }
-    rho = p.rho0 + (double)d;
-    const float r = (float)p.rho0 + d;
-    ux = (double)((jx + 0.5f * (float)p.Fx) / r);
-    uy = (double)(((float)p.a * jy + 0.5f * (float)p.Fy) / r);
+    rho = p.rho0 + widen(d);
+    const float r = p.rho032 + d;
+    ux = widen((jx + p.hFx32) / r);
+    uy = widen((p.a32 * jy + p.hFy32) / r);
 }
 __device__ __forceinline__ void macro_out(const AuxParams& p, const double g[9], double& rho,
                                           double& ux, double& uy) {
-    macro(p, g, rho, ux, uy);
+    Macro m;
+    long long fixed;
+    macro(p, g, m, fixed);
+    rho = m.rho;
+    ux = m.ux;
+    uy = m.uy;
 }
 
-template <typename T, bool MASK, bool EXACT64>
+template <typename T, bool MASK>
 __global__ void moments_kernel(const T* __restrict__ f, const AuxParams p,
                                double* rho, double* ux, double* uy) {
     LBM_FOR_CELLS(p) {
@@ -283,12 +468,32 @@ __global__ void moments_kernel(const T* __restrict__ f, const AuxParams p,
         if (sb != 0xFFu) {
             T g[9];
             pull(f, p, x, y, sb, g);
-            if constexpr (EXACT64) macro(p, g, r, u, v);
-            else macro_out(p, g, r, u, v);
+            macro_out(p, g, r, u, v);
         }
         if (rho) rho[c] = r;
         if (ux) ux[c] = u;
         if (uy) uy[c] = v;
+    }
+}
+
+// The density of every cell in FP64 (0 in a solid cell), for the stress.
+template <typename T, bool MASK>
+__global__ void __launch_bounds__(kThreads)
+density_kernel(const T* __restrict__ f, const AuxParams p, double* __restrict__ rho) {
+    LBM_FOR_TILES(p, t) {
+        const int x = tiles.x(t), y = tiles.y(t);
+        if (x >= p.nx || y >= p.ny) continue;
+        const unsigned sb = link_bits<MASK>(p, x, y);
+        double r = 0.0;
+        if (sb != 0xFFu) {
+            T g[9];
+            pull(f, p, x, y, sb, g);
+            Raw s;
+            long long fixed;
+            raw_sums(g, s, fixed);
+            r = p.rho0 + s.d;
+        }
+        rho[(long long)y * p.nx + x] = r;
     }
 }
 
@@ -298,65 +503,68 @@ __global__ void moments_kernel(const T* __restrict__ f, const AuxParams p,
 // FP64.  The density gradient is the central difference of the step (spacing
 // 2 along x and 2a along y), a wall or solid neighbour counting with the
 // cell's own density.
+// Bound by the FP64 lanes: about 60 operations a cell, with the moments as
+// deviations from the rest state (the rest part cancels analytically), two
+// reciprocals and products in place of the five divisions, and the constants
+// from the host.
+struct StressConst {
+    double a, a2, cs2, nu4, nu5, zeta, b1c, b2c, c1c, c2c, g1, g2, e5, hFx, hFy;
+};
 template <typename T, bool MASK>
-__global__ void stress_kernel(const T* __restrict__ f, const AuxParams p,
-                              const double* __restrict__ rho, double* dxux, double* dyuy,
-                              double* sxy, double* txx, double* tyy, double* txy) {
-    const long long N = (long long)p.nx * p.ny;
-    const double a = p.a, a2 = a * a, cs2 = p.cs2;
-    const double nu4 = cs2 * (1.0 / p.w4 - 0.5), nu5 = cs2 * (1.0 / p.w5 - 0.5);
-    const double zeta = cs2 * (1.0 / p.w3 - 0.5);
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(c % p.nx), y = (int)(c / p.nx);
+__global__ void __launch_bounds__(kThreads)
+stress_kernel(const T* __restrict__ f, const AuxParams p, const StressConst q,
+              const double* __restrict__ rho,
+              double* __restrict__ dxux, double* __restrict__ dyuy, double* __restrict__ sxy,
+              double* __restrict__ txx, double* __restrict__ tyy, double* __restrict__ txy) {
+    LBM_FOR_TILES(p, t) {
+        const int x = tiles.x(t), y = tiles.y(t);
+        if (x >= p.nx || y >= p.ny) continue;
+        const long long row = (long long)y * p.nx, c = row + x;
         const unsigned sb = link_bits<MASK>(p, x, y);
-        double e_xx = 0.0, e_yy = 0.0, e_xy = 0.0, r = 0.0;
+        double e_xx = 0.0, e_yy = 0.0, e_xy = 0.0, s_m = 0.0, s_d = 0.0, s_xy = 0.0;
         if (sb != 0xFFu) {
             T g[9];
             pull(f, p, x, y, sb, g);
-            double m0 = 0, m1 = 0, m2 = 0, m3 = 0, m4 = 0, m5 = 0;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const double fi = (double)g[i] + p.wrest[i];
-                const double ex_ = ex(i), ey_ = a * ey(i);
-                m0 += fi;
-                m1 += fi * ex_;
-                m2 += fi * ey_;
-                m3 += fi * (ex_ * ex_ + ey_ * ey_);
-                m4 += fi * (ex_ * ex_ - ey_ * ey_);
-                m5 += fi * ex_ * ey_;
-            }
-            r = m0;
-            const double ux = (m1 + 0.5 * p.Fx) / r, uy = (m2 + 0.5 * p.Fy) / r;
-            const double rc = rho[c];
             const int xm = x == 0 ? p.nx - 1 : x - 1, xp = x == p.nx - 1 ? 0 : x + 1;
             const int ym = y == 0 ? p.ny - 1 : y - 1, yp = y == p.ny - 1 ? 0 : y + 1;
-            const long long row = (long long)y * p.nx;
+            const double rc = rho[c];
             const double rW = (sb & 1u) ? rc : rho[row + xm];
             const double rS = (sb & 2u) ? rc : rho[(long long)ym * p.nx + x];
             const double rE = (sb & 4u) ? rc : rho[row + xp];
             const double rN = (sb & 8u) ? rc : rho[(long long)yp * p.nx + x];
-            const double dxr = 0.5 * (rE - rW), dyr = (rN - rS) / (2.0 * a);
+            Raw s;
+            long long fixed;
+            raw_sums(g, s, fixed);
+            const double r = p.rho0 + s.d;
+            const double ir = rcp64_ok(r) ? rcp64(r) : 1.0 / r;
+            const double jx = s.jx + q.hFx, jy = fma(q.a, s.jy, q.hFy);
+            const double ux = jx * ir, uy = jy * ir;
+            // non-equilibrium second-order moments m - m^eq
             const double ux2 = ux * ux, uy2 = uy * uy;
-            const double B1 = r * (-2.0 * cs2 / p.w3 - 0.5 * (1.0 - 3.0 * cs2) + 1.5 * ux2);
-            const double B2 = r * (-2.0 * cs2 / p.w3 - 0.5 * (a2 - 3.0 * cs2) + 1.5 * uy2);
-            const double B3 = 0.5 * (3.0 * cs2 - 1.0) * ux, B4 = 0.5 * (3.0 * cs2 - a2) * uy;
-            const double C1 = r * (-2.0 * cs2 / p.w4 - 0.5 * (1.0 - 3.0 * cs2) + 1.5 * ux2);
-            const double C2 = r * (2.0 * cs2 / p.w4 - 0.5 * (3.0 * cs2 - a2) - 1.5 * uy2);
-            const double C3 = B3, C4 = -B4;
-            const double R3 = m3 - (2.0 * r * cs2 + r * (ux2 + uy2)) - B3 * dxr - B4 * dyr;
-            const double R4 = m4 - r * (ux2 - uy2) - C3 * dxr - C4 * dyr;
-            e_xx = (C2 * R3 - B2 * R4) / (C2 * B1 - C1 * B2);
-            e_yy = (C1 * R3 - B1 * R4) / (C1 * B2 - C2 * B1);
-            e_xy = (m5 - r * ux * uy) / (-r * cs2 / p.w5);
+            const double n20 = fma(-jx, ux, fma(-q.cs2, s.d, s.sxx));
+            const double n02 = fma(-jy, uy, fma(-q.cs2, s.d, q.a2 * s.syy));
+            const double n11 = fma(-jx, uy, q.a * s.sxy);
+            const double gx = q.g1 * ux * (rE - rW), gy = q.g2 * uy * (rN - rS);
+            const double m20 = n20 + gx, m02 = n02 + gy;
+            const double R3 = m20 + m02, R4 = m20 - m02;
+            const double B1 = fma(1.5, ux2, q.b1c), B2 = fma(1.5, uy2, q.b2c);
+            const double C1 = fma(1.5, ux2, q.c1c), C2 = fma(-1.5, uy2, q.c2c);
+            const double det = fma(B1, C2, -(B2 * C1));
+            const double id = (rcp64_ok(det) ? rcp64(det) : 1.0 / det) * ir;
+            e_xx = fma(C2, R3, -(B2 * R4)) * id;
+            e_yy = fma(B1, R4, -(C1 * R3)) * id;
+            const double e11 = q.e5 * n11;
+            s_xy = q.nu5 * e11;
+            e_xy = e11 * ir;
+            s_m = r * (q.zeta * (e_xx + e_yy));
+            s_d = r * (q.nu4 * (e_xx - e_yy));
         }
-        const double div = e_xx + e_yy;
         if (dxux) dxux[c] = e_xx;
         if (dyuy) dyuy[c] = e_yy;
         if (sxy) sxy[c] = e_xy;
-        if (txx) txx[c] = r * (nu4 * (2.0 * e_xx - div) + zeta * div);
-        if (tyy) tyy[c] = r * (nu4 * (2.0 * e_yy - div) + zeta * div);
-        if (txy) txy[c] = r * nu5 * e_xy;
+        if (txx) txx[c] = s_m + s_d;
+        if (tyy) tyy[c] = s_m - s_d;
+        if (txy) txy[c] = s_xy;
     }
 }
 
@@ -396,6 +604,54 @@ __device__ __forceinline__ bool add_fixed(long long limb[kMassLimbs], double v) 
     return true;
 }
 
+// The mass of a thread's cells as one 128-bit integer, where every value is
+// an exact multiple of the integer's unit; the rest goes through add_fixed.
+// FP32 storage: the sum of a cell's deviations in units of 2^-kFixedShift.
+__device__ __forceinline__ bool add_mass(__int128& acc, long long limb[kMassLimbs],
+                                         const float g[9], bool exact, long long fixed) {
+    if (exact) {
+        acc += fixed;
+        return true;
+    }
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) ok &= add_fixed(limb, (double)g[i]);
+    return ok;
+}
+// FP64 storage: each deviation in units of 2^-100, where it is zero or
+// between 2^-47 and 2^6 in magnitude (below 2^19 values a thread: < 2^125).
+__device__ __forceinline__ bool add_mass(__int128& acc, long long limb[kMassLimbs],
+                                         const double g[9], bool, long long) {
+    bool ok = true;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(g[i]);
+        const int sh = (int)((b >> 52) & 0x7FF) - 975;  // exponent - 1075 + 100
+        if (sh >= 0 && sh < 1029 - 975) {
+            const __int128 v = (__int128)((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << sh;
+            acc += (long long)b < 0 ? -v : v;
+        } else {
+            ok &= add_fixed(limb, g[i]);
+        }
+    }
+    return ok;
+}
+// Spreads a 128-bit integer in units of 2^-58 (FP32) or 2^-100 (FP64) over
+// the 24-bit limbs.
+template <typename T>
+__device__ __forceinline__ void spread(__int128 acc, long long limb[kMassLimbs]) {
+    constexpr int kBit = kMassShift - (sizeof(T) == 4 ? kFixedShift : 100);
+    constexpr int k0 = kBit / 24, o = kBit % 24;
+    limb[k0] += (long long)(acc & ((1 << (24 - o)) - 1)) << o;
+    acc >>= 24 - o;
+#pragma unroll
+    for (int k = k0 + 1; k < kMassLimbs - 1; ++k) {
+        limb[k] += (long long)(acc & 0xFFFFFF);
+        acc >>= 24;
+    }
+    limb[kMassLimbs - 1] += (long long)acc;
+}
+
 template <typename V>
 __device__ __forceinline__ V warp_sum(V v) {
 #pragma unroll
@@ -403,9 +659,11 @@ __device__ __forceinline__ V warp_sum(V v) {
     return v;
 }
 
-// Sums one DiagPartial per thread over the block in a fixed order.
+// Sums one DiagPartial per thread over the block in a fixed order: over each
+// warp by shuffles, then one thread per field over the warps.
 __device__ void block_reduce(DiagPartial& d, DiagPartial* out) {
-    __shared__ DiagPartial sh[kThreads / 32];
+    constexpr int kWarps = kThreads / 32;
+    __shared__ DiagPartial sh[kWarps];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     d.mx = warp_sum(d.mx);
     d.my = warp_sum(d.my);
@@ -418,19 +676,17 @@ __device__ void block_reduce(DiagPartial& d, DiagPartial* out) {
     for (int k = 0; k < kMassLimbs; ++k) d.limb[k] = warp_sum(d.limb[k]);
     if (lane == 0) sh[w] = d;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        DiagPartial s = sh[0];
-        for (int i = 1; i < (int)(blockDim.x / 32); ++i) {
-            s.mx += sh[i].mx;
-            s.my += sh[i].my;
-            s.en += sh[i].en;
-            s.dres += sh[i].dres;
-            s.ures += sh[i].ures;
-            s.sres += sh[i].sres;
-            s.nonfinite += sh[i].nonfinite;
-            for (int k = 0; k < kMassLimbs; ++k) s.limb[k] += sh[i].limb[k];
-        }
-        *out = s;
+    const int k = threadIdx.x;
+    double* real = &out->mx;
+    long long* whole = &out->nonfinite;
+    if (k < kDiagReals) {
+        double s = (&sh[0].mx)[k];
+        for (int i = 1; i < kWarps; ++i) s += (&sh[i].mx)[k];
+        real[k] = s;
+    } else if (k < kDiagReals + 1 + kMassLimbs) {
+        long long s = 0;
+        for (int i = 0; i < kWarps; ++i) s += (&sh[i].nonfinite)[k - kDiagReals];
+        whole[k - kDiagReals] = s;
     }
 }
 
@@ -447,48 +703,58 @@ diag_kernel(const T* __restrict__ f, const T* __restrict__ fprev, const AuxParam
             double* __restrict__ uprev, int have_prev, DiagPartial* part) {
     const long long N = (long long)p.nx * p.ny;
     DiagPartial d = {};
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(c % p.nx), y = (int)(c / p.nx);
+    __int128 acc = 0;
+    LBM_FOR_TILES(p, t) {
+        const int x = tiles.x(t), y = tiles.y(t);
+        if (x >= p.nx || y >= p.ny) continue;
+        const long long c = (long long)y * p.nx + x;
         const unsigned sb = link_bits<MASK>(p, x, y);
         if (sb == 0xFFu) continue;
-        T g[9];
+        // every read first: one latency a cell
+        T g[9], q[9];
+        double pu = 0.0, pv = 0.0;
         pull(f, p, x, y, sb, g);
-        bool ok = true;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) ok &= add_fixed(d.limb, (double)g[i]);
-        double rho, ux, uy;
-        macro(p, g, rho, ux, uy);
-        if (!ok || !isfinite(rho) || !isfinite(ux) || !isfinite(uy)) {
+        if (fprev) pull(fprev, p, x, y, sb, q);
+        if (have_prev) {
+            pu = uprev[c];
+            pv = uprev[N + c];
+        }
+        Macro m;
+        long long fixed;
+        const bool exact = macro(p, g, m, fixed);
+        const bool ok = add_mass(acc, d.limb, g, exact, fixed);
+        if (!ok || !finite64(m.rho) || !finite64(m.ux) || !finite64(m.uy)) {
             d.nonfinite += 1;
             continue;
         }
-        d.mx += rho * ux;
-        d.my += rho * uy;
-        d.en += 0.5 * rho * (ux * ux + uy * uy);
-        double mx = ux, my = uy;
+        d.mx += m.jx;
+        d.my += m.jy;
+        d.en = fma(0.5, fma(m.jx, m.ux, m.jy * m.uy), d.en);
+        double mx = m.ux, my = m.uy;
         if (fprev) {
-            T q[9];
-            pull(fprev, p, x, y, sb, q);
-            double r1, ux1, uy1;
-            macro(p, q, r1, ux1, uy1);
-            const double sx = ux - ux1, sy = uy - uy1;
-            d.sres += sx * sx + sy * sy;
-            mx = 0.5 * (ux + ux1);
-            my = 0.5 * (uy + uy1);
+            Macro m1;
+            macro(p, q, m1, fixed);
+            const double sx = m.ux - m1.ux, sy = m.uy - m1.uy;
+            d.sres = fma(sx, sx, fma(sy, sy, d.sres));
+            mx = 0.5 * (m.ux + m1.ux);
+            my = 0.5 * (m.uy + m1.uy);
         }
-        d.ures += mx * mx + my * my;
+        d.ures = fma(mx, mx, fma(my, my, d.ures));
         if (have_prev) {
-            const double du = mx - uprev[c], dv = my - uprev[N + c];
-            d.dres += du * du + dv * dv;
+            const double du = mx - pu, dv = my - pv;
+            d.dres = fma(du, du, fma(dv, dv, d.dres));
         }
         uprev[c] = mx;
         uprev[N + c] = my;
     }
+    spread<T>(acc, d.limb);
     block_reduce(d, part + blockIdx.x);
 }
 
-__global__ void __launch_bounds__(kThreads) diag_final(DiagPartial* part, int n) {
+// Sums the n partials into *out, beside the step kernels' status word (so
+// that the host reads one result).
+__global__ void __launch_bounds__(kThreads)
+diag_final(const DiagPartial* part, int n, const int* status, DiagPartial* out) {
     DiagPartial d = {};
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const DiagPartial& q = part[i];
@@ -499,9 +765,11 @@ __global__ void __launch_bounds__(kThreads) diag_final(DiagPartial* part, int n)
         d.ures += q.ures;
         d.sres += q.sres;
         d.nonfinite += q.nonfinite;
+#pragma unroll
         for (int k = 0; k < kMassLimbs; ++k) d.limb[k] += q.limb[k];
     }
-    block_reduce(d, part + n);
+    block_reduce(d, out);
+    if (threadIdx.x == 0) out->status = *status;
 }
 
 // Residual sums of one thread summed over the block, in a fixed order.
@@ -524,8 +792,8 @@ __device__ void res_block_reduce(ResPartial& d, ResPartial* out) {
     }
 }
 
-// Block w sums reduction chunk w - rbegin[j] of active lattice j: cells
-// chunk * kThreads + t + m * nchunk * kThreads.
+// Block w sums reduction chunk w - rbegin[j] of active lattice j: its tiles
+// chunk, chunk + nchunk, ...
 __global__ void __launch_bounds__(kThreads)
 batch_res_kernel(const BatchLattice<float>* __restrict__ lat, const BatchAux* __restrict__ aux,
                  const int* __restrict__ active, const int* __restrict__ rbegin,
@@ -549,31 +817,34 @@ batch_res_kernel(const BatchLattice<float>* __restrict__ lat, const BatchAux* __
     const long long N = (long long)p.nx * p.ny;
     double* __restrict__ up = B.uprev;
     ResPartial d = {};
-    for (long long c = (long long)chunk * kThreads + threadIdx.x; c < N;
-         c += (long long)B.nchunk * kThreads) {
-        const int x = (int)(c % p.nx), y = (int)(c / p.nx);
+    const Tiles tiles(p.nx, p.ny);
+    for (int t = chunk; t < tiles.n; t += B.nchunk) {
+        const int x = tiles.x(t), y = tiles.y(t);
+        if (x >= p.nx || y >= p.ny) continue;
+        const long long c = (long long)y * p.nx + x;
         const unsigned sb = link_bits<true>(p, x, y);
         if (sb == 0xFFu) continue;
-        float g[9];
+        float g[9], q[9];
         pull(f, p, x, y, sb, g);
-        double rho, ux, uy;
-        macro(p, g, rho, ux, uy);
-        if (!isfinite(rho) || !isfinite(ux) || !isfinite(uy)) {
+        if (fp) pull(fp, p, x, y, sb, q);
+        const double pu = up[c], pv = up[N + c];
+        Macro m;
+        long long fixed;
+        macro(p, g, m, fixed);
+        if (!finite64(m.rho) || !finite64(m.ux) || !finite64(m.uy)) {
             d.nonfinite += 1;
             continue;
         }
-        double mx = ux, my = uy;  // the two-step mean velocity, as in diag_kernel
+        double mx = m.ux, my = m.uy;  // the two-step mean velocity, as in diag_kernel
         if (fp) {
-            float q[9];
-            pull(fp, p, x, y, sb, q);
-            double r1, ux1, uy1;
-            macro(p, q, r1, ux1, uy1);
-            mx = 0.5 * (ux + ux1);
-            my = 0.5 * (uy + uy1);
+            Macro m1;
+            macro(p, q, m1, fixed);
+            mx = 0.5 * (m.ux + m1.ux);
+            my = 0.5 * (m.uy + m1.uy);
         }
-        const double du = mx - up[c], dv = my - up[N + c];
-        d.dres += du * du + dv * dv;
-        d.ures += mx * mx + my * my;
+        const double du = mx - pu, dv = my - pv;
+        d.dres = fma(du, du, fma(dv, dv, d.dres));
+        d.ures = fma(mx, mx, fma(my, my, d.ures));
         up[c] = mx;
         up[N + c] = my;
     }
@@ -598,9 +869,10 @@ batch_res_final(const BatchAux* __restrict__ aux, const int* __restrict__ active
     res_block_reduce(d, out + k);
 }
 
-int grid_for(long long N) {
-    long long b = (N + kThreads - 1) / kThreads;
-    return (int)(b < 4096 ? (b > 0 ? b : 1) : 4096);
+// blocks of LBM_FOR_TILES, at most `most`
+int tile_grid(const AuxParams& p, int most = 4096) {
+    const int n = Tiles(p.nx, p.ny).n;
+    return n < most ? n : most;
 }
 
 // grid of LBM_FOR_CELLS: blocks across a row, rows down the grid, at most
@@ -622,7 +894,7 @@ cudaError_t launch_init(T* f, const AuxParams& p, const double* rho, const doubl
         if (p.lmask) init32_kernel<true><<<g, kInitThreads, 0, s>>>(f, p, rho, ux, uy, rows);
         else init32_kernel<false><<<g, kInitThreads, 0, s>>>(f, p, rho, ux, uy, rows);
     } else {
-        const dim3 g = grid2_for(p.nx, p.ny);
+        const int g = tile_grid(p);
         if (p.lmask) init_kernel<true><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
         else init_kernel<false><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
     }
@@ -631,7 +903,7 @@ cudaError_t launch_init(T* f, const AuxParams& p, const double* rho, const doubl
 
 template <typename T>
 cudaError_t launch_set_f(T* f, const AuxParams& p, const double* fin, cudaStream_t s) {
-    const int g = grid_for((long long)p.nx * p.ny);
+    const int g = tile_grid(p);
     if (p.lmask) set_f_kernel<T, true><<<g, kThreads, 0, s>>>(f, p, fin);
     else set_f_kernel<T, false><<<g, kThreads, 0, s>>>(f, p, fin);
     return cudaGetLastError();
@@ -639,7 +911,7 @@ cudaError_t launch_set_f(T* f, const AuxParams& p, const double* fin, cudaStream
 
 template <typename T>
 cudaError_t launch_get_f(const T* f, const AuxParams& p, double* fout, cudaStream_t s) {
-    const int g = grid_for((long long)p.nx * p.ny);
+    const int g = tile_grid(p);
     if (p.lmask) get_f_kernel<T, true><<<g, kThreads, 0, s>>>(f, p, fout);
     else get_f_kernel<T, false><<<g, kThreads, 0, s>>>(f, p, fout);
     return cudaGetLastError();
@@ -647,15 +919,18 @@ cudaError_t launch_get_f(const T* f, const AuxParams& p, double* fout, cudaStrea
 
 template <typename T>
 cudaError_t launch_moments(const T* f, const AuxParams& p, double* rho, double* ux,
-                           double* uy, cudaStream_t s, bool exact64) {
+                           double* uy, cudaStream_t s) {
     const dim3 g = grid2_for(p.nx, p.ny);
-    if (exact64) {
-        if (p.lmask) moments_kernel<T, true, true><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
-        else moments_kernel<T, false, true><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
-    } else {
-        if (p.lmask) moments_kernel<T, true, false><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
-        else moments_kernel<T, false, false><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
-    }
+    if (p.lmask) moments_kernel<T, true><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
+    else moments_kernel<T, false><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_density(const T* f, const AuxParams& p, double* rho, cudaStream_t s) {
+    const int g = tile_grid(p);
+    if (p.lmask) density_kernel<T, true><<<g, kThreads, 0, s>>>(f, p, rho);
+    else density_kernel<T, false><<<g, kThreads, 0, s>>>(f, p, rho);
     return cudaGetLastError();
 }
 
@@ -663,24 +938,43 @@ template <typename T>
 cudaError_t launch_stress(const T* f, const AuxParams& p, const double* rho, double* dxux,
                           double* dyuy, double* sxy, double* txx, double* tyy, double* txy,
                           cudaStream_t s) {
-    const int g = grid_for((long long)p.nx * p.ny);
+    const int g = tile_grid(p);
+    const double a2 = p.a * p.a, c = p.cs2;
+    StressConst q;
+    q.a = p.a;
+    q.a2 = a2;
+    q.cs2 = c;
+    q.nu4 = c * (1.0 / p.w4 - 0.5);
+    q.nu5 = c * (1.0 / p.w5 - 0.5);
+    q.zeta = c * (1.0 / p.w3 - 0.5);
+    q.b1c = -2.0 * c / p.w3 - 0.5 * (1.0 - 3.0 * c);
+    q.b2c = -2.0 * c / p.w3 - 0.5 * (a2 - 3.0 * c);
+    q.c1c = -2.0 * c / p.w4 - 0.5 * (1.0 - 3.0 * c);
+    q.c2c = 2.0 * c / p.w4 + 0.5 * (a2 - 3.0 * c);
+    q.g1 = 0.25 * (1.0 - 3.0 * c);           // with the spacing 2 of the differences
+    q.g2 = 0.25 * (a2 - 3.0 * c) / p.a;      // and 2a
+    q.e5 = -p.w5 / c;
+    q.hFx = 0.5 * p.Fx;
+    q.hFy = 0.5 * p.Fy;
     if (p.lmask)
-        stress_kernel<T, true><<<g, kThreads, 0, s>>>(f, p, rho, dxux, dyuy, sxy, txx, tyy, txy);
+        stress_kernel<T, true><<<g, kThreads, 0, s>>>(f, p, q, rho, dxux, dyuy, sxy, txx, tyy, txy);
     else
-        stress_kernel<T, false><<<g, kThreads, 0, s>>>(f, p, rho, dxux, dyuy, sxy, txx, tyy, txy);
+        stress_kernel<T, false><<<g, kThreads, 0, s>>>(f, p, q, rho, dxux, dyuy, sxy, txx, tyy, txy);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_diag(const T* f, const T* fprev, const AuxParams& p, double* uprev,
-                        int have_prev, DiagPartial* part, int nblocks, cudaStream_t s) {
+                        int have_prev, DiagPartial* part, int nblocks, const int* status,
+                        cudaStream_t s) {
+    const int n = tile_grid(p, nblocks);
     if (p.lmask)
-        diag_kernel<T, true><<<nblocks, kThreads, 0, s>>>(f, fprev, p, uprev, have_prev, part);
+        diag_kernel<T, true><<<n, kThreads, 0, s>>>(f, fprev, p, uprev, have_prev, part);
     else
-        diag_kernel<T, false><<<nblocks, kThreads, 0, s>>>(f, fprev, p, uprev, have_prev, part);
+        diag_kernel<T, false><<<n, kThreads, 0, s>>>(f, fprev, p, uprev, have_prev, part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    diag_final<<<1, kThreads, 0, s>>>(part, nblocks);
+    diag_final<<<1, kThreads, 0, s>>>(part, n, status, part + nblocks);
     return cudaGetLastError();
 }
 
@@ -705,12 +999,14 @@ cudaError_t launch_batch_residual(const BatchLattice<float>* lat, const BatchAux
     template cudaError_t launch_get_f<T>(const T*, const AuxParams&, double*,         \
                                          cudaStream_t);                               \
     template cudaError_t launch_moments<T>(const T*, const AuxParams&, double*,       \
-                                           double*, double*, cudaStream_t, bool);     \
+                                           double*, double*, cudaStream_t);           \
+    template cudaError_t launch_density<T>(const T*, const AuxParams&, double*,       \
+                                           cudaStream_t);                             \
     template cudaError_t launch_stress<T>(const T*, const AuxParams&, const double*,  \
                                           double*, double*, double*, double*, double*, \
                                           double*, cudaStream_t);                     \
     template cudaError_t launch_diag<T>(const T*, const T*, const AuxParams&, double*, int, \
-                                        DiagPartial*, int, cudaStream_t);
+                                        DiagPartial*, int, const int*, cudaStream_t);
 LBM_AUX_INST(float)
 LBM_AUX_INST(double)
 
