@@ -148,11 +148,12 @@ lbm_status lbm_set_force(lbm_handle* h, double Fx, double Fy);
  * fused step per launch at every size).  A lattice of at most 4096 cells
  * whose cluster fits the device runs the steps of an lbm_step call in
  * launches of up to 1024 steps each, every launch one thread-block cluster
- * of min(ny, 16) CTAs that synchronise twice per step (density field, then
- * collide and stream); the states are bit for bit those of the row-band
- * kernel.  enable = 0 makes the handle use the row-band kernel (one launch
- * per step); enable = 1 (the default where available) brings the cluster
- * back.  enable not 0 or 1, or 1 for a lattice without the cluster path:
+ * of min(ny, 16) CTAs that keep the state in shared memory and synchronise
+ * once per step; the states are bit for bit those of the row-band kernel.
+ * enable = 0 makes the handle use the row-band kernel (one launch per step);
+ * enable = 1 brings the cluster back.  The default is the cluster where it
+ * is available, but for lattices so wide that a CTA holds more than 768
+ * (FP32) or 320 (FP64) cells.  enable not 0 or 1, or 1 for a lattice without the cluster path:
  * LBM_ERR_INVALID. */
 lbm_status lbm_set_small_path(lbm_handle* h, int enable);
 

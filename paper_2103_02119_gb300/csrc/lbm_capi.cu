@@ -64,7 +64,7 @@ struct lbm_handle {
     int diag_blocks = 0;
     int bx = 0, nbands = 0;
     int64_t steps = 0, launches = 0;
-    void* dfield = nullptr;    // small lattices: the density field of a step
+    uint8_t* bits = nullptr;   // small lattices: link bits of the nx * ny cells (device)
     bool small = false;        // steps run as one cluster launch (small_step.cu)
     cudaStream_t cap = nullptr;                     // owned, for graph capture only
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // runs of steps from f[0] / f[1]
@@ -411,7 +411,7 @@ lbm_status step_lattice(lbm_handle* h, int64_t nsteps) {
     if (h->small) {  // one cluster launch runs up to kSmallRun steps
         for (int64_t left = nsteps; left > 0;) {
             const int n = left < kSmallRun ? (int)left : kSmallRun;
-            CK(h, lbm::launch_small_run<T>((T*)h->f[0], (T*)h->f[1], (T*)h->dfield, k, h->cur, n,
+            CK(h, lbm::launch_small_run<T>((T*)h->f[0], (T*)h->f[1], h->bits, k, h->cur, n,
                                            h->stream),
                "small-lattice step kernel");
             h->cur ^= n & 1;
@@ -575,8 +575,19 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
         const bool fits = f64 ? lbm::small_run_fits<double>(kparams<double>(h))
                               : lbm::small_run_fits<float>(kparams<float>(h));
         if (fits) {
-            CKC(lbm::dev_alloc(&h->dfield, (size_t)h->N * elem_size(h)), "cudaMalloc(density field)");
-            h->small = true;
+            std::vector<uint8_t> fluid, lb;
+            if (!solid_mask) fluid.assign((size_t)h->N, 0);
+            build_link_mask(*p, solid_mask ? solid_mask : fluid.data(), p->nx, lb);
+            CKC(lbm::dev_alloc(&h->bits, lb.size()), "cudaMalloc(link bits)");
+            CKC(cudaMemcpy(h->bits, lb.data(), lb.size(), cudaMemcpyHostToDevice),
+                "cudaMemcpy(link bits)");
+            // taken by default while a CTA's cells keep its steps shorter than
+            // the row-band kernel's, which spreads wide rows over more SMs
+            // (us a step, cluster / bands: FP64 300 x 5 17 / 21, 240 x 17 (480
+            // cells a CTA) 28 / 21, 1365 x 3 91 / 21; FP32 240 x 17 3.2 / 5.7,
+            // 1365 x 3 9.3 / 6.5)
+            const int C = p->ny < lbm::kSmallCluster ? p->ny : lbm::kSmallCluster;
+            h->small = (p->ny + C - 1) / C * p->nx <= (f64 ? 320 : 768);
         }
     }
 #undef CKC
@@ -593,7 +604,7 @@ void lbm_destroy(lbm_handle* h) {
     if (h->f[0]) cudaFree(h->f[0]);
     if (h->f[1]) cudaFree(h->f[1]);
     if (h->lmask) cudaFree(h->lmask);
-    if (h->dfield) cudaFree(h->dfield);
+    if (h->bits) cudaFree(h->bits);
     if (h->uprev) cudaFree(h->uprev);
     if (h->stage) cudaFree(h->stage);
     if (h->part) cudaFree(h->part);
@@ -642,7 +653,7 @@ lbm_status lbm_set_small_path(lbm_handle* h, int enable) {
         set_err(h, "enable must be 0 or 1");
         return LBM_ERR_INVALID;
     }
-    if (enable && !h->dfield) {
+    if (enable && !h->bits) {
         set_err(h, "this lattice has no small-lattice path (more than 4096 cells, or the cluster "
                    "does not fit the device)");
         return LBM_ERR_INVALID;

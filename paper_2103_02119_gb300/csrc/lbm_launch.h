@@ -43,12 +43,13 @@ int step_occupancy(int bx, bool mask);
 
 // Small lattices (at most kSmallCells cells): nsteps steps in one launch of
 // one thread-block cluster of min(ny, kSmallCluster) CTAs, from buffer
-// `from` (f0 or f1); dfield: nx*ny values of T (the density field of a step).
+// `from` (f0 or f1); bits: the link bits of the nx * ny cells (device).
 constexpr long long kSmallCells = 4096;
 constexpr int kSmallCluster = 16;
+constexpr int kSmallSmemMax = 227 * 1024;  // shared memory of one CTA
 template <typename T>
-cudaError_t launch_small_run(T* f0, T* f1, T* dfield, const KParams<T>& p, int from, int nsteps,
-                             cudaStream_t s);
+cudaError_t launch_small_run(T* f0, T* f1, const uint8_t* bits, const KParams<T>& p, int from,
+                             int nsteps, cudaStream_t s);
 // whether such a cluster launch fits this device (queried, no launch)
 template <typename T>
 bool small_run_fits(const KParams<T>& p);
