@@ -187,14 +187,19 @@ KParams<T> kparams_of(const lbm_params& q, const Geometry& g) {
     for (int w = 0; w < 4; ++w) {
         const bool exists = w < 2 ? !q.periodic_x : !q.periodic_y;
         if (exists && (q.wall_u[w][0] != 0.0 || q.wall_u[w][1] != 0.0)) k.moving = 1;
-        k.wall_u[w][0] = T(q.wall_u[w][0]);
-        k.wall_u[w][1] = T(q.wall_u[w][1]);
+        const double Ux = q.wall_u[w][0], Uy = q.wall_u[w][1];
+        for (int j = 0; j < 3; ++j) {
+            const int i = lbm::wall_link(w, j);
+            const double iah2 = 0.5 / (q.a * q.a);
+            const auto odd = [&](int sx, int sy) {
+                return lbm::phi_x<double>(sx, Ux, q.cs2) * lbm::phi_y<double>(sy, Uy, q.cs2, q.a, iah2);
+            };
+            const int sx = lbm::ex(i), sy = lbm::ey(i);
+            k.wall_odd[w][j] = T(exists && (Ux != 0.0 || Uy != 0.0) ? odd(sx, sy) - odd(-sx, -sy) : 0.0);
+        }
     }
     const double a = q.a, cs2 = q.cs2, a2 = a * a;
-    k.a = T(a);
     k.iah = T(0.5 / a);
-    k.iah2 = T(0.5 / a2);
-    k.cs2 = T(cs2);
     k.rho0 = T(q.rho0);
     const double* w = q.omega;
     const double g1 = 1.0 - 3.0 * cs2, g2 = a2 - 3.0 * cs2;
@@ -1219,13 +1224,10 @@ lbm::KParams<float, lbm::CollConstF> kparams_table(const KParams<float>& k) {
     t.raw = k.raw;
     t.forced = k.forced;
     t.spin_limit = k.spin_limit;
-    t.a = k.a;
     t.iah = k.iah;
-    t.iah2 = k.iah2;
-    t.cs2 = k.cs2;
     t.rho0 = k.rho0;
     for (int w = 0; w < 4; ++w)
-        for (int d = 0; d < 2; ++d) t.wall_u[w][d] = k.wall_u[w][d];
+        for (int j = 0; j < 3; ++j) t.wall_odd[w][j] = k.wall_odd[w][j];
     t.lmask = k.lmask;
     t.status = k.status;
     t.cc = lbm::compact(k.cc);
