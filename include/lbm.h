@@ -311,8 +311,10 @@ const char* lbm_last_error(const lbm_handle* h);
  * Otherwise one kernel per
  * scheme reads the parameters from a table in global memory (slower: they
  * then take vector registers).  Runs of 50 steps replay a captured CUDA
- * graph.  Lattices
- * can be retired (made inactive) and brought back; an inactive lattice keeps
+ * graph.  When every active lattice has at most 4096 cells (and they fit the
+ * constant-memory tables), each steps on a thread-block cluster of its own
+ * that keeps its state in shared memory, up to 1024 steps per launch and
+ * group; the launch shape does not matter then.  Lattices can be retired (made inactive) and brought back; an inactive lattice keeps
  * its state and is not stepped.  Conventions as for lbm_handle; work is
  * issued on the stream given to lbm_batch_create.
  * ------------------------------------------------------------------------ */
@@ -419,8 +421,8 @@ lbm_status lbm_batch_diagnostics(lbm_batch* b, int k, double out[LBM_DIAG_COUNT]
 /* Steps taken by lattice k since its last init (-1 for a bad argument). */
 int64_t lbm_batch_step_count(const lbm_batch* b, int k);
 
-/* Batch step kernel launches issued so far: one per step, two when the
- * batch holds lattices of both schemes (one persistent launch each). */
+/* Batch step kernel launches issued so far: one per group of lattices and
+ * step, or (active lattices of at most 4096 cells) run of up to 1024 steps. */
 int64_t lbm_batch_launch_count(const lbm_batch* b);
 
 /* Message of the last error on b (or of the last failed lbm_batch_create

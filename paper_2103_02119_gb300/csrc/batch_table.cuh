@@ -19,6 +19,7 @@
 // The block's work is step_block's, so a lattice goes through the same states
 // bit for bit as with the single-lattice kernel.
 #pragma once
+#include "small_step.cuh"
 #include "step_block.cuh"
 
 #ifndef LBM_BATCH_SLOT
@@ -87,6 +88,43 @@ cudaError_t launch_table_sch(int parity, int bx, int grid, cudaStream_t s) {
     }
 }
 
+// Batches of small lattices: a cluster per lattice runs nsteps steps with the
+// state in shared memory (small_step.cuh).
+__global__ void __launch_bounds__(kSmallMaxThreads<float>) batch_small_kernel(int from, int nsteps) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned C;
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(C));
+    const BatchTableLattice& L = c_table[blockIdx.x / C];
+    small_run<float>(L.kp, L.f[0], L.f[1], L.kp.lmask, L.kp.pitch, from, nsteps, smem,
+                     (int)(blockIdx.x % C), (int)C);
+}
+
+cudaLaunchConfig_t small_batch_config(const SmallBatch& b, int n, cudaStream_t s,
+                                      cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n * b.cluster, 1, 1);
+    cfg.blockDim = dim3(b.threads, 1, 1);
+    cfg.dynamicSmemBytes = b.smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = b.cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+cudaError_t configure_small_batch() {
+    static bool configured = false;
+    if (!configured) {
+        cudaError_t e = cudaFuncSetAttribute(
+            batch_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    return cudaSuccess;
+}
+
 template <int BXT>
 int table_occ_bx() {
     constexpr size_t smem = step_smem_bytes<float, BXT>();
@@ -116,6 +154,26 @@ cudaError_t LBM_SLOT_NAME(batch_table_upload_)(const BatchTableLattice* lat, con
 cudaError_t LBM_SLOT_NAME(batch_table_launch_)(int parity, int bx, int grid, int raw,
                                                cudaStream_t s) {
     return raw ? launch_table_sch<1>(parity, bx, grid, s) : launch_table_sch<0>(parity, bx, grid, s);
+}
+
+cudaError_t LBM_SLOT_NAME(batch_small_launch_)(const SmallBatch& b, int n, int from, int nsteps,
+                                               cudaStream_t s) {
+    if (cudaError_t e = configure_small_batch(); e != cudaSuccess) return e;
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = small_batch_config(b, n, s, attr);
+    return cudaLaunchKernelEx(&cfg, batch_small_kernel, from, nsteps);
+}
+
+bool LBM_SLOT_NAME(batch_small_fits_)(const SmallBatch& b) {
+    if (configure_small_batch() != cudaSuccess) return false;
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = small_batch_config(b, 1, nullptr, attr);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, batch_small_kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n >= 1;
 }
 
 int LBM_SLOT_NAME(batch_table_occupancy_)(int bx) {

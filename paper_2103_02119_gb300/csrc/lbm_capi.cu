@@ -1101,6 +1101,9 @@ struct lbm_batch {
     int ggrid[lbm::kBatchTables] = {};
     std::vector<lbm::BatchTableLattice> gtab[lbm::kBatchTables];
     std::vector<int> gbegin[lbm::kBatchTables];  // first work item of each, then the total
+    // cluster != 0: the groups' lattices are all small and step by clusters,
+    // many steps per launch (small_step.cuh)
+    lbm::SmallBatch small;
     unsigned long long serial = 0;   // which batch the device's tables hold
     int device = 0;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -1306,6 +1309,21 @@ void plan_groups(lbm_batch* b) {
                 g0 += ng;
             }
             b->ngroups = g0;
+        }
+    }
+    // small lattices alone: a cluster each, many steps per launch
+    b->small = lbm::SmallBatch{};
+    if (b->ngroups) {
+        std::vector<int> nx, ny;
+        for (int k = 0; k < b->count; ++k)
+            if (b->active[k] && b->N[k] <= lbm::kSmallCells) {
+                nx.push_back(b->p[k].nx);
+                ny.push_back(b->p[k].ny);
+            }
+        if ((int)nx.size() == b->n_active) {
+            b->small = lbm::small_batch_shape(nx.data(), ny.data(), b->n_active, b->sms);
+            for (int g = 0; b->small.cluster && g < b->ngroups; ++g)
+                if (!lbm::batch_small_fits(g, b->small)) b->small = lbm::SmallBatch{};
         }
     }
     // the captured graphs hold the groups' launches: a new set of groups
@@ -1703,6 +1721,15 @@ lbm_status advance(lbm_batch* b, int64_t nsteps, bool graphs) {
     if (b->n_active == 0 || nsteps == 0) return LBM_OK;
     if (lbm_status s = ensure_tables(b); s != LBM_OK) return s;
     int64_t left = nsteps;
+    while (b->small.cluster && left > 0) {  // one launch per group and run of steps
+        const int n = left < kSmallRun ? (int)left : kSmallRun;
+        const int from = (int)((b->parity + (nsteps - left)) & 1);
+        for (int g = 0; g < b->ngroups; ++g)
+            BCK(b, lbm::batch_small_launch(g, b->small, (int)b->gtab[g].size(), from, n, b->stream),
+                "batch step kernel (clusters)");
+        b->launches += b->ngroups;
+        left -= n;
+    }
     while (graphs && left >= kGraphSteps) {
         if (lbm_status s = ensure_graph(b, b->parity); s != LBM_OK) return s;
         BCK(b, cudaGraphLaunch(b->graph[b->parity], b->stream), "cudaGraphLaunch");

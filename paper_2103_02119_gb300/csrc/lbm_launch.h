@@ -87,7 +87,19 @@ struct BatchTableLattice {
 // module's constant bank holds 64 KiB.
 constexpr int kBatchTables = 4;
 constexpr int kBatchTableCap = 62000 / (int)sizeof(BatchTableLattice);
+// Launch shape of a batch of small lattices: a cluster of `cluster` CTAs per
+// lattice; cluster = 0: not used.
+struct SmallBatch {
+    int cluster = 0, threads = 0;
+    size_t smem = 0;
+};
+// The shape for lattices of these sizes (at most kSmallCells cells each;
+// cluster = 0 when they do not fit), for a device of `sms` SMs.
+SmallBatch small_batch_shape(const int* nx, const int* ny, int n, int sms);
 #define LBM_DECLARE_BATCH_TABLE(S)                                                         \
+    cudaError_t batch_small_launch_##S(const SmallBatch& b, int n, int from, int nsteps,   \
+                                       cudaStream_t s);                                    \
+    bool batch_small_fits_##S(const SmallBatch& b);                                        \
     cudaError_t batch_table_upload_##S(const BatchTableLattice* lat, const int* begin, int n, \
                                        cudaStream_t s);                                     \
     cudaError_t batch_table_launch_##S(int parity, int bx, int grid, int raw, cudaStream_t s); \
@@ -116,6 +128,21 @@ inline cudaError_t batch_table_launch(int slot, int parity, int bx, int grid, in
            : slot == 1 ? batch_table_launch_1(parity, bx, grid, raw, s)
            : slot == 2 ? batch_table_launch_2(parity, bx, grid, raw, s)
                        : batch_table_launch_3(parity, bx, grid, raw, s);
+}
+// nsteps steps of the n lattices of table `slot` (each at most kSmallCells
+// cells), from buffer f[from], in one launch.
+inline cudaError_t batch_small_launch(int slot, const SmallBatch& b, int n, int from, int nsteps,
+                                      cudaStream_t s) {
+    return slot == 0   ? batch_small_launch_0(b, n, from, nsteps, s)
+           : slot == 1 ? batch_small_launch_1(b, n, from, nsteps, s)
+           : slot == 2 ? batch_small_launch_2(b, n, from, nsteps, s)
+                       : batch_small_launch_3(b, n, from, nsteps, s);
+}
+inline bool batch_small_fits(int slot, const SmallBatch& b) {
+    return slot == 0   ? batch_small_fits_0(b)
+           : slot == 1 ? batch_small_fits_1(b)
+           : slot == 2 ? batch_small_fits_2(b)
+                       : batch_small_fits_3(b);
 }
 inline int batch_table_occupancy(int slot, int bx) {
     return slot == 0   ? batch_table_occupancy_0(bx)

@@ -51,6 +51,30 @@ cudaError_t configure_small() {
 
 }  // namespace
 
+// CTAs per lattice of a batch: as many (1, 2, 4, 8) as shared memory asks for,
+// and more while the batch makes at most two CTAs per SM.  Us a step with a
+// target of one / two / four CTAs per SM (and of the band kernel, one launch a
+// step): 64 lattices of 16-32 cells a side 1.89 / 1.83 / 1.94 (11.0), 32 of 60-64
+// 2.80 / 2.64 / 2.64 (11.9), 128 of 16-64 4.34 / 4.35 / 6.55 (24.5).
+SmallBatch small_batch_shape(const int* nx, const int* ny, int n, int sms) {
+    SmallBatch best;
+    // (a CTA past a lattice's last row has none and only joins the barriers)
+    for (int C = 1; C <= 8; C *= 2) {
+        SmallBatch b;
+        b.cluster = C;
+        for (int k = 0; k < n; ++k) {
+            const size_t m = small_smem_bytes<float>(nx[k], ny[k], C);
+            const int t = small_threads<float>(nx[k], ny[k], C);
+            if (m > b.smem) b.smem = m;
+            if (t > b.threads) b.threads = t;
+        }
+        if (b.smem > (size_t)kSmallSmemMax) continue;
+        if (best.cluster && (long long)n * C > 2LL * sms) break;
+        best = b;
+    }
+    return best;
+}
+
 template <typename T>
 cudaError_t launch_small_run(T* f0, T* f1, const uint8_t* bits, const KParams<T>& p, int from,
                              int nsteps, cudaStream_t s) {

@@ -42,3 +42,41 @@ def test_cluster_kernel_at_the_ends_of_its_range(nx, ny, kind, precision):
         assert a.launch_count == 4 and b.launch_count == 26
         a.close()
         b.close()
+
+
+def _batch_flows(sizes):
+    return [_flow(nx, ny, "periodic" if k % 2 else "walls") for k, (nx, ny) in enumerate(sizes)]
+
+
+# one CTA a lattice and several; more CTAs than rows; rows wider than a CTA's
+# threads; a lattice above 4096 cells (the whole batch then takes the band
+# kernel: one launch a step)
+@pytest.mark.parametrize("sizes,launches", [
+    ([(16, 16)], 4), ([(64, 64), (3, 3), (17, 240), (33, 31)], 4), ([(300, 5), (40, 7)], 4),
+    ([(20, 24)] * 160, 4), ([(1365, 3), (16, 16)], 4), ([(65, 64), (16, 16)], 1131)])
+def test_batches_of_small_lattices(sizes, launches):
+    from paper_2103_02119_gb300.lbm import Batch, Lattice
+    ws = _batch_flows(sizes)
+    b = Batch(ws)
+    pick = sorted(set([0, 1, 2, len(ws) - 1]) & set(range(len(ws))))
+    ref = {k: Lattice.from_workload(
+        ws[k] if ws[k].mask is not None else ws[k].with_(mask=np.zeros((ws[k].ny, ws[k].nx), np.uint8)),
+        precision=32) for k in pick}
+    for n in (1, 30, 1100):                 # 1100 steps: two launches of a cluster kernel
+        b.step(n)
+        for k in pick:
+            ref[k].step(n)
+            # (a flow that blows up does so alike)
+            assert np.array_equal(b.get_f(k), ref[k].get_f(), equal_nan=True), (k, n)
+    assert b.launch_count == launches
+    if len(ws) > 1:                         # one leaves for an odd number of steps
+        b.set_active(0, False)
+        b.step(7)
+        b.set_active(0, True)
+        b.step(4)
+        ref[0].step(4)
+        for k in pick[1:]:
+            ref[k].step(11)
+        for k in pick:
+            assert np.array_equal(b.get_f(k), ref[k].get_f(), equal_nan=True), k
+    b.close()
