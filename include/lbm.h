@@ -135,7 +135,10 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
 /* Advance nsteps >= 0 time steps (collide + stream, Sec. 4), one kernel
  * launch per step; runs of 50 steps replay a CUDA graph the handle captures
  * once per starting buffer (on a stream of its own; lbm_set_force drops
- * it).  Small lattices run many steps per launch (lbm_set_small_path).  Asynchronous: the return value reports launch errors only. */
+ * it).  Small lattices run many steps per launch (lbm_set_small_path), large
+ * FP32 ones (from 200,000 cells) two steps per launch but for the last one or
+ * two of a call; the states are bit for bit the same.  Asynchronous: the
+ * return value reports launch errors only. */
 lbm_status lbm_step(lbm_handle* h, int64_t nsteps);
 
 /* Replace the uniform body force density F (Sec. 4: it shifts the velocity
@@ -166,6 +169,8 @@ lbm_status lbm_set_small_path(lbm_handle* h, int enable);
  * invalid; lbm_diagnostics and lbm_diagnostics_noalloc then return
  * LBM_ERR_TIMEOUT until lbm_init_fields, lbm_set_f or lbm_set_state gives
  * the handle a new state.  polls = 0 makes every such wait run out at once.
+ * (The kernels of small lattices and the two-step kernel wait at barriers
+ * of their own blocks only and give up none.)
  * Takes effect from the next lbm_step.  polls outside [0, 2^22]:
  * LBM_ERR_INVALID. */
 lbm_status lbm_set_wait_limit(lbm_handle* h, int64_t polls);

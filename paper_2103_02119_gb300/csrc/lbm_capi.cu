@@ -63,6 +63,7 @@ struct lbm_handle {
     unsigned wait_limit = lbm::kWaitPolls;  // polls of the step kernel's row wait
     int diag_blocks = 0;
     int bx = 0, nbands = 0;
+    int chain_bands = 0;       // bands of the two-step kernel (0: not used)
     int64_t steps = 0, launches = 0;
     uint8_t* bits = nullptr;   // small lattices: link bits of the nx * ny cells (device)
     bool small = false;        // steps run as one cluster launch (small_step.cu)
@@ -427,6 +428,19 @@ lbm_status step_lattice(lbm_handle* h, int64_t nsteps) {
         return LBM_OK;
     }
     int64_t left = nsteps;
+    if constexpr (sizeof(T) == 4) {
+        // Two steps per launch; the last one or two are single steps, so that
+        // the other buffer then holds the state one step earlier.
+        while (h->chain_bands && k.collide && left >= 3) {
+            CK(h, lbm::launch_chain2((const float*)h->f[h->cur], (float*)h->f[h->cur ^ 1], k,
+                                     h->chain_bands, h->stream),
+               "two-step kernel");
+            h->cur ^= 1;
+            h->launches += 1;
+            h->steps += 2;
+            left -= 2;
+        }
+    }
     while (left >= kRunSteps) {
         if (lbm_status st = ensure_run_graph<T>(h, k, h->cur); st != LBM_OK) return st;
         CK(h, cudaGraphLaunch(h->graph[h->cur], h->stream), "cudaGraphLaunch");
@@ -574,6 +588,18 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
     if (nb > p->ny) nb = p->ny;
     if (nb > 65535) nb = 65535;  // grid.y limit
     h->nbands = nb;
+    // Two steps per launch (chain_step.cuh) where that is faster than the
+    // row-band kernel; us a step, two-step / row-band kernel:
+    //   periodic 400 x 300 7.3 / 8.3, 2048 x 1024 28 / 39, 2048 x 8192 166 / 222;
+    //   cavities 400 x 300 10.3 / 7.3, 512^2 12.2 / 16.1, 2048 x 8192 170 / 209,
+    //   200 x 6000 (two of four strips along a wall) 28.7 / 25.3;
+    //   cavities with obstacles 512^2 15.5 / 17.2, 1001 x 2003 40 / 34 (two
+    //   buffers that the L2 nearly holds, and a launch as long as the chains
+    //   along the obstacles), 1543 x 3001 75 / 81, 2048 x 8192 199 / 215.
+    if (!f64 && !kRowInterleaved && h->N >= 200000 && (p->periodic_x || p->nx > 280) &&
+        !(solid_mask && h->N >= 1150000 && h->N < 3000000))
+        h->chain_bands = lbm::chain2_bands(p->nx, p->ny, h->pitch,
+                                            solid_mask != nullptr, sms);
     // small lattices: all the steps of an lbm_step call in one launch of one
     // thread-block cluster, when the device can hold it
     if (h->N <= lbm::kSmallCells && !kRowInterleaved) {

@@ -275,10 +275,16 @@ __device__ __forceinline__ float2 vneg(float2 a) { return make_float2(-a.x, -a.y
 __device__ __forceinline__ float2 vsub(float2 a, float2 b) { return __fadd2_rn(a, vneg(b)); }
 __device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-// FP32: the hardware reciprocal approximation (at most 2 ulp off, below the
-// FP32 storage rounding); FP64: an IEEE division.
+// FP32: the hardware reciprocal approximation (at most 1 ulp off, below the
+// FP32 storage rounding; one instruction, where __fdividef(1, a) takes five);
+// FP64: an IEEE division.
+__device__ __forceinline__ float rcp_approx(float a) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
 __device__ __forceinline__ float2 vrcp(float2 a) {
-    return make_float2(__fdividef(1.0f, a.x), __fdividef(1.0f, a.y));
+    return make_float2(rcp_approx(a.x), rcp_approx(a.y));
 }
 
 // Collision of one lane (Sec. 4) in increment form on deviations:
@@ -465,16 +471,16 @@ __device__ __forceinline__ typename Lane<T>::V collide_raw(const CollConst<T>& c
         for (int q = 0; q < 3; ++q) {
             const V s = vadd(gp[q], gm[q]);
             k0[q] = vadd(gz[q], s);
-            k1[q] = vmul(c.a, vsub(gp[q], gm[q]));
-            k2[q] = vmul(c.a2, s);
+            k1[q] = vmul(bc(c.a), vsub(gp[q], gm[q]));
+            k2[q] = vmul(bc(c.a2), s);
         }
     }
-    const V rho = vadd(c.rho0, d);
+    const V rho = vadd(bc(c.rho0), d);
     const V jx = vsub(k0[1], k0[2]);
     const V jy = vadd(vadd(k1[0], k1[1]), k1[2]);
     const V ir = vrcp(rho);
-    const V ux = vmul(vadd(jx, c.hFx), ir);
-    const V uy = vmul(vadd(jy, c.hFy), ir);
+    const V ux = vmul(vadd(jx, bc(c.hFx)), ir);
+    const V uy = vmul(vadd(jy, bc(c.hFy)), ir);
     V R[3][3];
     {
         const V* kq[3] = {k0, k1, k2};
@@ -491,58 +497,58 @@ __device__ __forceinline__ typename Lane<T>::V collide_raw(const CollConst<T>& c
     // yy and rho0 cs2^2 on xxyy.
     const V ux2 = vmul(ux, ux), uy2 = vmul(uy, uy);
     const V nd = vneg(d), nrho = vneg(rho);
-    const V n20 = vfma(nrho, ux2, vfma(nd, c.cs2, R[2][0]));
-    const V n02 = vfma(nrho, uy2, vfma(nd, c.cs2, R[0][2]));
+    const V n20 = vfma(nrho, ux2, vfma(nd, bc(c.cs2), R[2][0]));
+    const V n02 = vfma(nrho, uy2, vfma(nd, bc(c.cs2), R[0][2]));
     const V n11 = vfma(vmul(nrho, ux), uy, R[1][1]);
-    const V n21 = vfma(vmul(nrho, uy), vadd(c.cs2, ux2), R[2][1]);
-    const V n12 = vfma(vmul(nrho, ux), vadd(c.cs2, uy2), R[1][2]);
-    const V n22 = vfma(nrho, vfma(c.cs2, vadd(ux2, uy2), vmul(ux2, uy2)),
-                       vfma(nd, c.cs4, R[2][2]));
+    const V n21 = vfma(vmul(nrho, uy), vadd(bc(c.cs2), ux2), R[2][1]);
+    const V n12 = vfma(vmul(nrho, ux), vadd(bc(c.cs2), uy2), R[1][2]);
+    const V n22 = vfma(nrho, vfma(bc(c.cs2), vadd(ux2, uy2), vmul(ux2, uy2)),
+                       vfma(nd, bc(c.cs4), R[2][2]));
     const V N3 = vadd(n20, n02), N4 = vsub(n20, n02);
 
     // Local strain rates, Eq. 37-38, and corrections, Eq. 23-26.
-    const V b1 = vfma(c.c15, ux2, c.b1c), b2 = vfma(c.c15, uy2, c.b2c);
-    const V c1 = vfma(c.c15, ux2, c.c1c), c2 = vfma(c.nc15, uy2, c.c2c);
-    const V gx = vmul(vmul(c.g1h, ux), dxr), gy = vmul(vmul(c.g2h, uy), dyr);
+    const V b1 = vfma(bc(c.c15), ux2, bc(c.b1c)), b2 = vfma(bc(c.c15), uy2, bc(c.b2c));
+    const V c1 = vfma(bc(c.c15), ux2, bc(c.c1c)), c2 = vfma(bc(c.nc15), uy2, bc(c.c2c));
+    const V gx = vmul(vmul(bc(c.g1h), ux), dxr), gy = vmul(vmul(bc(c.g2h), uy), dyr);
     const V R3 = vadd(vadd(N3, gx), gy);
     const V R4 = vsub(vadd(N4, gx), gy);
     const V idet = vrcp(vmul(rho, vfma(b1, c2, vmul(vneg(b2), c1))));
     const V dxux = vmul(vfma(c2, R3, vmul(vneg(b2), R4)), idet);
     const V dyuy = vmul(vfma(b1, R4, vmul(vneg(c1), R3)), idet);
     const V rdx = vmul(rho, dxux), rdy = vmul(rho, dyuy);
-    const V Px = vfma(c.g1i, vfma(ux, dxr, rdx), vmul(vmul(c.ng3, rdx), ux2));
-    const V Py = vfma(c.g2i, vfma(uy, dyr, rdy), vmul(vmul(c.ng3, rdy), uy2));
+    const V Px = vfma(bc(c.g1i), vfma(ux, dxr, rdx), vmul(vmul(bc(c.ng3), rdx), ux2));
+    const V Py = vfma(bc(c.g2i), vfma(uy, dyr, rdy), vmul(vmul(bc(c.ng3), rdy), uy2));
 
     // Relaxation with the raw source moments of Eq. 13: increments of the
     // raw moments.  m1 relaxes to rho ux = m1 + Fx/2, so its increment is Fx
     // whatever omega_1 (same for m2).
-    const V uFx = vmul(ux, c.Fx), uFy = vmul(uy, c.Fy);
-    const V dm3 = vfma(c.lw3, vfma(c.two, vadd(uFx, uFy), vadd(Px, Py)), vmul(c.nw3, N3));
-    const V dm4 = vfma(c.lw4, vfma(c.two, vsub(uFx, uFy), vsub(Px, Py)), vmul(c.nw4, N4));
-    const V D20 = vmul(c.half, vadd(dm3, dm4)), D02 = vmul(c.half, vsub(dm3, dm4));
-    const V D11 = vfma(c.lw5, vfma(c.Fx, uy, vmul(c.Fy, ux)), vmul(c.nw5, n11));
-    const V D21 = vfma(c.lw6, vfma(c.Fy, ux2, vmul(vmul(c.twoFx, ux), uy)), vmul(c.nw6, n21));
-    const V D12 = vfma(c.lw7, vfma(c.Fx, uy2, vmul(vmul(c.twoFy, ux), uy)), vmul(c.nw7, n12));
-    const V D22 = vfma(c.lw8, vmul(c.two, vfma(uFx, uy2, vmul(uFy, ux2))), vmul(c.nw8, n22));
+    const V uFx = vmul(ux, bc(c.Fx)), uFy = vmul(uy, bc(c.Fy));
+    const V dm3 = vfma(bc(c.lw3), vfma(bc(c.two), vadd(uFx, uFy), vadd(Px, Py)), vmul(bc(c.nw3), N3));
+    const V dm4 = vfma(bc(c.lw4), vfma(bc(c.two), vsub(uFx, uFy), vsub(Px, Py)), vmul(bc(c.nw4), N4));
+    const V D20 = vmul(bc(c.half), vadd(dm3, dm4)), D02 = vmul(bc(c.half), vsub(dm3, dm4));
+    const V D11 = vfma(bc(c.lw5), vfma(bc(c.Fx), uy, vmul(bc(c.Fy), ux)), vmul(bc(c.nw5), n11));
+    const V D21 = vfma(bc(c.lw6), vfma(bc(c.Fy), ux2, vmul(vmul(bc(c.twoFx), ux), uy)), vmul(bc(c.nw6), n21));
+    const V D12 = vfma(bc(c.lw7), vfma(bc(c.Fx), uy2, vmul(vmul(bc(c.twoFy), ux), uy)), vmul(bc(c.nw7), n12));
+    const V D22 = vfma(bc(c.lw8), vmul(bc(c.two), vfma(uFx, uy2, vmul(uFy, ux2))), vmul(bc(c.nw8), n22));
 
     // Back along x (raw x-moments -> columns), then along y.
     V h[3][3];
     h[0][0] = vneg(D20);
-    h[1][0] = vmul(c.half, vadd(D20, c.Fx));
-    h[2][0] = vmul(c.half, vsub(D20, c.Fx));
-    h[0][1] = vsub(c.Fy, D21);
-    h[1][1] = vmul(c.half, vadd(D21, D11));
-    h[2][1] = vmul(c.half, vsub(D21, D11));
+    h[1][0] = vmul(bc(c.half), vadd(D20, bc(c.Fx)));
+    h[2][0] = vmul(bc(c.half), vsub(D20, bc(c.Fx)));
+    h[0][1] = vsub(bc(c.Fy), D21);
+    h[1][1] = vmul(bc(c.half), vadd(D21, D11));
+    h[2][1] = vmul(bc(c.half), vsub(D21, D11));
     h[0][2] = vsub(D02, D22);
-    h[1][2] = vmul(c.half, vadd(D22, D12));
-    h[2][2] = vmul(c.half, vsub(D22, D12));
+    h[1][2] = vmul(bc(c.half), vadd(D22, D12));
+    h[2][2] = vmul(bc(c.half), vsub(D22, D12));
     {
         const int iz[3] = {0, 1, 3}, ip[3] = {2, 5, 6}, im[3] = {4, 8, 7};
 #pragma unroll
         for (int X = 0; X < 3; ++X) {
-            f[iz[X]] = vadd(f[iz[X]], vfma(c.nia2, h[X][2], h[X][0]));
-            f[ip[X]] = vfma(c.iah2, h[X][2], vfma(c.iah, h[X][1], f[ip[X]]));
-            f[im[X]] = vfma(c.iah2, h[X][2], vfma(c.niah, h[X][1], f[im[X]]));
+            f[iz[X]] = vadd(f[iz[X]], vfma(bc(c.nia2), h[X][2], h[X][0]));
+            f[ip[X]] = vfma(bc(c.iah2), h[X][2], vfma(bc(c.iah), h[X][1], f[ip[X]]));
+            f[im[X]] = vfma(bc(c.iah2), h[X][2], vfma(bc(c.niah), h[X][1], f[im[X]]));
         }
     }
     return rho;

@@ -38,6 +38,16 @@ cudaError_t launch_step_rnr(const T* fin, T* fout, const KParams<T>& p, int bx, 
 template <typename T>
 cudaError_t launch_step_free(const T* fin, T* fout, const KParams<T>& p, int bx, int nbands,
                              cudaStream_t s);
+// Two steps of an FP32 lattice in one launch (chain_step.cuh): fin holds the
+// state, fout the state two steps later; p.collide set.  nbands: chain2_bands.
+cudaError_t launch_chain2(const float* fin, float* fout, const KParams<float>& p, int nbands,
+                          cudaStream_t s);
+// Bands of the lattice for launch_chain2 on a device of `sms` SMs: the fewest
+// clocks by a model of the march (a row of a chain takes longer the more
+// chains share its SM; every band marches ten rows more than it stores; the
+// launch ends when its slowest chain does, uneven: solid
+// cells, whose chains take longer); 0 when the lattice cannot take the path.
+int chain2_bands(int nx, int ny, int pitch, bool uneven, int sms);
 template <typename T>
 int step_occupancy(int bx, bool mask);
 
