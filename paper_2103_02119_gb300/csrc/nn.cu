@@ -39,7 +39,7 @@ namespace {
 using bf16 = __nv_bfloat16;
 
 constexpr int kThreads = 256;
-constexpr int kSplitPixels = 4096;  // pixels per block of the weight-gradient GEMM
+constexpr unsigned kBiasBlocks = 304;  // most blocks of one launch of the bias-gradient sums
 
 // Division by a divisor fixed at launch, for dividends in [0, 2^31):
 // q = (n m) >> s with m = ceil(2^s / d), s = 31 + ceil(log2 d) (exact in that
@@ -482,89 +482,157 @@ cudaError_t launch_gemm(const Op& op, long long kchunk, int splits, int* err, cu
 
 // ---- elementwise and reduction kernels ----
 
-__global__ void relu_mask_kernel(const bf16* out, const bf16* g, bf16* gpre, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        gpre[i] = __bfloat162float(out[i]) > 0.0f ? g[i] : __float2bfloat16_rn(0.0f);
+// Eight channels of one pixel (16 bytes; channel counts are padded to
+// multiples of 8) at a time, with 32-bit index arithmetic: the scalar forms
+// spent most of their time on 64-bit divisions.
+struct Oct {
+    float v[8];
+};
+__device__ __forceinline__ Oct load8(const bf16* p) {
+    const uint4 q = *reinterpret_cast<const uint4*>(p);
+    const unsigned w[4] = {q.x, q.y, q.z, q.w};
+    Oct o;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        o.v[2 * k] = __uint_as_float(w[k] << 16);
+        o.v[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
+    }
+    return o;
 }
+__device__ __forceinline__ void store8(bf16* p, const Oct& o) {
+    unsigned w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(o.v[2 * k], o.v[2 * k + 1]);
+        w[k] = *reinterpret_cast<const unsigned*>(&h);
+    }
+    *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+// Octet i of an (n, h, w, 8 c8) tensor: its pixel and channel group.
+struct At {
+    unsigned p, y, x, g;
+    unsigned long long off;  // element offset
+    __device__ __forceinline__ At(unsigned i, const FastDiv& c8, const FastDiv& fw,
+                                  const FastDiv& fh) {
+        p = c8.div(i);
+        g = i - p * c8.d;
+        const unsigned r = fw.div(p);
+        x = p - r * fw.d;
+        y = r - fh.div(r) * fh.d;
+        off = 8ull * i;
+    }
+};
 
-// 2x2 average: (((x00 + x10) + x01) + x11) / 4, rounded once.
-__global__ void pool_kernel(const bf16* in, bf16* out, int n, int h, int w, int c) {
-    const int ho = h / 2, wo = w / 2;
-    const long long total = (long long)n * ho * wo * c;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = (int)(i % c);
-        long long r = i / c;
-        const int x = (int)(r % wo);
-        r /= wo;
-        const int y = (int)(r % ho);
-        const int nn = (int)(r / ho);
-        auto at = [&](int yy, int xx) {
-            return __bfloat162float(in[(((long long)nn * h + yy) * w + xx) * c + ch]);
-        };
-        const float s = ((at(2 * y, 2 * x) + at(2 * y + 1, 2 * x)) + at(2 * y, 2 * x + 1)) +
-                        at(2 * y + 1, 2 * x + 1);
-        out[i] = __float2bfloat16_rn(0.25f * s);
+// 2x2 average: (((x00 + x10) + x01) + x11) / 4, rounded once.  total: output octets
+__global__ void __launch_bounds__(kThreads)
+pool_kernel(const bf16* in, bf16* out, unsigned total, FastDiv c8, FastDiv fwo, FastDiv fho) {
+    const unsigned c = 8 * c8.d, row = 2 * fwo.d * c;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += gridDim.x * blockDim.x) {
+        const At t(i, c8, fwo, fho);
+        // output row r of (n, ho) has its input rows at 2 r, 2 r + 1 of (n, h)
+        const bf16* q = in + 2ull * fwo.div(t.p) * row + 2ull * t.x * c + 8 * t.g;
+        const Oct a = load8(q), b = load8(q + row), d = load8(q + c), e = load8(q + row + c);
+        Oct o;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o.v[k] = 0.25f * (((a.v[k] + b.v[k]) + d.v[k]) + e.v[k]);
+        store8(out + t.off, o);
     }
 }
 
-// gin(2y+a, 2x+b) = 0.25 g(y, x) + gin(2y+a, 2x+b) (the skip gradient already there)
-__global__ void pool_back_kernel(const bf16* g, bf16* gin, int n, int h, int w, int c,
-                                 int accumulate) {
-    const long long total = (long long)n * h * w * c;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = (int)(i % c);
-        long long r = i / c;
-        const int x = (int)(r % w);
-        r /= w;
-        const int y = (int)(r % h);
-        const int nn = (int)(r / h);
-        const float v =
-            0.25f * __bfloat162float(g[(((long long)nn * (h / 2) + y / 2) * (w / 2) + x / 2) * c + ch]);
-        gin[i] = __float2bfloat16_rn(accumulate ? v + __bfloat162float(gin[i]) : v);
+// gin(2y+a, 2x+b) = 0.25 g(y, x) + gin(2y+a, 2x+b) (the skip gradient already
+// there).  total: octets of gin (n, h, w)
+__global__ void __launch_bounds__(kThreads)
+pool_back_kernel(const bf16* g, bf16* gin, unsigned total, FastDiv c8, FastDiv fw, FastDiv fh) {
+    const unsigned c = 8 * c8.d;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += gridDim.x * blockDim.x) {
+        const At t(i, c8, fw, fh);
+        // rows come in pairs (h is even), so row r of (n, h) lies under r / 2
+        const unsigned long long q =
+            ((unsigned long long)(fw.div(t.p) / 2) * (fw.d / 2) + t.x / 2) * c + 8 * t.g;
+        const Oct a = load8(g + q), b = load8(gin + t.off);
+        Oct o;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o.v[k] = 0.25f * a.v[k] + b.v[k];
+        store8(gin + t.off, o);
     }
 }
 
-__global__ void up_kernel(const bf16* in, bf16* out, int n, int h, int w, int c) {
-    // out is (n, 2h, 2w, c)
-    const long long total = (long long)n * 4 * h * w * c;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = (int)(i % c);
-        long long r = i / c;
-        const int x = (int)(r % (2 * w));
-        r /= 2 * w;
-        const int y = (int)(r % (2 * h));
-        const int nn = (int)(r / (2 * h));
-        out[i] = in[(((long long)nn * h + y / 2) * w + x / 2) * c + ch];
+// out (n, 2h, 2w) from in (n, h, w).  total: output octets
+__global__ void __launch_bounds__(kThreads)
+up_kernel(const bf16* in, bf16* out, unsigned total, FastDiv c8, FastDiv fwo, FastDiv fho) {
+    const unsigned c = 8 * c8.d;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += gridDim.x * blockDim.x) {
+        const At t(i, c8, fwo, fho);
+        const unsigned long long q =
+            ((unsigned long long)(fwo.div(t.p) / 2) * (fwo.d / 2) + t.x / 2) * c + 8 * t.g;
+        *reinterpret_cast<uint4*>(out + t.off) = __ldg(reinterpret_cast<const uint4*>(in + q));
     }
 }
 
-// gin(y, x) = ((g(2y,2x) + g(2y+1,2x)) + g(2y,2x+1)) + g(2y+1,2x+1), rounded once
-__global__ void up_back_kernel(const bf16* g, bf16* gin, int n, int h, int w, int c) {
-    const long long total = (long long)n * h * w * c;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ch = (int)(i % c);
-        long long r = i / c;
-        const int x = (int)(r % w);
-        r /= w;
-        const int y = (int)(r % h);
-        const int nn = (int)(r / h);
-        auto at = [&](int yy, int xx) {
-            return __bfloat162float(g[(((long long)nn * 2 * h + yy) * 2 * w + xx) * c + ch]);
-        };
-        gin[i] = __float2bfloat16_rn(((at(2 * y, 2 * x) + at(2 * y + 1, 2 * x)) +
-                                      at(2 * y, 2 * x + 1)) + at(2 * y + 1, 2 * x + 1));
+// gin(y, x) = ((g(2y,2x) + g(2y+1,2x)) + g(2y,2x+1)) + g(2y+1,2x+1), rounded
+// once.  total: octets of gin (n, h, w)
+__global__ void __launch_bounds__(kThreads)
+up_back_kernel(const bf16* g, bf16* gin, unsigned total, FastDiv c8, FastDiv fw, FastDiv fh) {
+    const unsigned c = 8 * c8.d, row = 2 * fw.d * c;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += gridDim.x * blockDim.x) {
+        const At t(i, c8, fw, fh);
+        const bf16* q = g + 2ull * fw.div(t.p) * row + 2ull * t.x * c + 8 * t.g;
+        const Oct a = load8(q), b = load8(q + row), d = load8(q + c), e = load8(q + row + c);
+        Oct o;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o.v[k] = ((a.v[k] + b.v[k]) + d.v[k]) + e.v[k];
+        store8(gin + t.off, o);
     }
 }
 
-__global__ void add_kernel(const bf16* a, const bf16* b, bf16* out, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        out[i] = __float2bfloat16_rn(__bfloat162float(a[i]) + __bfloat162float(b[i]));
+__global__ void __launch_bounds__(kThreads)
+add_kernel(const bf16* a, const bf16* b, bf16* out, unsigned total) {
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += gridDim.x * blockDim.x) {
+        const Oct x = load8(a + 8ull * i), y = load8(b + 8ull * i);
+        Oct o;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o.v[k] = x.v[k] + y.v[k];
+        store8(out + 8ull * i, o);
+    }
+}
+
+// The gradient before the ReLU, gpre = g where out > 0, else 0 (RELU; gpre may
+// not alias g), and its sums over the pixels of every block: part[block][8 c8].
+// A thread keeps one channel group (its octets are a multiple of c8 apart), so
+// the bias gradient costs no pass of its own; the block adds its threads'
+// sums in a fixed order.  blockDim.x is a multiple of c8.
+template <bool RELU>
+__global__ void __launch_bounds__(512)
+relu_bias_kernel(const bf16* out, const bf16* g, bf16* gpre, unsigned total, int c8, float* part) {
+    __shared__ float sh[512][9];
+    Oct s;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s.v[k] = 0.0f;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += gridDim.x * blockDim.x) {
+        Oct x = load8(g + 8ull * i);
+        if (RELU) {
+            const Oct o = load8(out + 8ull * i);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x.v[k] = o.v[k] > 0.0f ? x.v[k] : 0.0f;
+            store8(gpre + 8ull * i, x);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s.v[k] += x.v[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) sh[threadIdx.x][k] = s.v[k];
+    __syncthreads();
+    for (int c = threadIdx.x; c < 8 * c8; c += blockDim.x) {
+        float t = 0.0f;
+        for (int r = c >> 3; r < (int)blockDim.x; r += c8) t += sh[r][c & 7];
+        part[(long long)blockIdx.x * 8 * c8 + c] = t;
+    }
 }
 
 // host float inputs (n, h, w, 4) -> bf16 (n, h, w, 8) with zero channels 4..7
@@ -659,17 +727,20 @@ __global__ void out_smooth_kernel(const void* in, int icp, FL fluid, void* out, 
     }
 }
 
-// Block k: sums over the fluid cells of instance k of (-1)^x v1, (-1)^y v2 and
-// the cell count, in a fixed order.
+// Block (j, k): sums over part j of the fluid cells of instance k of (-1)^x v1,
+// (-1)^y v2 and the cell count, in a fixed order, to sums[k][j][3].  (One block
+// per instance took 26 us for 16 instances of 64 x 64.)
+constexpr int kStaggerParts = 16;
 template <typename FL>
 __global__ void __launch_bounds__(kThreads) stagger_sum_kernel(const float* v, FL fluid,
                                                                double* sums, int h, int w) {
-    const long long hw = (long long)h * w, p0 = (long long)blockIdx.x * hw;
+    const long long hw = (long long)h * w, p0 = (long long)blockIdx.y * hw;
     double s1 = 0.0, s2 = 0.0, nf = 0.0;
-    for (long long i = threadIdx.x; i < hw; i += blockDim.x) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < hw;
+         i += kStaggerParts * (long long)blockDim.x) {
         const long long p = p0 + i;
         if (!fluid(p)) continue;
-        const int x = (int)(i % w), y = (int)(i / w);
+        const unsigned y = (unsigned)i / (unsigned)w, x = (unsigned)i - y * (unsigned)w;
         s1 += (x & 1) ? -(double)v[p * 3 + 1] : (double)v[p * 3 + 1];
         s2 += (y & 1) ? -(double)v[p * 3 + 2] : (double)v[p * 3 + 2];
         nf += 1.0;
@@ -678,26 +749,41 @@ __global__ void __launch_bounds__(kThreads) stagger_sum_kernel(const float* v, F
     s2 = block_sum(s2);
     nf = block_sum(nf);
     if (threadIdx.x == 0) {
-        sums[3 * blockIdx.x] = s1;
-        sums[3 * blockIdx.x + 1] = s2;
-        sums[3 * blockIdx.x + 2] = nf;
+        double* o = sums + 3 * ((long long)blockIdx.y * kStaggerParts + blockIdx.x);
+        o[0] = s1;
+        o[1] = s2;
+        o[2] = nf;
     }
 }
 
+// Block (j, k) applies the projection to part j of instance k.
 template <typename FL>
-__global__ void stagger_apply_kernel(const float* v, FL fluid, const double* sums, float* out,
-                                     long long P, int h, int w) {
-    const long long hw = (long long)h * w;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P;
-         p += (long long)gridDim.x * blockDim.x) {
-        const long long k = p / hw, i = p - k * hw;
-        const int x = (int)(i % w), y = (int)(i / w);
+__global__ void __launch_bounds__(kThreads)
+stagger_apply_kernel(const float* v, FL fluid, const double* sums, float* out, int h, int w) {
+    __shared__ float c[2];
+    __shared__ int any;
+    const long long hw = (long long)h * w, p0 = (long long)blockIdx.y * hw;
+    if (threadIdx.x == 0) {
+        const double* q = sums + 3 * (long long)blockIdx.y * kStaggerParts;
+        double s1 = 0.0, s2 = 0.0, nf = 0.0;
+        for (int j = 0; j < kStaggerParts; ++j) {
+            s1 += q[3 * j];
+            s2 += q[3 * j + 1];
+            nf += q[3 * j + 2];
+        }
+        any = nf > 0.0;
+        c[0] = nf > 0.0 ? (float)(s1 / nf) : 0.0f;
+        c[1] = nf > 0.0 ? (float)(s2 / nf) : 0.0f;
+    }
+    __syncthreads();
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < hw;
+         i += gridDim.x * (long long)blockDim.x) {
+        const long long p = p0 + i;
+        const unsigned y = (unsigned)i / (unsigned)w, x = (unsigned)i - y * (unsigned)w;
         float o1 = v[p * 3 + 1], o2 = v[p * 3 + 2];
-        const double nf = sums[3 * k + 2];
-        if (nf > 0.0 && fluid(p)) {
-            const float c1 = (float)(sums[3 * k] / nf), c2 = (float)(sums[3 * k + 1] / nf);
-            o1 -= (x & 1) ? -c1 : c1;
-            o2 -= (y & 1) ? -c2 : c2;
+        if (any && fluid(p)) {
+            o1 -= (x & 1) ? -c[0] : c[0];
+            o2 -= (y & 1) ? -c[1] : c[1];
         }
         out[p * 3] = v[p * 3];
         out[p * 3 + 1] = o1;
@@ -772,24 +858,22 @@ __global__ void __launch_bounds__(kThreads) sum_kernel(const double* part, int n
     if (threadIdx.x == 0) *out = b;
 }
 
-// bias gradient: gb[co] = sum_p gpre[p][co], one block per channel
-__global__ void __launch_bounds__(kThreads) bias_grad_kernel(const bf16* gpre, float* gb,
-                                                             long long pixels, int cout) {
-    const int co = blockIdx.x;
-    float s = 0.0f;
-    for (long long p = threadIdx.x; p < pixels; p += blockDim.x)
-        s += __bfloat162float(gpre[p * cout + co]);
-    const float b = block_sum(s);
-    if (threadIdx.x == 0) gb[co] = b;
-}
-
-// dW = sum over the splits in order
-__global__ void split_sum_kernel(const float* part, float* gw, int splits, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+// dW = sum over the splits in order, and gb = sum over the bias partials in
+// order (in the threads after the weights').
+__global__ void __launch_bounds__(kThreads)
+split_sum_kernel(const float* part, float* gw, int splits, long long n, const float* bpart,
+                 float* gb, int bparts, int cout) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n + cout;
          i += (long long)gridDim.x * blockDim.x) {
+        const bool w = i < n;
+        const float* q = w ? part + i : bpart + (i - n);
+        const long long step = w ? n : cout;
+        const int terms = w ? splits : bparts;
         float s = 0.0f;
-        for (int z = 0; z < splits; ++z) s += part[(long long)z * n + i];
-        gw[i] = s;
+#pragma unroll 8
+        for (int z = 0; z < terms; ++z) s += q[z * step];
+        if (w) gw[i] = s;
+        else gb[i - n] = s;
     }
 }
 
@@ -821,6 +905,43 @@ __global__ void weight_copies_kernel(const float* wm, bf16* wf, bf16* wd, int ci
         wf[i] = v;
         wd[((long long)ci * 9 + tap) * cout + co] = v;
     }
+}
+
+// The host's parameter order (dy, dx, cin, cout, then the biases) from or to a
+// convolution's device arrays w [coutp][9][cinp], b [coutp].  A block moves a
+// tile of 32 input by 32 output channels of one tap through shared memory, so
+// that both sides are read and written in rows.
+template <bool TO_HOST>
+__global__ void __launch_bounds__(kThreads)
+param_order_kernel(float* host, float* w, float* b, int cin, int cout, int cinp) {
+    __shared__ float t[32][33];
+    const int tap = blockIdx.z, ci0 = blockIdx.y * 32, co0 = blockIdx.x * 32;
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    for (int r = y; r < 32; r += kThreads / 32) {
+        if (TO_HOST) {  // rows of the device array: ci across
+            const int co = co0 + r, ci = ci0 + x;
+            if (co < cout && ci < cin) t[r][x] = w[((long long)co * 9 + tap) * cinp + ci];
+        } else {        // rows of the host array: co across
+            const int ci = ci0 + r, co = co0 + x;
+            if (co < cout && ci < cin) t[x][r] = host[((long long)tap * cin + ci) * cout + co];
+        }
+    }
+    __syncthreads();
+    for (int r = y; r < 32; r += kThreads / 32) {
+        if (TO_HOST) {
+            const int ci = ci0 + r, co = co0 + x;
+            if (co < cout && ci < cin) host[((long long)tap * cin + ci) * cout + co] = t[x][r];
+        } else {
+            const int co = co0 + r, ci = ci0 + x;
+            if (co < cout && ci < cin) w[((long long)co * 9 + tap) * cinp + ci] = t[r][x];
+        }
+    }
+    if (tap == 0 && blockIdx.y == 0)
+        for (int k = threadIdx.x; k < 32 && co0 + k < cout; k += kThreads) {
+            float* hb = host + 9ll * cin * cout + co0 + k;
+            if (TO_HOST) *hb = b[co0 + k];
+            else b[co0 + k] = *hb;
+        }
 }
 
 int grid_of(long long n) {
@@ -864,7 +985,10 @@ struct lbm_nn {
     unsigned char* abuf = nullptr;  // activations and gradients
     bf16* scratch = nullptr;   // relu-masked gradient
     float* part = nullptr;     // weight-gradient split partials
-    size_t part_floats = 0;
+    float* bpart = nullptr;    // bias-gradient partials [runs kBiasBlocks][coutp]
+    float* flat = nullptr;     // a parameter vector in the host's order
+    int sms = 1;
+    long long nfluid = 0;      // fluid cells of the batch at hand
     double* dpart = nullptr;   // loss partials (+1 for the total)
     float* xin = nullptr;      // staging of host inputs (float)
     float* tgt = nullptr;
@@ -872,7 +996,7 @@ struct lbm_nn {
     float* yout = nullptr;     // the network's output after the output stage [P][3]
     float* gout = nullptr;     // the loss gradient of yout [P][3]
     float* tmp3 = nullptr;     // the output stage's intermediate [P][3]
-    double* ssum = nullptr;    // per instance: the staggered sums and fluid count
+    double* ssum = nullptr;    // per instance and part: the staggered sums and fluid count
     float* fine = nullptr;     // lbm_nn_prolong: two fine fields [max_batch][H f][W f][3]
     uint8_t* fine_fl = nullptr;  // and their fluid flags
     long long fine_cells = 0;  // cells per fine field the buffers hold
@@ -907,6 +1031,28 @@ int pad8(int c) { return (c + 7) / 8 * 8; }
 
 long long pixels(const lbm_nn* nn, int id, int n) {
     return (long long)n * nn->t[id].h * nn->t[id].w;
+}
+
+// f(first instance, octets) over the batch in runs of instances whose tensor
+// `id` has fewer than 2^31 groups of eight channels (one run but for the very
+// largest batches; an instance has at most 2^30).
+template <class F>
+cudaError_t by_octets(const lbm_nn* nn, int id, int n, const F& f) {
+    const long long one = (long long)nn->t[id].h * nn->t[id].w * (nn->t[id].cp / 8);
+    const int most = (int)(((1LL << 31) - 1) / one);
+    for (int i = 0; i < n; i += most) {
+        const int m = n - i < most ? n - i : most;
+        f(i, (unsigned)(m * one));
+        if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+// the address of instance i of an activation or gradient of tensor `id`
+const bf16* instance(const lbm_nn* nn, int id, const bf16* v, int i) {
+    return v + (long long)i * nn->t[id].h * nn->t[id].w * nn->t[id].cp;
+}
+bf16* instance(const lbm_nn* nn, int id, bf16* v, int i) {
+    return v + (long long)i * nn->t[id].h * nn->t[id].w * nn->t[id].cp;
 }
 
 int add_tensor(lbm_nn* nn, int h, int w, int c) {
@@ -994,18 +1140,33 @@ lbm_status upload_inputs(lbm_nn* nn, const float* x, const float* tgt, const uin
     pack_input_kernel<<<grid_of(P * X.cp), kThreads, 0, nn->stream>>>(nn->xin, X.v, P, 4, X.cp);
     NCK(nn, cudaGetLastError(), "input packing");
     ++nn->launches;
+    if (fluid) {
+        nn->nfluid = 0;
+        for (long long i = 0; i < P; ++i) nn->nfluid += fluid[i] != 0;
+    }
     return LBM_OK;
+}
+
+// Splits of a weight gradient's pixels over CTAs, and pixels per split: two
+// CTAs per SM, with at least 256 pixels each.  (Splits of 4096 pixels left most
+// SMs idle: 94 us a convolution of 16 x 64 x 64 pixels on average.)
+void wgrad_splits(const lbm_nn* nn, const lbm_nn::Conv& c, long long P, int& splits,
+                  long long& kchunk) {
+    const long long tiles = ((9LL * c.cinp + UM - 1) / UM) * ((c.coutp + 255) / 256);
+    long long s = (2LL * nn->sms + tiles - 1) / tiles;
+    if (s > (P + 255) / 256) s = (P + 255) / 256;
+    kchunk = ((P + s - 1) / s + UK - 1) / UK * UK;
+    splits = (int)((P + kchunk - 1) / kchunk);
 }
 
 // out = the staggered projection of v (FP32 [P][3] each), per instance.
 lbm_status unstagger(lbm_nn* nn, int n, const float* v, float* out) {
     const lbm_nn::Tensor& X = nn->t[nn->x_id];
-    const long long P = pixels(nn, nn->x_id, n);
     const FluidIn fl{X.v, X.cp};
-    stagger_sum_kernel<<<n, kThreads, 0, nn->stream>>>(v, fl, nn->ssum, X.h, X.w);
+    const dim3 g(kStaggerParts, n);
+    stagger_sum_kernel<<<g, kThreads, 0, nn->stream>>>(v, fl, nn->ssum, X.h, X.w);
     NCK(nn, cudaGetLastError(), "staggered sums");
-    stagger_apply_kernel<<<grid_of(P), kThreads, 0, nn->stream>>>(v, fl, nn->ssum, out, P, X.h,
-                                                                  X.w);
+    stagger_apply_kernel<<<g, kThreads, 0, nn->stream>>>(v, fl, nn->ssum, out, X.h, X.w);
     NCK(nn, cudaGetLastError(), "staggered projection");
     nn->launches += 3;  // with the smoothing launched beside it
     return LBM_OK;
@@ -1031,19 +1192,26 @@ lbm_status forward(lbm_nn* nn, int n) {
             e = launch_gemm(f, f.K(), 1, nn->gemm_err, s);
         } else if (op.k == lbm_nn::POOL) {
             const lbm_nn::Tensor& X = nn->t[op.a];
-            pool_kernel<<<grid_of(pixels(nn, op.out, n) * X.cp), kThreads, 0, s>>>(
-                X.v, nn->t[op.out].v, n, X.h, X.w, X.cp);
-            e = cudaGetLastError();
+            const lbm_nn::Tensor& O = nn->t[op.out];
+            e = by_octets(nn, op.out, n, [&](int i, unsigned t) {
+                pool_kernel<<<grid_of(t), kThreads, 0, s>>>(
+                    instance(nn, op.a, X.v, i), instance(nn, op.out, O.v, i), t, FastDiv(X.cp / 8),
+                    FastDiv(O.w), FastDiv(O.h));
+            });
         } else if (op.k == lbm_nn::UP) {
             const lbm_nn::Tensor& X = nn->t[op.a];
-            up_kernel<<<grid_of(pixels(nn, op.out, n) * X.cp), kThreads, 0, s>>>(
-                X.v, nn->t[op.out].v, n, X.h, X.w, X.cp);
-            e = cudaGetLastError();
+            const lbm_nn::Tensor& O = nn->t[op.out];
+            e = by_octets(nn, op.out, n, [&](int i, unsigned t) {
+                up_kernel<<<grid_of(t), kThreads, 0, s>>>(
+                    instance(nn, op.a, X.v, i), instance(nn, op.out, O.v, i), t, FastDiv(X.cp / 8),
+                    FastDiv(O.w), FastDiv(O.h));
+            });
         } else {
-            const long long cnt = pixels(nn, op.out, n) * nn->t[op.out].cp;
-            add_kernel<<<grid_of(cnt), kThreads, 0, s>>>(nn->t[op.a].v, nn->t[op.b].v,
-                                                         nn->t[op.out].v, cnt);
-            e = cudaGetLastError();
+            e = by_octets(nn, op.out, n, [&](int i, unsigned t) {
+                add_kernel<<<grid_of(t), kThreads, 0, s>>>(
+                    instance(nn, op.a, nn->t[op.a].v, i), instance(nn, op.b, nn->t[op.b].v, i),
+                    instance(nn, op.out, nn->t[op.out].v, i), t);
+            });
         }
         NCK(nn, e, "forward kernels");
         ++nn->launches;
@@ -1063,12 +1231,7 @@ lbm_status forward(lbm_nn* nn, int n) {
 lbm_status backward(lbm_nn* nn, int n, float* loss) {
     const cudaStream_t s = nn->stream;
     const long long P = (long long)n * nn->H * nn->W;
-    std::vector<uint8_t> host_fl(P);
-    NCK(nn, cudaMemcpyAsync(host_fl.data(), nn->fl, P, cudaMemcpyDeviceToHost, s),
-        "cudaMemcpyAsync(D2H)");
-    NCK(nn, cudaStreamSynchronize(s), "cudaStreamSynchronize");
-    long long nf = 0;
-    for (long long i = 0; i < P; ++i) nf += host_fl[i] != 0;
+    const long long nf = nn->nfluid;
     const float inv_cnt = nf > 0 ? (float)(1.0 / (3.0 * (double)nf)) : 0.0f;
     std::vector<bf16*> G(nn->t.size());
     for (size_t i = 0; i < nn->t.size(); ++i) G[i] = nn->t[i].g;
@@ -1096,16 +1259,28 @@ lbm_status backward(lbm_nn* nn, int n, float* loss) {
             const lbm_nn::Tensor& X = nn->t[c.in];
             const lbm_nn::Tensor& O = nn->t[c.out];
             const long long Pc = pixels(nn, c.in, n);
-            const bf16* gpre = G[c.out];
-            if (c.relu) {
-                relu_mask_kernel<<<grid_of(Pc * O.cp), kThreads, 0, s>>>(O.v, G[c.out], nn->scratch,
-                                                                         Pc * O.cp);
-                if ((e = cudaGetLastError()) != cudaSuccess) break;
-                ++nn->launches;
-                gpre = nn->scratch;
-            }
+            const bf16* gpre = c.relu ? nn->scratch : G[c.out];
+            // the gradient before the ReLU and the bias partials
+            const int c8 = O.cp / 8, bt = 512 / c8 * c8;
+            int bb = 0;  // partials so far
+            e = by_octets(nn, c.out, n, [&](int i, unsigned t) {
+                const unsigned want = (t + bt - 1) / bt;
+                const int blocks = (int)(want < kBiasBlocks ? want : kBiasBlocks);
+                float* part = nn->bpart + (long long)bb * 8 * c8;
+                const bf16* o = instance(nn, c.out, O.v, i);
+                const bf16* g = instance(nn, c.out, (const bf16*)G[c.out], i);
+                if (c.relu)
+                    relu_bias_kernel<true><<<blocks, bt, 0, s>>>(
+                        o, g, instance(nn, c.out, nn->scratch, i), t, c8, part);
+                else
+                    relu_bias_kernel<false><<<blocks, bt, 0, s>>>(o, g, nullptr, t, c8, part);
+                bb += blocks;
+            });
+            if (e != cudaSuccess) break;
             // weight gradient, split over pixels
-            const int splits = (int)((Pc + kSplitPixels - 1) / kSplitPixels);
+            int splits;
+            long long kchunk;
+            wgrad_splits(nn, c, Pc, splits, kchunk);
             WgradOp wg;
             wg.g = make_geo(n, X.h, X.w, Pc);
             wg.fk = FastDiv((unsigned)c.cinp);
@@ -1114,11 +1289,10 @@ lbm_status backward(lbm_nn* nn, int n, float* loss) {
             wg.part = nn->part;
             wg.cin = c.cinp;
             wg.cout = c.coutp;
-            if ((e = launch_gemm(wg, kSplitPixels, splits, nn->gemm_err, s)) != cudaSuccess) break;
+            if ((e = launch_gemm(wg, kchunk, splits, nn->gemm_err, s)) != cudaSuccess) break;
             const long long nw = (long long)conv_wsize(c);
-            split_sum_kernel<<<grid_of(nw), kThreads, 0, s>>>(nn->part, c.gw, splits, nw);
-            if ((e = cudaGetLastError()) != cudaSuccess) break;
-            bias_grad_kernel<<<c.coutp, kThreads, 0, s>>>(gpre, c.gb, Pc, c.coutp);
+            split_sum_kernel<<<grid_of(nw + c.coutp), kThreads, 0, s>>>(
+                nn->part, c.gw, splits, nw, nn->bpart, c.gb, bb, c.coutp);
             if ((e = cudaGetLastError()) != cudaSuccess) break;
             nn->launches += 3;
             if (c.in != nn->x_id) {
@@ -1136,15 +1310,19 @@ lbm_status backward(lbm_nn* nn, int n, float* loss) {
         } else if (op.k == lbm_nn::POOL) {
             const lbm_nn::Tensor& X = nn->t[op.a];
             // the skip addition of the decoder has set the gradient of op.a
-            pool_back_kernel<<<grid_of(pixels(nn, op.a, n) * X.cp), kThreads, 0, s>>>(
-                G[op.out], G[op.a], n, X.h, X.w, X.cp, 1);
-            e = cudaGetLastError();
+            e = by_octets(nn, op.a, n, [&](int i, unsigned t) {
+                pool_back_kernel<<<grid_of(t), kThreads, 0, s>>>(
+                    instance(nn, op.out, G[op.out], i), instance(nn, op.a, G[op.a], i), t,
+                    FastDiv(X.cp / 8), FastDiv(X.w), FastDiv(X.h));
+            });
             ++nn->launches;
         } else if (op.k == lbm_nn::UP) {
             const lbm_nn::Tensor& X = nn->t[op.a];
-            up_back_kernel<<<grid_of(pixels(nn, op.a, n) * X.cp), kThreads, 0, s>>>(
-                G[op.out], G[op.a], n, X.h, X.w, X.cp);
-            e = cudaGetLastError();
+            e = by_octets(nn, op.a, n, [&](int i, unsigned t) {
+                up_back_kernel<<<grid_of(t), kThreads, 0, s>>>(
+                    instance(nn, op.out, G[op.out], i), instance(nn, op.a, G[op.a], i), t,
+                    FastDiv(X.cp / 8), FastDiv(X.w), FastDiv(X.h));
+            });
             ++nn->launches;
         } else {
             // an addition passes its gradient to both inputs
@@ -1239,11 +1417,10 @@ lbm_status lbm_nn_create(int levels, const int* channels, int max_batch, int hei
         }                                                                       \
     } while (0)
     // parameters: 8 FP32 arrays per convolution (w, b, gw, gb, mw, vw, mb, vb)
-    size_t pf = 0, wb = 0, maxw = 0;
+    size_t pf = 0, wb = 0;
     for (auto& c : nn->conv) {
         pf += 4 * (conv_wsize(c) + c.coutp);
         wb += 2 * conv_wsize(c);
-        maxw = conv_wsize(c) > maxw ? conv_wsize(c) : maxw;
     }
     nn->pfloats = pf;
     NCKC(lbm::dev_alloc(&nn->pbuf, pf * sizeof(float)), "cudaMalloc(parameters)");
@@ -1287,9 +1464,31 @@ lbm_status lbm_nn_create(int levels, const int* channels, int max_batch, int hei
     }
     NCKC(lbm::dev_alloc(&nn->scratch, maxt * sizeof(bf16)), "cudaMalloc(scratch)");
     const long long Pmax = (long long)nn->nb * nn->H * nn->W;
-    const long long splits = (Pmax + kSplitPixels - 1) / kSplitPixels;
-    nn->part_floats = (size_t)splits * maxw;
-    NCKC(lbm::dev_alloc(&nn->part, nn->part_floats * sizeof(float)), "cudaMalloc(partials)");
+    int dev = 0;
+    NCKC(cudaGetDevice(&dev), "cudaGetDevice");
+    NCKC(cudaDeviceGetAttribute(&nn->sms, cudaDevAttrMultiProcessorCount, dev),
+         "cudaDeviceGetAttribute");
+    // weight-gradient partials: the most of any convolution and batch size
+    // (the splits grow with the pixels, up to two CTAs per SM)
+    size_t pfl = 0, maxc = 0;
+    for (auto& c : nn->conv) {
+        const long long tiles = ((9LL * c.cinp + UM - 1) / UM) * ((c.coutp + 255) / 256);
+        const long long most = (2LL * nn->sms + tiles - 1) / tiles;
+        const long long px = (pixels(nn, c.in, nn->nb) + 255) / 256;
+        const size_t need = (size_t)(most < px ? most : px) * conv_wsize(c);
+        pfl = need > pfl ? need : pfl;
+        maxc = (size_t)c.coutp > maxc ? (size_t)c.coutp : maxc;
+    }
+    NCKC(lbm::dev_alloc(&nn->part, pfl * sizeof(float)), "cudaMalloc(partials)");
+    size_t runs = 1;  // of by_octets
+    for (auto& T : nn->t) {
+        const size_t r = (size_t)nn->nb * T.h * T.w * (T.cp / 8) / (1u << 30) + 1;
+        runs = r > runs ? r : runs;
+    }
+    NCKC(lbm::dev_alloc(&nn->bpart, runs * kBiasBlocks * maxc * sizeof(float)),
+         "cudaMalloc(partials)");
+    NCKC(lbm::dev_alloc(&nn->flat, lbm_nn_param_count(nn) * sizeof(float)),
+         "cudaMalloc(parameter vector)");
     NCKC(lbm::dev_alloc(&nn->dpart, 1025 * sizeof(double)), "cudaMalloc(loss)");
     NCKC(lbm::dev_alloc(&nn->xin, Pmax * 4 * sizeof(float)), "cudaMalloc(inputs)");
     NCKC(lbm::dev_alloc(&nn->tgt, Pmax * 3 * sizeof(float)), "cudaMalloc(targets)");
@@ -1297,7 +1496,8 @@ lbm_status lbm_nn_create(int levels, const int* channels, int max_batch, int hei
     NCKC(lbm::dev_alloc(&nn->yout, Pmax * 3 * sizeof(float)), "cudaMalloc(outputs)");
     NCKC(lbm::dev_alloc(&nn->gout, Pmax * 3 * sizeof(float)), "cudaMalloc(output gradient)");
     NCKC(lbm::dev_alloc(&nn->tmp3, Pmax * 3 * sizeof(float)), "cudaMalloc(output stage)");
-    NCKC(lbm::dev_alloc(&nn->ssum, (size_t)nn->nb * 3 * sizeof(double)), "cudaMalloc(output sums)");
+    NCKC(lbm::dev_alloc(&nn->ssum, (size_t)nn->nb * kStaggerParts * 3 * sizeof(double)),
+         "cudaMalloc(output sums)");
     NCKC(lbm::dev_alloc(&nn->gemm_err, sizeof(int)), "cudaMalloc(error word)");
     NCKC(cudaMemsetAsync(nn->gemm_err, 0, sizeof(int), nn->stream), "cudaMemset");
 #undef NCKC
@@ -1324,6 +1524,8 @@ void lbm_nn_destroy(lbm_nn* nn) {
     cudaFree(nn->abuf);
     cudaFree(nn->scratch);
     cudaFree(nn->part);
+    cudaFree(nn->bpart);
+    cudaFree(nn->flat);
     cudaFree(nn->dpart);
     cudaFree(nn->xin);
     cudaFree(nn->tgt);
@@ -1346,46 +1548,30 @@ size_t lbm_nn_param_count(const lbm_nn* nn) {
 }
 
 // Host parameter vector (dy, dx, cin, cout per convolution, then biases) <->
-// device masters [coutp][tap][cinp].
+// device masters [coutp][tap][cinp]: reordered on the GPU, one copy.  (The
+// padding of the device arrays is zero from creation and stays so.)
 static lbm_status transfer_params(lbm_nn* nn, float* host, bool to_device, bool grads) {
+    const size_t bytes = lbm_nn_param_count(nn) * sizeof(float);
+    if (to_device)
+        NCK(nn, cudaMemcpyAsync(nn->flat, host, bytes, cudaMemcpyHostToDevice, nn->stream),
+            "cudaMemcpyAsync(H2D)");
+    float* q = nn->flat;
     for (auto& c : nn->conv) {
-        const size_t w = conv_wsize(c);
-        std::vector<float> dev(w + c.coutp, 0.0f);
-        float* dw = grads ? c.gw : c.wm;
-        float* db = grads ? c.gb : c.bm;
-        if (!to_device) {
-            NCK(nn, cudaMemcpyAsync(dev.data(), dw, w * sizeof(float), cudaMemcpyDeviceToHost,
-                                    nn->stream),
-                "cudaMemcpyAsync(D2H)");
-            NCK(nn, cudaMemcpyAsync(dev.data() + w, db, c.coutp * sizeof(float),
-                                    cudaMemcpyDeviceToHost, nn->stream),
-                "cudaMemcpyAsync(D2H)");
-            NCK(nn, cudaStreamSynchronize(nn->stream), "cudaStreamSynchronize");
-        }
-        for (int tap = 0; tap < 9; ++tap)
-            for (int ci = 0; ci < c.cin; ++ci)
-                for (int co = 0; co < c.cout; ++co) {
-                    float& h = host[((size_t)tap * c.cin + ci) * c.cout + co];
-                    float& d = dev[((size_t)co * 9 + tap) * c.cinp + ci];
-                    if (to_device) d = h;
-                    else h = d;
-                }
-        host += 9ull * c.cin * c.cout;
-        for (int co = 0; co < c.cout; ++co) {
-            if (to_device) dev[w + co] = host[co];
-            else host[co] = dev[w + co];
-        }
-        host += c.cout;
-        if (to_device) {
-            NCK(nn, cudaMemcpyAsync(dw, dev.data(), w * sizeof(float), cudaMemcpyHostToDevice,
-                                    nn->stream),
-                "cudaMemcpyAsync(H2D)");
-            NCK(nn, cudaMemcpyAsync(db, dev.data() + w, c.coutp * sizeof(float),
-                                    cudaMemcpyHostToDevice, nn->stream),
-                "cudaMemcpyAsync(H2D)");
-            NCK(nn, cudaStreamSynchronize(nn->stream), "cudaStreamSynchronize");
-        }
+        float* w = grads ? c.gw : c.wm;
+        float* b = grads ? c.gb : c.bm;
+        const dim3 g((c.cout + 31) / 32, (c.cin + 31) / 32, 9);
+        if (to_device)
+            param_order_kernel<false><<<g, kThreads, 0, nn->stream>>>(q, w, b, c.cin, c.cout, c.cinp);
+        else
+            param_order_kernel<true><<<g, kThreads, 0, nn->stream>>>(q, w, b, c.cin, c.cout, c.cinp);
+        NCK(nn, cudaGetLastError(), "parameter order");
+        ++nn->launches;
+        q += 9ull * c.cin * c.cout + c.cout;
     }
+    if (!to_device)
+        NCK(nn, cudaMemcpyAsync(host, nn->flat, bytes, cudaMemcpyDeviceToHost, nn->stream),
+            "cudaMemcpyAsync(D2H)");
+    NCK(nn, cudaStreamSynchronize(nn->stream), "cudaStreamSynchronize");
     return LBM_OK;
 }
 
@@ -1466,9 +1652,10 @@ lbm_status lbm_nn_prolong(lbm_nn* nn, const float* y, int n, int factor, const u
     NCK(nn, cudaGetLastError(), "prolongation");
     out_smooth_kernel<false, false><<<grid_of(P), kThreads, 0, s>>>(f0, 3, fl, f1, 3, n, H, W);
     NCK(nn, cudaGetLastError(), "output smoothing (fine)");
-    stagger_sum_kernel<<<n, kThreads, 0, s>>>(f1, fl, nn->ssum, H, W);
+    const dim3 parts(kStaggerParts, n);
+    stagger_sum_kernel<<<parts, kThreads, 0, s>>>(f1, fl, nn->ssum, H, W);
     NCK(nn, cudaGetLastError(), "staggered sums (fine)");
-    stagger_apply_kernel<<<grid_of(P), kThreads, 0, s>>>(f1, fl, nn->ssum, f0, P, H, W);
+    stagger_apply_kernel<<<parts, kThreads, 0, s>>>(f1, fl, nn->ssum, f0, H, W);
     NCK(nn, cudaGetLastError(), "staggered projection (fine)");
     nn->launches += 4;
     NCK(nn, cudaMemcpyAsync(out, f0, P * 3 * sizeof(float), cudaMemcpyDeviceToHost, s),
