@@ -858,22 +858,35 @@ __global__ void __launch_bounds__(kThreads) sum_kernel(const double* part, int n
     if (threadIdx.x == 0) *out = b;
 }
 
-// dW = sum over the splits in order, and gb = sum over the bias partials in
-// order (in the threads after the weights').
+// dW = sum over the splits, and gb = sum over the bias partials, in a fixed
+// order: a block takes 32 values, each by eight threads whose sums (terms z =
+// k, k + 8, ...) are added in order.  (One thread a value was a chain of 100 to
+// 300 dependent rounds: 25 us a convolution on average.)
 __global__ void __launch_bounds__(kThreads)
 split_sum_kernel(const float* part, float* gw, int splits, long long n, const float* bpart,
                  float* gb, int bparts, int cout) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n + cout;
-         i += (long long)gridDim.x * blockDim.x) {
-        const bool w = i < n;
-        const float* q = w ? part + i : bpart + (i - n);
-        const long long step = w ? n : cout;
+    __shared__ float sh[8][33];
+    const int x = threadIdx.x & 31, k = threadIdx.x >> 5;
+    // blocks of weights, then blocks of biases
+    const long long wblocks = (n + 31) / 32, blocks = wblocks + (cout + 31) / 32;
+    for (long long b = blockIdx.x; b < blocks; b += gridDim.x) {
+        const bool w = b < wblocks;
+        const long long i = (w ? b : b - wblocks) * 32 + x, size = w ? n : cout;
         const int terms = w ? splits : bparts;
         float s = 0.0f;
+        if (i < size) {
+            const float* q = (w ? part : bpart) + i;
 #pragma unroll 8
-        for (int z = 0; z < terms; ++z) s += q[z * step];
-        if (w) gw[i] = s;
-        else gb[i - n] = s;
+            for (int z = k; z < terms; z += 8) s += q[z * size];
+        }
+        sh[k][x] = s;
+        __syncthreads();
+        if (k == 0 && i < size) {
+#pragma unroll
+            for (int j = 1; j < 8; ++j) s += sh[j][x];
+            (w ? gw : gb)[i] = s;
+        }
+        __syncthreads();
     }
 }
 
@@ -1291,7 +1304,7 @@ lbm_status backward(lbm_nn* nn, int n, float* loss) {
             wg.cout = c.coutp;
             if ((e = launch_gemm(wg, kchunk, splits, nn->gemm_err, s)) != cudaSuccess) break;
             const long long nw = (long long)conv_wsize(c);
-            split_sum_kernel<<<grid_of(nw + c.coutp), kThreads, 0, s>>>(
+            split_sum_kernel<<<grid_of((nw + c.coutp + 64) * 8), kThreads, 0, s>>>(
                 nn->part, c.gw, splits, nw, nn->bpart, c.gb, bb, c.coutp);
             if ((e = cudaGetLastError()) != cudaSuccess) break;
             nn->launches += 3;

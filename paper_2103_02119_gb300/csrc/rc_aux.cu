@@ -81,7 +81,7 @@ struct Tiles {
 // and divisions in FP64: lbm_stress 558 against 2085 us, lbm_diagnostics after a
 // step 380 against 1260 us, lbm_get_f 84 against 146 us, lbm_set_f 91 against
 // 143 us, lbm_moments 51 against 68 us; the residual check of a 96-lattice batch
-// 0.75 against 2.56 ms.
+// 0.86 against 2.56 ms.
 
 // float -> double, exact, on the integer pipe, without a branch (a conversion
 // instruction under a predicate takes its place in the FP64 pipe even where
