@@ -34,13 +34,18 @@ __device__ __forceinline__ long long target(const AuxParams& p, int x, int y, in
 struct Feq32 {
     float cs2, a, iah2, rho0;
     __device__ __forceinline__ float operator()(int i, float dr, float u, float v) const {
+        // The fused multiply-adds are written out: a state that amplifies its
+        // last bits (an unstable flow) has to be the same whatever the code
+        // around this expression lets the compiler contract.
         const int sx = ex(i), sy = ey(i);
         const float X0 = sx == 0 ? 1.0f - cs2 : 0.5f * cs2;
-        const float dX = sx == 0 ? -u * u : 0.5f * (u * u + (float)sx * u);
-        const float Y0 = sy == 0 ? 1.0f - 2.0f * iah2 * cs2 : iah2 * cs2;
-        const float dY = sy == 0 ? -2.0f * iah2 * v * v : iah2 * (v * v + (float)sy * a * v);
-        const float X = X0 + dX, Y = Y0 + dY;
-        return dr * X * Y + rho0 * (dX * Y + X0 * dY);
+        const float dX = sx == 0 ? __fmul_rn(-u, u) : 0.5f * __fmaf_rn(u, u, (float)sx * u);
+        const float Y0 = sy == 0 ? __fmaf_rn(-2.0f * iah2, cs2, 1.0f) : __fmul_rn(iah2, cs2);
+        const float dY = sy == 0 ? __fmul_rn(-2.0f * iah2 * v, v)
+                                 : __fmul_rn(iah2, __fmaf_rn(v, v, __fmul_rn((float)sy * a, v)));
+        const float X = __fadd_rn(X0, dX), Y = __fadd_rn(Y0, dY);
+        const float d = __fmaf_rn(X0, dY, __fmul_rn(dX, Y));
+        return __fmaf_rn(__fmul_rn(dr, X), Y, __fmul_rn(rho0, d));
     }
 };
 
