@@ -136,7 +136,7 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
  * launch per step; runs of 50 steps replay a CUDA graph the handle captures
  * once per starting buffer (on a stream of its own; lbm_set_force drops
  * it).  Small lattices run many steps per launch (lbm_set_small_path), large
- * FP32 ones (from 200,000 cells) two steps per launch but for the last one or
+ * FP32 ones (from 80,000 cells) two steps per launch but for the last one or
  * two of a call; the states are bit for bit the same.  Asynchronous: the
  * return value reports launch errors only. */
 lbm_status lbm_step(lbm_handle* h, int64_t nsteps);
@@ -319,7 +319,9 @@ const char* lbm_last_error(const lbm_handle* h);
  * graph.  When every active lattice has at most 4096 cells (and they fit the
  * constant-memory tables), each steps on a thread-block cluster of its own
  * that keeps its state in shared memory, up to 1024 steps per launch and
- * group; the launch shape does not matter then.  Lattices can be retired (made inactive) and brought back; an inactive lattice keeps
+ * group.  Else, when every one collides and has at least 64 x 16 cells, a
+ * launch per group takes two steps, but for the last one or two of a call.  The
+ * launch shape does not matter to either.  Lattices can be retired (made inactive) and brought back; an inactive lattice keeps
  * its state and is not stepped.  Conventions as for lbm_handle; work is
  * issued on the stream given to lbm_batch_create.
  * ------------------------------------------------------------------------ */
@@ -384,8 +386,8 @@ int lbm_batch_is_active(const lbm_batch* b, int k);
 
 /* Launch shape of the batch step: threads per block along x (32, 64 or 128;
  * a block covers 2 x block_x columns) and target rows per band (1 .. 65536;
- * lattice k gets max(1, round(ny_k / rows_per_band)) bands).  The shape
- * changes the schedule only, never the results.  Default 32, 16. */
+ * lattice k gets max(1, round(ny_k / rows_per_band)) bands), for single
+ * steps.  The shape changes the schedule only, never the results.  Default 32, 16. */
 lbm_status lbm_batch_set_shape(lbm_batch* b, int block_x, int rows_per_band);
 lbm_status lbm_batch_get_shape(const lbm_batch* b, int* block_x, int* rows_per_band);
 
@@ -407,7 +409,7 @@ int lbm_batch_table_groups(lbm_batch* b);
 lbm_status lbm_batch_set_wait_limit(lbm_batch* b, int64_t polls);
 
 /* Autotuner: times trial_steps (>= 1) steps of the active lattices at each
- * block_x in {32, 64, 128} and rows_per_band in {1, 2, 4, 8, 16, 32, 64} (one warm-up
+ * block_x in {32, 64, 128} and rows_per_band in {1, 2, 4, 8, 16, 32, 64} (single steps, one warm-up
  * step each, CUDA events on the batch's stream), keeps the fastest shape and
  * returns it (outputs nullable).  The trial steps are real steps of the
  * active lattices (21 (trial_steps + 1) in all): the shape does not change
@@ -427,7 +429,7 @@ lbm_status lbm_batch_diagnostics(lbm_batch* b, int k, double out[LBM_DIAG_COUNT]
 int64_t lbm_batch_step_count(const lbm_batch* b, int k);
 
 /* Batch step kernel launches issued so far: one per group of lattices and
- * step, or (active lattices of at most 4096 cells) run of up to 1024 steps. */
+ * step, or two steps, or (active lattices of at most 4096 cells) run of up to 1024 steps. */
 int64_t lbm_batch_launch_count(const lbm_batch* b);
 
 /* Message of the last error on b (or of the last failed lbm_batch_create

@@ -19,6 +19,7 @@
 // The block's work is step_block's, so a lattice goes through the same states
 // bit for bit as with the single-lattice kernel.
 #pragma once
+#include "chain_step.cuh"
 #include "small_step.cuh"
 #include "step_block.cuh"
 
@@ -39,6 +40,8 @@ __constant__ BatchTableLattice c_table[kBatchTableCap];
 // number of work items
 __constant__ int c_table_begin[kBatchTableCap + 1];
 __constant__ int c_table_n;
+// first chain of each lattice for two steps at once; the last: their number
+__constant__ int c_chain_begin[kBatchTableCap + 1];
 
 template <int BXT, int SCH>
 __global__ void __launch_bounds__(BXT, step_min_blocks<float>(BXT))
@@ -86,6 +89,58 @@ cudaError_t launch_table_sch(int parity, int bx, int grid, cudaStream_t s) {
     case 128: return launch_table_bx<128, SCH>(parity, grid, s);
     default: return cudaErrorInvalidValue;
     }
+}
+
+// Two steps of every lattice: a chain of two warps (chain_step.cuh) per strip
+// and band of a lattice, one block each, so that chains of lattices of every
+// size balance as the hardware hands out the blocks.
+// Registers bound it (128, as in the single-lattice kernel, whose constants are
+// operands from the constant bank; here an instruction loads each).  What kept
+// it from spilling, us a step of 96 lattices of 64-1024 cells a side (257 with
+// the row-band kernel): nothing 251, 12 warps per SM in place of 16 224,
+// collision constants reloaded every row (the entry is hidden from the
+// compiler, which else keeps them in registers) and plane offsets of 32 bits
+// 190, ring slots derived from one, row counters and link bits of two rows
+// joined 136.
+template <int SCH>
+__global__ void __launch_bounds__(64, 8) batch_chain_kernel(int parity) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int w = blockIdx.x;
+    int lo = 0, hi = c_table_n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (c_chain_begin[mid] <= w) lo = mid;
+        else hi = mid - 1;
+    }
+    const BatchTableLattice& L = c_table[lo];
+    const int local = w - c_chain_begin[lo];
+    const int strips = (L.kp.nx + kChainColumns - 1) / kChainColumns;
+    const int nbands = (c_chain_begin[lo + 1] - c_chain_begin[lo]) / strips;
+    const int band = local / strips, strip = local % strips;
+    const int y0 = (int)((long long)band * L.kp.ny / nbands);
+    const int y1 = (int)((long long)(band + 1) * L.kp.ny / nbands);
+    chain_march<SCH, true, 2, unsigned>(
+        L.f[parity], L.f[parity ^ 1], L.kp, strip, y0, y1, threadIdx.x >> 5,
+        reinterpret_cast<float2*>(smem), [&] {
+            int k = lo;
+            asm volatile("" : "+r"(k));
+            return to_lanes(c_table[k].kp.cc);
+        });
+}
+
+template <int SCH>
+cudaError_t launch_chain_sch(int parity, int chains, cudaStream_t s) {
+    constexpr size_t smem = chain_smem_bytes<2>();
+    static bool configured = false;
+    if (!configured) {
+        cudaError_t e = cudaFuncSetAttribute(batch_chain_kernel<SCH>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    batch_chain_kernel<SCH><<<chains, 64, smem, s>>>(parity);
+    return cudaGetLastError();
 }
 
 // Batches of small lattices: a cluster per lattice runs nsteps steps with the
@@ -140,12 +195,16 @@ int table_occ_bx() {
 }  // namespace
 
 cudaError_t LBM_SLOT_NAME(batch_table_upload_)(const BatchTableLattice* lat, const int* begin,
-                                               int n, cudaStream_t s) {
+                                               const int* chain_begin, int n,
+                                               cudaStream_t s) {
     if (n < 1 || n > kBatchTableCap) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemcpyToSymbolAsync(c_table, lat, sizeof(BatchTableLattice) * (size_t)n, 0,
                                             cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
     e = cudaMemcpyToSymbolAsync(c_table_begin, begin, sizeof(int) * (size_t)(n + 1), 0,
+                                cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyToSymbolAsync(c_chain_begin, chain_begin, sizeof(int) * (size_t)(n + 1), 0,
                                 cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return e;
     return cudaMemcpyToSymbolAsync(c_table_n, &n, sizeof(int), 0, cudaMemcpyHostToDevice, s);
@@ -154,6 +213,10 @@ cudaError_t LBM_SLOT_NAME(batch_table_upload_)(const BatchTableLattice* lat, con
 cudaError_t LBM_SLOT_NAME(batch_table_launch_)(int parity, int bx, int grid, int raw,
                                                cudaStream_t s) {
     return raw ? launch_table_sch<1>(parity, bx, grid, s) : launch_table_sch<0>(parity, bx, grid, s);
+}
+
+cudaError_t LBM_SLOT_NAME(batch_chain_launch_)(int parity, int chains, int raw, cudaStream_t s) {
+    return raw ? launch_chain_sch<1>(parity, chains, s) : launch_chain_sch<0>(parity, chains, s);
 }
 
 cudaError_t LBM_SLOT_NAME(batch_small_launch_)(const SmallBatch& b, int n, int from, int nsteps,

@@ -24,23 +24,30 @@
 // (two per step and end) are computed by both neighbours: 56 of 64 columns are
 // stored.  The bounced-back population of a blocked link is the cell's own
 // opposite one, in row q - 1 of the ring; rows without blocked links (most)
-// skip the selection.
+// skip the selection.  The link bits of a turn's two rows come with loads a
+// turn ahead, which nothing touches meanwhile: an instruction between the load
+// and the row (a conversion, a select, the move of a register rotation) waits
+// for memory, also where it is predicated off.
 //
 // What bounds it: the FP32 pipe (55 to 60 % busy) with four warps a scheduler
 // to hide the latency of a row; 128 registers and 23 KB a chain let no more in.
 // Measured, MLUPS, against the row-band kernel (100 steps): periodic
-// 2048 x 8192 101k / 75.6k and 2048 x 1024 74k / 54k, cavity 2048 x 8192 98.6k /
-// 80.2k, raw-moment scheme 102k / 81.0k, channel 1543 x 3001 with obstacles 64k /
-// 48k.  Not kept (2048 x 8192, at the time 96.2k): one step per launch (75k) or
-// three (82k: halo columns); populations shifted by the copies, 4 bytes at a
-// time (80k: shared-memory bandwidth); previous rows carried in registers
-// (86.6k); two rows ahead instead of one (92.5k: the L1 cache gets what shared
-// memory leaves); 20 warps per SM (58k: spills); two or four chains per block
-// (79k, 70k); a barrier every row (89k).
+// 2048 x 8192 105k / 75.6k and 2048 x 1024 75.5k / 52.8k, cavity 2048 x 8192
+// 103k / 80.3k, raw-moment scheme 106k / 81.0k, cavities with obstacles
+// 2048 x 8192 101k / 78.1k and 1543 x 3001 86k / 58.8k.  Not kept (2048 x 8192):
+// one step per launch (75k) or three (82k: halo columns); populations shifted
+// by the copies, 4 bytes at a time (80k: shared-memory bandwidth); previous
+// rows carried in registers (86.6k); two rows ahead instead of one (92.5k: the
+// L1 cache gets what shared memory leaves); 20 warps per SM (58k: spills); two
+// or four chains per block (79k, 70k); a barrier every row (89k); the strips at
+// the lattice's sides read cell by cell (98.6k; with obstacles 84k: now only
+// where an odd width wraps around); tall bands first, then short ones for the
+// last quarter (91k).
 //
 // The arithmetic is that of step_block in the same order, so a lattice goes
 // through the same states bit for bit on either path.
 #pragma once
+#include <type_traits>
 #include "lbm_device.cuh"
 #include "lbm_launch.h"
 
@@ -79,11 +86,13 @@ __host__ __device__ constexpr size_t chain_smem_bytes() {  // of one chain
 }
 
 // K steps of rows y0 .. y1 - 1 and the strip's columns by the chain's warp
-// `stage`; sm: chain_smem_bytes<K>().  nx >= 64, ny >= 16, 4 plane < 2^32.
-template <int SCH, bool MASK, int K, typename PT>
-__device__ __forceinline__ void chain_march(const float* __restrict__ fin, float* __restrict__ fout,
+// `stage`; sm: chain_smem_bytes<K>(); constants(): the collision's.  nx >= 64,
+// ny >= 16, 4 plane < 2^32.  PB: the type of a plane's byte offset, unsigned
+// where 36 plane < 2^32 (the tight variant, fewer registers).
+template <int SCH, bool MASK, int K, bool PAIRS, typename PB, typename PT, typename CC>
+__device__ __forceinline__ void march_strip(const float* __restrict__ fin, float* __restrict__ fout,
                                             const PT& p, int strip, int y0, int y1, int stage,
-                                            float2* sm) {
+                                            float2* sm, CC constants) {
     constexpr int kHaloC = 2 * K, kValid = kStrip - 2 * kHaloC;
     const int lane = threadIdx.x & 31;
     const int nx = p.nx, ny = p.ny;
@@ -91,14 +100,14 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
     const int c0 = xs + 2 * lane;       // logical column of the lane's first cell
     auto col = [&](int c) {             // where a logical column is stored
         if (p.px) return c < 0 ? c + nx : c >= nx ? c - nx : c;
-        return min(max(c, 0), nx - 1);
+        // beyond a wall: any column, which no link reads
+        return min(max(c, 0), p.pitch - 2);
     };
     auto row_of = [&](int r) {
         if (p.py) return r < 0 ? r + ny : r >= ny ? r - ny : r;
         return min(max(r, 0), ny - 1);
     };
-    const int ca = col(c0), cb = col(c0 + 1);
-    const bool plain = xs >= 0 && xs + kStrip <= nx;
+    const int ca = col(c0), cb = PAIRS ? ca + 1 : col(c0 + 1);
     const bool stores = lane >= kHaloC / 2 && lane < 32 - kHaloC / 2 && c0 < nx;
     // walls along x, as link bits of the two cells
     unsigned xb = 0;
@@ -112,22 +121,34 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
     const bool xmoves = p.wall_odd[0][0] != 0.0f || p.wall_odd[0][1] != 0.0f ||
                         p.wall_odd[0][2] != 0.0f || p.wall_odd[1][0] != 0.0f ||
                         p.wall_odd[1][1] != 0.0f || p.wall_odd[1][2] != 0.0f;
-    auto bits_of = [&](int r) -> unsigned {
+    // Link bits of the two rows of a turn, the first in the low half: with a
+    // mask the loads of the next turn's rows are in flight meanwhile (put
+    // together at its start: anything done to them earlier waits for them).
+    unsigned in[MASK ? (PAIRS ? 2 : 4) : 1];
+    auto fetch_bits = [&](int r) {
         if constexpr (MASK) {
-            const uint8_t* m = p.lmask + (unsigned)row_of(r) * (unsigned)p.pitch;
-            unsigned short a, b;
-            if (plain) {
-                asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(a) : "l"(m + (unsigned)c0));
-                return a;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const uint8_t* m = p.lmask + (unsigned)row_of(r + k) * (unsigned)p.pitch;
+                if constexpr (PAIRS) {
+                    asm volatile("ld.global.nc.u16 %0, [%1];" : "=r"(in[k]) : "l"(m + (unsigned)ca));
+                } else {
+                    asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(in[2 * k]) : "l"(m + (unsigned)ca));
+                    asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(in[2 * k + 1]) : "l"(m + (unsigned)cb));
+                }
             }
-            asm volatile("ld.global.nc.u8 %0, [%1];" : "=h"(a) : "l"(m + (unsigned)ca));
-            asm volatile("ld.global.nc.u8 %0, [%1];" : "=h"(b) : "l"(m + (unsigned)cb));
-            return (unsigned)a | ((unsigned)b << 8);
-        } else {
-            unsigned y = 0;
-            if (!p.py) y = (r == 0 ? 0x3232u : 0u) | (r == ny - 1 ? 0xC8C8u : 0u);
-            return xb | y;
         }
+    };
+    auto bits_of = [&]() -> unsigned {
+        if constexpr (MASK && PAIRS) return in[0] | in[1] << 16;
+        else if constexpr (MASK) return in[0] | in[1] << 8 | in[2] << 16 | in[3] << 24;
+        else return 0;
+    };
+    // without a mask: of one row, made where they are used
+    auto wall_bits = [&](int r) -> unsigned {
+        unsigned b = xb;
+        if (!p.py) b |= (r == 0 ? 0x3232u : 0u) | (r == ny - 1 ? 0xC8C8u : 0u);
+        return b;
     };
     auto any_of = [&](unsigned b, int r) -> bool {
         // a fluid cell with blocked links (0xFF: solid)
@@ -137,7 +158,11 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
     };
     // byte offsets of 32 bits from the planes' (uniform) addresses
     const char* fbase = reinterpret_cast<const char*>(fin);
-    const long long pb = p.plane * 4;
+    const PB pb = (PB)(p.plane * 4);
+    auto at = [&](auto* base, int i, unsigned o) {  // byte o of plane i
+        if constexpr (sizeof(PB) == 4) return base + (o + (unsigned)i * pb);
+        else return base + i * pb + o;
+    };
     const unsigned dst0 = (unsigned)__cvta_generic_to_shared(sm) + 8u * lane;
     bool bad = false;  // checked build: a failed bounds check (the access is skipped)
     auto issue = [&](int r, int s) {
@@ -145,21 +170,21 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
         const unsigned row = (unsigned)row_of(r) * (unsigned)p.rstride;
         if constexpr (kChecked) {
             if (!(idx_ok(row_of(r), ny) && idx_ok(s, kFetchSlots) && idx_ok(ca, p.rstride) &&
-                  idx_ok(cb, p.rstride) && (!plain || (ca == c0 && cb == c0 + 1)))) {
+                  idx_ok(cb, p.rstride) && (!PAIRS || (ca & 1) == 0))) {
                 bad = true;
                 return;
             }
         }
-        if (plain) {
-            const unsigned o = (row + (unsigned)c0) * 4u;
+        if constexpr (PAIRS) {
+            const unsigned o = (row + (unsigned)ca) * 4u;
 #pragma unroll
-            for (int i = 0; i < 9; ++i) fetch8(dst + i * 256, (fbase + i * pb) + o);
+            for (int i = 0; i < 9; ++i) fetch8(dst + i * 256, at(fbase, i, o));
         } else {
             const unsigned oa = (row + (unsigned)ca) * 4u, ob = (row + (unsigned)cb) * 4u;
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-                fetch4(dst + i * 256, (fbase + i * pb) + oa);
-                fetch4(dst + i * 256 + 4, (fbase + i * pb) + ob);
+                fetch4(dst + i * 256, at(fbase, i, oa));
+                fetch4(dst + i * 256 + 4, at(fbase, i, ob));
             }
         }
     };
@@ -167,12 +192,12 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
     // rows of this stage: first .. last arrive (and one more where their number
     // is odd), two a turn; a stage starts three turns after the one before it
     const int first = y0 - 2 * (K - stage), last = y1 - 1 + 2 * (K - stage);
-    const int turns = (last - first + 2) / 2;
+    const int stop = first + (last - first + 2) / 2 * 2;
     const float2 z = make_float2(0.0f, 0.0f);
     float2 G[9] = {z, z, z, z, z, z, z, z, z}, dS = z, dC = z;
-    unsigned b1 = 0, b2 = 0;
+    unsigned bt = 0, bp = 0;  // link bits of this turn's rows and of the previous turn's
     bool a1 = false, a2 = false;
-    unsigned nb = bits_of(first), nb2 = MASK ? bits_of(first + 1) : 0u;
+    fetch_bits(first);
     const int nslots = stage == 0 ? kFetchSlots : kHandSlots;
     // slots of rows q, q - 1, q - 2 of my ring, and of the row I write next
     int s0 = 0, s1 = nslots - 1, s2 = nslots - 2;
@@ -187,8 +212,10 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
     float2* hout = sm + (kFetchSlots + kHandSlots * stage) * kRowPairs + lane;
     if constexpr (K > 1)
         for (int w = 0; w < 3 * stage; ++w) __syncthreads();
-    int q = first;
-    for (int t = 0; t < turns; ++t) {
+    for (int q = first; q < stop;) {
+        bp = bt;
+        bt = bits_of();
+        fetch_bits(q + 2);
 #pragma unroll
         for (int k = 0; k < 2; ++k, ++q) {
             if (stage == 0) {
@@ -199,16 +226,17 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
                 asm volatile("cp.async.commit_group;" ::: "memory");
                 asm volatile("cp.async.wait_group %0;" ::"n"(kChainDepth) : "memory");
             }
+            if constexpr (sizeof(PB) == 4) {  // two registers fewer
+                s1 = s0 >= 1 ? s0 - 1 : s0 - 1 + nslots;
+                s2 = s0 >= 2 ? s0 - 2 : s0 - 2 + nslots;
+            }
             const float2 *r0 = mine + s0 * kRowPairs, *r1 = mine + s1 * kRowPairs,
                          *r2 = mine + s2 * kRowPairs;
-            const unsigned b0 = nb;
-            if constexpr (MASK) {  // a global read: two rows ahead
-                nb = nb2;
-                nb2 = bits_of(q + 2);
-            } else {
-                nb = bits_of(q + 1);
-            }
-            const bool a0 = any_of(b0, q);
+            // link bits of rows q - 1 and q - 2, from bit h1 and h2 on
+            const int h1 = MASK && !k ? 16 : 0, h2 = MASK && k ? 16 : 0;
+            const unsigned b1 = !MASK ? wall_bits(q - 1) : k ? bt : bp;
+            const unsigned b2 = !MASK ? wall_bits(q - 2) : bp;
+            const bool a0 = any_of(k ? bt >> 16 : bt & 0xFFFFu, q);
             // the pulled populations of row q - 1
             float2 g[9];
             g[0] = r1[0];
@@ -222,7 +250,7 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
             g[8] = from_west(r0[8 * 32]);
             if (a1) {  // bounced back: the cell's own opposite populations
 #pragma unroll
-                for (int i = 1; i < 9; ++i) g[i] = pick(b1, 1u << (i - 1), r1[opp(i) * 32], g[i]);
+                for (int i = 1; i < 9; ++i) g[i] = pick(b1, 1u << (i - 1 + h1), r1[opp(i) * 32], g[i]);
             }
             s2 = s1;
             s1 = s0;
@@ -235,15 +263,15 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
             {
                 float2 w = from_west(dC), e = from_east(dC), sd = dS, nn = dN;
                 if (a2) {
-                    w = pick(b2, 1u, dC, w);
-                    sd = pick(b2, 2u, dC, sd);
-                    e = pick(b2, 4u, dC, e);
-                    nn = pick(b2, 8u, dC, nn);
+                    w = pick(b2, 1u << h2, dC, w);
+                    sd = pick(b2, 2u << h2, dC, sd);
+                    e = pick(b2, 4u << h2, dC, e);
+                    nn = pick(b2, 8u << h2, dC, nn);
                 }
                 const float2 dxr = vmul(make_float2(0.5f, 0.5f), vsub(e, w));
                 const float2 dyr = vmul(make_float2(p.iah, p.iah), vsub(nn, sd));
-                const float2 rho = SCH == 1 ? collide_raw<float>(to_lanes(p.cc), G, dC, dxr, dyr)
-                                            : collide<float, SCH != 3>(to_lanes(p.cc), G, dC, dxr, dyr);
+                const float2 rho = SCH == 1 ? collide_raw<float>(constants(), G, dC, dxr, dyr)
+                                            : collide<float, SCH != 3>(constants(), G, dC, dxr, dyr);
                 if (p.moving && a2 && (xmoves || r == 0 || r == ny - 1)) {
                     float fa[9], fb[9];
 #pragma unroll
@@ -266,12 +294,13 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
 #pragma unroll
                     for (int i = 0; i < 9; ++i) o[i * 32] = G[i];
                 } else if (stores && r >= y0 && r < y1) {
-                    if (MASK && ((b2 & 0xFFu) == 0xFFu || (b2 >> 8) == 0xFFu)) {
+                    const unsigned lo = 0xFFu << h2, hi = 0xFF00u << h2;
+                    if (MASK && ((b2 & lo) == lo || (b2 & hi) == hi)) {
                         // a solid cell keeps its zeros
 #pragma unroll
                         for (int i = 0; i < 9; ++i) {
-                            if ((b2 & 0xFFu) == 0xFFu) G[i].x = 0.0f;
-                            if ((b2 >> 8) == 0xFFu) G[i].y = 0.0f;
+                            if ((b2 & lo) == lo) G[i].x = 0.0f;
+                            if ((b2 & hi) == hi) G[i].y = 0.0f;
                         }
                     }
                     const unsigned o = ((unsigned)r * (unsigned)p.rstride + (unsigned)c0) * 4u;
@@ -279,15 +308,13 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
                     else
 #pragma unroll
                     for (int i = 0; i < 9; ++i)
-                        *reinterpret_cast<float2*>((reinterpret_cast<char*>(fout) + i * pb) + o) = G[i];
+                        *reinterpret_cast<float2*>(at(reinterpret_cast<char*>(fout), i, o)) = G[i];
                 }
             }
 #pragma unroll
             for (int i = 0; i < 9; ++i) G[i] = g[i];
             dS = dC;
             dC = dN;
-            b2 = b1;
-            b1 = b0;
             a2 = a1;
             a1 = a0;
         }
@@ -296,6 +323,18 @@ __device__ __forceinline__ void chain_march(const float* __restrict__ fin, float
     if constexpr (K > 1)
         for (int w = stage; w < K - 1; ++w) __syncthreads();
     if (kChecked && bad) atomicOr(p.status, kStatusBounds);
+}
+
+// The strip's lanes read their two cells as an aligned pair, but where an odd
+// width wraps around.
+template <int SCH, bool MASK, int K, typename PB, typename PT, typename CC>
+__device__ __forceinline__ void chain_march(const float* fin, float* fout, const PT& p, int strip,
+                                            int y0, int y1, int stage, float2* sm, CC constants) {
+    const int xs = strip * (kStrip - 4 * K) - 2 * K;
+    if (!p.px || (p.nx & 1) == 0 || (xs >= 0 && xs + kStrip <= p.nx))
+        march_strip<SCH, MASK, K, true, PB>(fin, fout, p, strip, y0, y1, stage, sm, constants);
+    else
+        march_strip<SCH, MASK, K, false, PB>(fin, fout, p, strip, y0, y1, stage, sm, constants);
 }
 
 template <int SCH, bool MASK, int K>
@@ -308,8 +347,8 @@ chain_kernel(const float* __restrict__ fin, float* __restrict__ fout,
     const int y1 = (int)((long long)(band + 1) * p.ny / nbands);
     // the strips along the walls take longer: first in every band
     const int x = blockIdx.x, n = gridDim.x;
-    chain_march<SCH, MASK, K>(fin, fout, p, x == 0 ? n - 1 : x - 1, y0, y1, threadIdx.x >> 5,
-                              reinterpret_cast<float2*>(smem));
+    chain_march<SCH, MASK, K, long long>(fin, fout, p, x == 0 ? n - 1 : x - 1, y0, y1, threadIdx.x >> 5,
+                              reinterpret_cast<float2*>(smem), [&] { return to_lanes(p.cc); });
 }
 
 }  // namespace

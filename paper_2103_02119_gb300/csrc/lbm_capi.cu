@@ -590,16 +590,14 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
     h->nbands = nb;
     // Two steps per launch (chain_step.cuh) where that is faster than the
     // row-band kernel; us a step, two-step / row-band kernel:
-    //   periodic 400 x 300 7.3 / 8.3, 2048 x 1024 28 / 39, 2048 x 8192 166 / 222;
-    //   cavities 400 x 300 10.3 / 7.3, 512^2 12.2 / 16.1, 2048 x 8192 170 / 209,
-    //   200 x 6000 (two of four strips along a wall) 28.7 / 25.3;
-    //   cavities with obstacles 512^2 15.5 / 17.2, 1001 x 2003 40 / 34 (two
-    //   buffers that the L2 nearly holds, and a launch as long as the chains
-    //   along the obstacles), 1543 x 3001 75 / 81, 2048 x 8192 199 / 215.
-    if (!f64 && !kRowInterleaved && h->N >= 200000 && (p->periodic_x || p->nx > 280) &&
-        !(solid_mask && h->N >= 1150000 && h->N < 3000000))
-        h->chain_bands = lbm::chain2_bands(p->nx, p->ny, h->pitch,
-                                            solid_mask != nullptr, sms);
+    //   periodic 256^2 6.2 / 6.7, 400 x 300 6.3 / 8.2, 2048 x 1024 27.8 / 39.7,
+    //   2048 x 8192 160 / 222;
+    //   cavities 200^2 7.2 / 6.1, 300^2 7.2 / 7.2, 100 x 1000 7.4 / 16.4, 512^2
+    //   10.4 / 16.0, 200 x 6000 21.6 / 25.2, 2048 x 8192 162 / 209;
+    //   cavities with obstacles 256^2 7.2 / 6.7, 300^2 7.3 / 7.6, 1001 x 2003
+    //   27.8 / 33.8, 1543 x 3001 54 / 79, 2048 x 8192 165 / 215.
+    if (!f64 && !kRowInterleaved && h->N >= 80000)
+        h->chain_bands = lbm::chain2_bands(p->nx, p->ny, h->pitch, sms);
     // small lattices: all the steps of an lbm_step call in one launch of one
     // thread-block cluster, when the device can hold it
     if (h->N <= lbm::kSmallCells && !kRowInterleaved) {
@@ -1127,6 +1125,11 @@ struct lbm_batch {
     int ggrid[lbm::kBatchTables] = {};
     std::vector<lbm::BatchTableLattice> gtab[lbm::kBatchTables];
     std::vector<int> gbegin[lbm::kBatchTables];  // first work item of each, then the total
+    // two steps per launch where every active lattice can take them
+    // (chain_step.cuh): first chain of each lattice, then the total
+    bool chains = false;
+    bool tuning = false;             // the launch shapes are being timed: single steps
+    std::vector<int> gchain[lbm::kBatchTables];
     // cluster != 0: the groups' lattices are all small and step by clusters,
     // many steps per launch (small_step.cuh)
     lbm::SmallBatch small;
@@ -1269,6 +1272,73 @@ std::mutex g_table_mu;
 unsigned long long g_table_owner[64] = {};
 bool g_table_fresh[64] = {};
 
+// Two steps per launch (chain_step.cuh) where every active lattice can take
+// them: faster than the row-band kernel in its best shape from the smallest
+// batches on that clusters do not take.  us a step of lattices with obstacles,
+// two-step kernel / row-band kernel in the best of its shapes: 2 of 64-100
+// cells a side 8.5 / 10.3, 8 of 64-200 10.6 / 12.4, 24 of 64-300 18.3 / 34.2,
+// 96 of 64-1024 136 / 257.
+// The bands: every one marches ten rows more than it stores, and the launch
+// ends with the march of its last chains; so a lattice's bands are as tall as
+// the rows that are left for each chain in flight, within limits that a model
+// of the launch chooses (96 of 64-1024: 190 us a step against 210 with bands
+// of one height, when the kernel was slower by other causes).
+void plan_chains(lbm_batch* b) {
+    b->chains = b->ngroups > 0 && b->small.cluster == 0;
+    for (int g = 0; g < b->ngroups; ++g) {
+        b->gchain[g].assign(b->gtab[g].size() + 1, 0);
+        for (const lbm::BatchTableLattice& L : b->gtab[g])  // (36 plane: offsets of 32 bits)
+            b->chains &= L.kp.collide && lbm::chain2_takes(L.kp.nx, L.kp.ny, L.kp.pitch) &&
+                         36.0 * (double)L.kp.plane < 4294967296.0;
+    }
+    if (!b->chains) return;
+    const double full = 8.0 * b->sms;  // chains in flight
+    auto strips = [](const lbm::BatchTableLattice& L) {
+        return (L.kp.nx + lbm::kChainColumns - 1) / lbm::kChainColumns;
+    };
+    static const int kHeights[] = {8, 12, 16, 24, 32, 48, 64, 96, 128, 192};
+    for (int g = 0; g < b->ngroups; ++g) {
+        const std::vector<lbm::BatchTableLattice>& tab = b->gtab[g];
+        std::vector<int>& first = b->gchain[g];
+        double all = 0.0;  // rows of chains
+        for (const lbm::BatchTableLattice& L : tab) all += (double)strips(L) * L.kp.ny;
+        // first chain of every lattice with bands of the rows left for each
+        // chain in flight, but of least .. most rows; returns the clocks
+        auto plan = [&](int least, int most) {
+            double left = all, rows = 0.0;
+            int at = 0, tallest = 0, last = 0;
+            for (size_t j = 0; j < tab.size(); ++j) {
+                const int ny = tab[j].kp.ny;
+                const int r = (int)std::min<double>(most, std::max<double>(least, left / full));
+                const int nb = std::max(1, (ny + r / 2) / r);
+                first[j] = at;
+                at += strips(tab[j]) * nb;
+                last = (ny + nb - 1) / nb + 10;
+                tallest = std::max(tallest, last);
+                rows += (double)strips(tab[j]) * nb * last;
+                left -= (double)strips(tab[j]) * ny;
+            }
+            first.back() = at;
+            const double per_sm = std::max(1.0, (double)at / b->sms);
+            return at <= full ? tallest * (1100.0 + 212.0 * per_sm) * 1.5
+                              : (rows / full + 0.5 * last) * 2800.0;
+        };
+        double cost = 0.0;
+        int lo = 0, hi = 0;
+        for (int most : kHeights)
+            for (int least : kHeights) {
+                if (least > most) break;
+                const double c = plan(least, most);
+                if (lo == 0 || c < cost) {
+                    cost = c;
+                    lo = least;
+                    hi = most;
+                }
+            }
+        plan(lo, hi);
+    }
+}
+
 // Splits the active lattices into table groups, one scheme each and at most
 // kBatchTableCap lattices each, balancing their work items (largest lattice
 // first to the lightest group); no groups when they do not fit in the
@@ -1352,6 +1422,7 @@ void plan_groups(lbm_batch* b) {
                 if (!lbm::batch_small_fits(g, b->small)) b->small = lbm::SmallBatch{};
         }
     }
+    plan_chains(b);
     // the captured graphs hold the groups' launches: a new set of groups
     // (not new table contents) needs new graphs
     bool same = old == b->ngroups;
@@ -1374,7 +1445,7 @@ lbm_status ensure_tables(lbm_batch* b) {
         BCK(b, cudaDeviceSynchronize(), "cudaDeviceSynchronize");
     for (int g = 0; g < b->ngroups; ++g)
         BCK(b, lbm::batch_table_upload(g, b->gtab[g].data(), b->gbegin[g].data(),
-                                       (int)b->gtab[g].size(), b->stream),
+                                       b->gchain[g].data(), (int)b->gtab[g].size(), b->stream),
             "upload of a batch lattice table");
     g_table_owner[d] = b->serial;
     g_table_fresh[d] = true;
@@ -1747,29 +1818,41 @@ lbm_status advance(lbm_batch* b, int64_t nsteps, bool graphs) {
     if (b->n_active == 0 || nsteps == 0) return LBM_OK;
     if (lbm_status s = ensure_tables(b); s != LBM_OK) return s;
     int64_t left = nsteps;
+    int parity = b->parity;  // of the buffers that hold the state
     while (b->small.cluster && left > 0) {  // one launch per group and run of steps
         const int n = left < kSmallRun ? (int)left : kSmallRun;
-        const int from = (int)((b->parity + (nsteps - left)) & 1);
         for (int g = 0; g < b->ngroups; ++g)
-            BCK(b, lbm::batch_small_launch(g, b->small, (int)b->gtab[g].size(), from, n, b->stream),
+            BCK(b, lbm::batch_small_launch(g, b->small, (int)b->gtab[g].size(), parity, n, b->stream),
                 "batch step kernel (clusters)");
         b->launches += b->ngroups;
+        parity ^= n & 1;
         left -= n;
     }
+    // two steps per launch, the last one or two steps single, so that the
+    // other buffers then hold the states one step earlier
+    while (b->chains && !b->tuning && left >= 3) {
+        for (int g = 0; g < b->ngroups; ++g)
+            BCK(b, lbm::batch_chain_launch(g, parity, b->gchain[g].back(), b->graw[g], b->stream),
+                "batch two-step kernel");
+        b->launches += b->ngroups;
+        parity ^= 1;
+        left -= 2;
+    }
     while (graphs && left >= kGraphSteps) {
-        if (lbm_status s = ensure_graph(b, b->parity); s != LBM_OK) return s;
-        BCK(b, cudaGraphLaunch(b->graph[b->parity], b->stream), "cudaGraphLaunch");
+        if (lbm_status s = ensure_graph(b, parity); s != LBM_OK) return s;
+        BCK(b, cudaGraphLaunch(b->graph[parity], b->stream), "cudaGraphLaunch");
         left -= kGraphSteps;
         b->launches += kGraphSteps * kernels_per_step(b);
     }
     while (left > 0) {
         const int n = left < (1 << 20) ? (int)left : (1 << 20);
-        BCK(b, launch_steps(b, n, (int)((b->parity + (nsteps - left)) & 1), b->stream),
+        BCK(b, launch_steps(b, n, parity, b->stream),
             "batch step kernel");
         b->launches += n * kernels_per_step(b);
+        parity ^= n & 1;
         left -= n;
     }
-    b->parity = (int)((b->parity + nsteps) & 1);
+    b->parity = parity;
     for (int k = 0; k < b->count; ++k)
         if (b->active[k]) {
             b->steps[k] += nsteps;
@@ -1920,6 +2003,7 @@ lbm_status lbm_batch_tune(lbm_batch* b, int trial_steps, int* block_x, int* rows
     float best = 0.0f;
     int bbx = b->bx, brows = b->rows;
     lbm_status s = LBM_OK;
+    b->tuning = true;
     for (int bx : kBx) {
         for (int rows : kRows) {
             if ((s = set_shape(b, bx, rows)) != LBM_OK) break;
@@ -1938,6 +2022,7 @@ lbm_status lbm_batch_tune(lbm_batch* b, int trial_steps, int* block_x, int* rows
         }
         if (s != LBM_OK || ce != cudaSuccess) break;
     }
+    b->tuning = false;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (s != LBM_OK) return s;

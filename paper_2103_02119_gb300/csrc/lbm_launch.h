@@ -45,9 +45,14 @@ cudaError_t launch_chain2(const float* fin, float* fout, const KParams<float>& p
 // Bands of the lattice for launch_chain2 on a device of `sms` SMs: the fewest
 // clocks by a model of the march (a row of a chain takes longer the more
 // chains share its SM; every band marches ten rows more than it stores; the
-// launch ends when its slowest chain does, uneven: solid
-// cells, whose chains take longer); 0 when the lattice cannot take the path.
-int chain2_bands(int nx, int ny, int pitch, bool uneven, int sms);
+// launch ends when its slowest chain does); 0 when the lattice cannot take the
+// path.
+int chain2_bands(int nx, int ny, int pitch, int sms);
+// Columns that a chain stores, and whether a lattice can take the kernel.
+constexpr int kChainColumns = 56;
+inline bool chain2_takes(int nx, int ny, int pitch) {
+    return nx >= 64 && ny >= 16 && 4.0 * pitch * ny < 4294967296.0;
+}
 template <typename T>
 int step_occupancy(int bx, bool mask);
 
@@ -110,8 +115,9 @@ SmallBatch small_batch_shape(const int* nx, const int* ny, int n, int sms);
     cudaError_t batch_small_launch_##S(const SmallBatch& b, int n, int from, int nsteps,   \
                                        cudaStream_t s);                                    \
     bool batch_small_fits_##S(const SmallBatch& b);                                        \
-    cudaError_t batch_table_upload_##S(const BatchTableLattice* lat, const int* begin, int n, \
-                                       cudaStream_t s);                                     \
+    cudaError_t batch_table_upload_##S(const BatchTableLattice* lat, const int* begin,      \
+                                       const int* chain_begin, int n, cudaStream_t s);      \
+    cudaError_t batch_chain_launch_##S(int parity, int chains, int raw, cudaStream_t s);    \
     cudaError_t batch_table_launch_##S(int parity, int bx, int grid, int raw, cudaStream_t s); \
     int batch_table_occupancy_##S(int bx);
 LBM_DECLARE_BATCH_TABLE(0)
@@ -120,15 +126,24 @@ LBM_DECLARE_BATCH_TABLE(2)
 LBM_DECLARE_BATCH_TABLE(3)
 #undef LBM_DECLARE_BATCH_TABLE
 // Table `slot`: copy n lattices (host array) and their first work items
-// begin[0 .. n] (begin[n]: the group's number of work items) into it,
+// begin[0 .. n] (begin[n]: the group's number of work items) into it, and the
+// first chains chain_begin[0 .. n] of the two-step kernel,
 // asynchronously on s (after the kernels of the slot that were issued before
 // on s; the caller orders them).
 inline cudaError_t batch_table_upload(int slot, const BatchTableLattice* lat, const int* begin,
-                                      int n, cudaStream_t s) {
-    return slot == 0   ? batch_table_upload_0(lat, begin, n, s)
-           : slot == 1 ? batch_table_upload_1(lat, begin, n, s)
-           : slot == 2 ? batch_table_upload_2(lat, begin, n, s)
-                       : batch_table_upload_3(lat, begin, n, s);
+                                      const int* chain_begin, int n, cudaStream_t s) {
+    return slot == 0   ? batch_table_upload_0(lat, begin, chain_begin, n, s)
+           : slot == 1 ? batch_table_upload_1(lat, begin, chain_begin, n, s)
+           : slot == 2 ? batch_table_upload_2(lat, begin, chain_begin, n, s)
+                       : batch_table_upload_3(lat, begin, chain_begin, n, s);
+}
+// Two steps of every lattice of table `slot` (each chain2_takes, collision
+// on), from buffer f[parity] to the other: one block per chain.
+inline cudaError_t batch_chain_launch(int slot, int parity, int chains, int raw, cudaStream_t s) {
+    return slot == 0   ? batch_chain_launch_0(parity, chains, raw, s)
+           : slot == 1 ? batch_chain_launch_1(parity, chains, raw, s)
+           : slot == 2 ? batch_chain_launch_2(parity, chains, raw, s)
+                       : batch_chain_launch_3(parity, chains, raw, s);
 }
 // One step of every lattice of table `slot` (all of one scheme: raw = 1 for
 // RNR-LBM), from buffer f[parity], on a persistent grid of `grid` blocks.
