@@ -46,17 +46,17 @@ constexpr unsigned kBiasBlocks = 304;  // most blocks of one launch of the bias-
 // range: the error of m / 2^s is below 2^-31 / d).
 struct FastDiv {
     unsigned d = 1;
-    unsigned long long m = 1ull << 31;
+    unsigned m = 1u << 31;  // (below 2^32 for every d)
     int s = 31;
     FastDiv() = default;
     explicit FastDiv(unsigned dv) : d(dv) {
         int l = 0;
         while ((1ull << l) < dv) ++l;
         s = 31 + l;
-        m = ((1ull << s) + dv - 1) / dv;
+        m = (unsigned)(((1ull << s) + dv - 1) / dv);
     }
     __device__ __forceinline__ unsigned div(unsigned n) const {
-        return (unsigned)(((unsigned long long)n * m) >> s);
+        return (unsigned)((unsigned long long)n * m >> s);
     }
 };
 
@@ -77,17 +77,32 @@ Geo make_geo(int n, int h, int w, long long P) {
     return g;
 }
 
-__device__ __forceinline__ bool shifted(const Geo& g, long long p, int dy, int dx, long long& q) {
-    const unsigned pp = (unsigned)p;
-    const unsigned nn = g.fhw.div(pp);
-    const unsigned rem = pp - nn * g.fhw.d;
-    const unsigned yy = g.fw.div(rem);
-    const int y = (int)yy + dy, x = (int)(rem - yy * g.fw.d) + dx;
-    if (y < 0 || y >= g.h || x < 0 || x >= g.w) return false;
-    q = ((long long)nn * g.h + y) * g.w + x;
-    return true;
+// Eight channels of one pixel (16 bytes; channel counts are padded to
+// multiples of 8) at a time, with 32-bit index arithmetic: the scalar forms
+// spent most of their time on 64-bit divisions.
+struct Oct {
+    float v[8];
+};
+__device__ __forceinline__ Oct load8(const bf16* p) {
+    const uint4 q = *reinterpret_cast<const uint4*>(p);
+    const unsigned w[4] = {q.x, q.y, q.z, q.w};
+    Oct o;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        o.v[2 * k] = __uint_as_float(w[k] << 16);
+        o.v[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
+    }
+    return o;
 }
-
+__device__ __forceinline__ void put8(bf16* p, const Oct& o) {
+    unsigned w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(o.v[2 * k], o.v[2 * k + 1]);
+        w[k] = *reinterpret_cast<const unsigned*>(&h);
+    }
+    *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
+}
 // ---- operand tiles of the tensor-core GEMM ----
 //
 // A tile holds rows r (UM = 128 of A, BN of B) and the K chunk [k0, k0 + UK)
@@ -99,6 +114,7 @@ __device__ __forceinline__ bool shifted(const Geo& g, long long p, int dy, int d
 // one k.  Every operand arrives in 16-byte pieces of one of those two kinds,
 // copied by cp.async (zero-filled outside the operand).
 constexpr int UM = 128, UK = 64, kGemmThreads = 128;
+constexpr int kConvSmemMax = 227 * 1024;
 constexpr unsigned kLBO = 128, kSBO = (UK / 8) * 128;
 
 // byte offset of the 16-byte piece holding rows r .. r+7 at k (MN-major) or
@@ -112,12 +128,93 @@ __device__ __forceinline__ unsigned mnmajor_off(int r8, int kc) {
 __device__ __forceinline__ unsigned smem_addr(const void* p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
-// 16 bytes global -> shared, or 16 zero bytes when !valid
-__device__ __forceinline__ void cp16(unsigned dst, const void* src, bool valid) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
+// 16 bytes global -> shared, or 16 zero bytes when !valid (any: an address
+// inside the operand, for those)
+__device__ __forceinline__ void cp16(unsigned dst, const bf16* src, const bf16* any, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(valid ? src : any),
                  "r"(valid ? 16 : 0)
                  : "memory");
 }
+
+// The A tile of a convolution over pixels, K-major: row r is pixel m0 + r,
+// column k channel k mod c of tap k / c (TS = 1: the pixel's neighbour at the
+// tap, TS = -1: its opposite).  A thread copies one 16-byte piece of eight
+// rows, always the same rows and the same column of a chunk, so what depends on
+// the row (whether each tap leaves the grid: nine bits) is found once, and a
+// chunk costs one division and an add and a bit test per piece.  (With the
+// pixel's and the tap's divisions at every piece the copies were what bounded
+// the kernel: forward and input-gradient convolutions of a batch of 16 at
+// 64 x 64, 32 to 256 channels, 546 and 472 us.)
+template <int TS>
+struct ConvRows {
+    static constexpr int kRows = UM * UK / 8 / kGemmThreads;
+    const bf16* in;
+    const bf16* base;    // piece of row r0 at channel 0 of the centre tap
+    long long stride;    // elements between the thread's rows
+    unsigned mask[kRows];
+    int c, w, kc;
+    unsigned dst;
+    FastDiv fk;
+    __device__ __forceinline__ ConvRows(const Geo& g, const FastDiv& fk_, const bf16* in_, int c_,
+                                        long long m0, int tid)
+        : in(in_), c(c_), w(g.w), fk(fk_) {
+        const int r0 = tid >> 3;
+        kc = (tid & 7) * 8;
+        base = in + (m0 + r0) * c;
+        stride = (long long)(kGemmThreads / 8) * c;
+        dst = kmajor_off(r0, kc);
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) {
+            const long long p = m0 + r0 + i * (kGemmThreads / 8);
+            mask[i] = 0;
+            if (p < g.P) {
+                const unsigned pp = (unsigned)p, nn = g.fhw.div(pp), rem = pp - nn * g.fhw.d,
+                               y = g.fw.div(rem), x = rem - y * g.fw.d;
+                // taps (rows of three) that stay inside
+                const unsigned row = (x > 0 ? 1u : 0u) | 2u | ((int)x < g.w - 1 ? 4u : 0u);
+                mask[i] = (y > 0 ? row : 0u) | row << 3 | ((int)y < g.h - 1 ? row << 6 : 0u);
+            }
+        }
+    }
+    __device__ __forceinline__ void load(unsigned t, long long k0, long long kend) const {
+        const unsigned k = (unsigned)k0 + kc;
+        unsigned tap = fk.div(k);
+        const int ci = (int)(k - tap * c);
+        if (TS < 0) tap = 8 - tap;
+        const unsigned ty = tap / 3;
+        const bf16* src = base + (long long)(((int)ty - 1) * w + (int)(tap - 3 * ty) - 1) * c + ci;
+        const unsigned bit = k < (unsigned)kend ? 1u << tap : 0u;
+#pragma unroll
+        for (int i = 0; i < kRows; ++i, src += stride)
+            cp16(t + dst + i * (kGemmThreads / 64) * kSBO, src, in, (mask[i] & bit) != 0);
+    }
+};
+// The B tile, K-major: row r is row n0 + r of a [n][kall] matrix.
+template <int BN>
+struct WeightRows {
+    const bf16* wt;
+    const bf16* base;
+    long long stride;
+    int left, kc;        // rows from the thread's first on
+    unsigned dst;
+    __device__ __forceinline__ WeightRows(const bf16* wt_, int n, long long kall, int n0, int tid)
+        : wt(wt_) {
+        const int r0 = tid >> 3;
+        kc = (tid & 7) * 8;
+        base = wt + (n0 + r0) * kall + kc;
+        stride = kGemmThreads / 8 * kall;
+        left = n - n0 - r0;
+        dst = kmajor_off(r0, kc);
+    }
+    __device__ __forceinline__ void load(unsigned t, long long k0, long long kend) const {
+        const bf16* src = base + k0;
+        const bool in = k0 + kc < kend;
+#pragma unroll
+        for (int i = 0; i < BN / (kGemmThreads / 8); ++i, src += stride)
+            cp16(t + dst + i * (kGemmThreads / 64) * kSBO, src, wt,
+                 in && i * (kGemmThreads / 8) < left);
+    }
+};
 
 // Forward: out = act(conv(in) + b).  M = pixels, N = cout, K = 9 cin:
 // A[p][(tap, ci)] = in(p + s(tap))[ci], B[co][(tap, ci)] = W; both K-major.
@@ -133,47 +230,32 @@ struct FwdOp {
     __host__ __device__ long long M() const { return g.P; }
     __host__ __device__ int N() const { return cout; }
     __host__ __device__ long long K() const { return 9LL * cin; }
-    __device__ void load_a(unsigned t, long long m0, long long k0, long long kend, int tid) const {
-#pragma unroll
-        for (int i = 0; i < UM * UK / 8 / kGemmThreads; ++i) {
-            const int v = tid + i * kGemmThreads, r = v >> 3, kc = (v & 7) * 8;
-            const long long p = m0 + r, k = k0 + kc;
-            const bf16* src = in;
-            bool ok = false;
-            if (p < g.P && k < kend) {
-                const int tap = (int)fk.div((unsigned)k), ci = (int)k - tap * cin;
-                long long q;
-                if (shifted(g, p, tap / 3 - 1, tap % 3 - 1, q)) {
-                    src = in + q * cin + ci;
-                    ok = true;
-                }
-            }
-            cp16(t + kmajor_off(r, kc), src, ok);
-        }
+    __device__ ConvRows<1> rows_a(long long m0, int tid) const {
+        return ConvRows<1>(g, fk, in, cin, m0, tid);
     }
-    __device__ void load_b(unsigned t, int n0, long long k0, long long kend, int tid,
-                           int bn) const {
-        for (int v = tid; v < bn * (UK / 8); v += kGemmThreads) {
-            const int r = v >> 3, kc = (v & 7) * 8;
-            const long long k = k0 + kc;
-            const bool ok = n0 + r < cout && k < kend;
-            cp16(t + kmajor_off(r, kc), ok ? wf + (long long)(n0 + r) * K() + k : wf, ok);
+    template <int BN>
+    __device__ WeightRows<BN> rows_b(int n0, int tid) const {
+        return WeightRows<BN>(wf, cout, K(), n0, tid);
+    }
+    static constexpr int kTap = 1;  // sign of a tap's shift
+    __host__ __device__ int channels() const { return cin; }
+    __device__ const bf16* pixels() const { return in; }
+    __device__ const bf16* weights() const { return wf; }
+    // eight output channels (a multiple of 8 of them) of pixel p
+    __device__ void store8(long long p, int col, const float* v) const {
+        if (col >= cout) return;
+        Oct o;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            o.v[j] = v[j] + bias[col + j];
+            if (relu) o.v[j] = fmaxf(o.v[j], 0.0f);
         }
+        put8(out + p * cout + col, o);
     }
     __device__ void store16(long long row, int col0, const float* v, int) const {
         if (row >= g.P) return;
-#pragma unroll
-        for (int j = 0; j < 16; j += 2) {
-            const int col = col0 + j;
-            if (col >= cout) break;
-            float v0 = v[j] + bias[col], v1 = v[j + 1] + bias[col + 1];
-            if (relu) {
-                v0 = fmaxf(v0, 0.0f);
-                v1 = fmaxf(v1, 0.0f);
-            }
-            *reinterpret_cast<__nv_bfloat162*>(out + row * cout + col) =
-                __floats2bfloat162_rn(v0, v1);
-        }
+        store8(row, col0, v);
+        store8(row, col0 + 8, v + 8);
     }
 };
 
@@ -190,41 +272,93 @@ struct DgradOp {
     __host__ __device__ long long M() const { return g.P; }
     __host__ __device__ int N() const { return cin; }
     __host__ __device__ long long K() const { return 9LL * cout; }
-    __device__ void load_a(unsigned t, long long m0, long long k0, long long kend, int tid) const {
-#pragma unroll
-        for (int i = 0; i < UM * UK / 8 / kGemmThreads; ++i) {
-            const int v = tid + i * kGemmThreads, r = v >> 3, kc = (v & 7) * 8;
-            const long long p = m0 + r, k = k0 + kc;
-            const bf16* src = gpre;
-            bool ok = false;
-            if (p < g.P && k < kend) {
-                const int tap = (int)fk.div((unsigned)k), co = (int)k - tap * cout;
-                long long q;
-                if (shifted(g, p, 1 - tap / 3, 1 - tap % 3, q)) {
-                    src = gpre + q * cout + co;
-                    ok = true;
-                }
-            }
-            cp16(t + kmajor_off(r, kc), src, ok);
-        }
+    __device__ ConvRows<-1> rows_a(long long m0, int tid) const {
+        return ConvRows<-1>(g, fk, gpre, cout, m0, tid);
     }
-    __device__ void load_b(unsigned t, int n0, long long k0, long long kend, int tid,
-                           int bn) const {
-        for (int v = tid; v < bn * (UK / 8); v += kGemmThreads) {
-            const int r = v >> 3, kc = (v & 7) * 8;
-            const long long k = k0 + kc;
-            const bool ok = n0 + r < cin && k < kend;
-            cp16(t + kmajor_off(r, kc), ok ? wd + (long long)(n0 + r) * K() + k : wd, ok);
-        }
+    template <int BN>
+    __device__ WeightRows<BN> rows_b(int n0, int tid) const {
+        return WeightRows<BN>(wd, cin, K(), n0, tid);
+    }
+    static constexpr int kTap = -1;
+    __host__ __device__ int channels() const { return cout; }
+    __device__ const bf16* pixels() const { return gpre; }
+    __device__ const bf16* weights() const { return wd; }
+    __device__ void store8(long long p, int col, const float* v) const {
+        if (col >= cin) return;
+        Oct o;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) o.v[j] = v[j];
+        put8(gin + p * cin + col, o);
     }
     __device__ void store16(long long row, int col0, const float* v, int) const {
         if (row >= g.P) return;
+        store8(row, col0, v);
+        store8(row, col0 + 8, v + 8);
+    }
+};
+
+// The A tile of the weight gradient, MN-major: eight channels (one 16-byte
+// piece) of tap m / cin at pixel k.  A thread's channels and tap are the same in
+// every chunk; its eight pixels of a chunk lie eight apart.
+struct PixelColumns {
+    static constexpr int kPixels = UM * UK / 8 / kGemmThreads;
+    const bf16* x0;
+    const bf16* base;   // the channels, at the tap's neighbour of pixel 0
+    const Geo& g;
+    int c, dy, dx, kk;
+    bool in;
+    unsigned dst;
+    __device__ __forceinline__ PixelColumns(const Geo& g_, const FastDiv& fk, const bf16* x, int c_,
+                                            long long m0, long long M, int tid)
+        : x0(x), g(g_), c(c_) {
+        // consecutive threads on consecutive channel groups of one pixel
+        const int grp = tid & 15;
+        kk = tid >> 4;
+        const long long m = m0 + grp * 8;
+        in = m < M;
+        const unsigned tap = fk.div((unsigned)m), ty = tap / 3;
+        dy = (int)ty - 1;
+        dx = (int)(tap - 3 * ty) - 1;
+        base = x + (long long)(dy * g.w + dx) * c + ((int)m - (int)tap * c);
+        dst = mnmajor_off(grp * 8, kk);
+    }
+    __device__ __forceinline__ void load(unsigned t, long long k0, long long kend) const {
 #pragma unroll
-        for (int j = 0; j < 16; j += 2) {
-            const int col = col0 + j;
-            if (col >= cin) break;
-            *reinterpret_cast<__nv_bfloat162*>(gin + row * cin + col) =
-                __floats2bfloat162_rn(v[j], v[j + 1]);
+        for (int i = 0; i < kPixels; ++i) {
+            const long long p = k0 + kk + i * (kGemmThreads / 16);
+            const unsigned pp = (unsigned)p, nn = g.fhw.div(pp), rem = pp - nn * g.fhw.d,
+                           yy = g.fw.div(rem);
+            const unsigned y = yy + dy, x = rem - yy * g.fw.d + dx;
+            const bool ok = in && p < kend && y < (unsigned)g.h && x < (unsigned)g.w;
+            cp16(t + dst + i * (kGemmThreads / 128) * kLBO, base + p * c, x0, ok);
+        }
+    }
+};
+// Its B tile, MN-major: eight channels of the output gradient at pixel k.
+template <int BN>
+struct GradColumns {
+    static constexpr int kGroups = BN / 8, kStep = kGemmThreads / kGroups;  // threads of a pixel
+    const bf16* g0;
+    const bf16* base;
+    int c, kk;
+    bool in;
+    unsigned dst;
+    __device__ __forceinline__ GradColumns(const bf16* gpre, int c_, int n0, int tid)
+        : g0(gpre), c(c_) {
+        const int grp = tid % kGroups, co = n0 + grp * 8;
+        kk = tid / kGroups;
+        in = co < c;
+        base = gpre + co;
+        dst = mnmajor_off(grp * 8, 0);
+    }
+    __device__ __forceinline__ void load(unsigned t, long long k0, long long kend) const {
+        static_assert(UK % kStep == 0);
+#pragma unroll
+        for (int i = 0; i < UK / kStep; ++i) {
+            const int k = kk + i * kStep;
+            const long long p = k0 + k;
+            cp16(t + dst + (unsigned)(k >> 3) * kLBO + (unsigned)(k & 7) * 16, base + p * c, g0,
+                 in && p < kend);
         }
     }
 };
@@ -246,35 +380,12 @@ struct WgradOp {
     __host__ __device__ long long M() const { return 9LL * cin; }
     __host__ __device__ int N() const { return cout; }
     __host__ __device__ long long K() const { return g.P; }
-    __device__ void load_a(unsigned t, long long m0, long long k0, long long kend, int tid) const {
-        // pieces (group of 8 rows, pixel): 16 x 64, consecutive threads on
-        // consecutive channel groups of one pixel
-#pragma unroll
-        for (int i = 0; i < UM * UK / 8 / kGemmThreads; ++i) {
-            const int v = tid + i * kGemmThreads, grp = v & 15, kk = v >> 4;
-            const long long m = m0 + grp * 8, p = k0 + kk;
-            const bf16* src = in;
-            bool ok = false;
-            if (m < M() && p < kend) {
-                const int tap = (int)fk.div((unsigned)m), ci = (int)m - tap * cin;
-                long long q;
-                if (shifted(g, p, tap / 3 - 1, tap % 3 - 1, q)) {
-                    src = in + q * cin + ci;
-                    ok = true;
-                }
-            }
-            cp16(t + mnmajor_off(grp * 8, kk), src, ok);
-        }
+    __device__ PixelColumns rows_a(long long m0, int tid) const {
+        return PixelColumns(g, fk, in, cin, m0, M(), tid);
     }
-    __device__ void load_b(unsigned t, int n0, long long k0, long long kend, int tid,
-                           int bn) const {
-        for (int v = tid; v < (bn / 8) * UK; v += kGemmThreads) {
-            const int grp = v % (bn / 8), kk = v / (bn / 8);
-            const int co = n0 + grp * 8;
-            const long long p = k0 + kk;
-            const bool ok = co < cout && p < kend;
-            cp16(t + mnmajor_off(grp * 8, kk), ok ? gpre + p * cout + co : gpre, ok);
-        }
+    template <int BN>
+    __device__ GradColumns<BN> rows_b(int n0, int tid) const {
+        return GradColumns<BN>(gpre, cout, n0, tid);
     }
     __device__ void store16(long long row, int col0, const float* v, int z) const {
         if (row >= M()) return;
@@ -366,11 +477,13 @@ __global__ void __launch_bounds__(kGemmThreads) umma_gemm_kernel(const Op op, lo
     constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) |
                                ((Op::kAmn ? 1u : 0u) << 15) | ((Op::kBmn ? 1u : 0u) << 16) |
                                ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(UM >> 4) << 24);
+    const auto rows_a = op.rows_a(m0, tid);
+    const auto rows_b = op.template rows_b<BN>(n0, tid);
     auto load = [&](int kb) {
         const unsigned st = s0 + (unsigned)(kb % NS) * kStage;
         const long long k0 = kbeg + (long long)kb * UK;
-        op.load_a(st, m0, k0, kend, tid);
-        op.load_b(st + UM * UK * 2, n0, k0, kend, tid, BN);
+        rows_a.load(st, k0, kend);
+        rows_b.load(st + UM * UK * 2, k0, kend);
     };
 #pragma unroll
     for (int kb = 0; kb < NS - 1; ++kb) {
@@ -465,49 +578,229 @@ cudaError_t launch_umma_bn(const Op& op, long long kchunk, int splits, int* err,
     return cudaGetLastError();
 }
 
-// The tile width: the smallest UMMA N (16, 32, 64, 128, 256) that covers N,
-// 256 above.
-#ifndef LBM_GEMM_WIDE
-#define LBM_GEMM_WIDE 1
-#endif
+// ---- convolutions over a tile of pixels ----
+//
+// A 3 x 3 convolution as a GEMM reads every pixel nine times, and the copies of
+// the nine shifted tiles are what bounds it.  Here a CTA copies its pixels and
+// their neighbours once: the pixels of the batch are laid out as positions, one
+// padding column after each row and one padding row after each image (zeros),
+// so that a tap's neighbours of 128 consecutive positions are 128 consecutive
+// positions too.  In shared memory eight channels of a position are 16 bytes,
+// positions adjacent and channel groups a plane apart: the tensor core's
+// no-swizzle K-major layout with row groups 128 bytes and K core matrices a
+// plane apart, in which a tap's tile begins 16 bytes per position further.  So
+// the nine taps' operands are nine start addresses in one tile.
+// The CTA copies everything it needs up front (the tile and the first tap's
+// weights, then the weights of each further tap, as cp.async groups) and issues
+// a tap's MMAs as its weights land, in the order of the GEMM's K: taps, then
+// channels in steps of 16, so the sums are the GEMM's, bit for bit.
+// Planes are an odd number of 16-byte pieces apart (copies then write to
+// distinct banks).
+// Measured, a batch of 16 at 64 x 64, 32 to 256 channels: the 15 forward
+// convolutions 546 us as GEMMs with divisions at every piece, 370 without them
+// and in narrower tiles where the tiles are few, 249 here; the 14 input gradients
+// 472, 342, 218.  What bounds it now is latency: a CTA's copies, nine taps and
+// read-out follow one another (9 to 29 us a convolution of 1.2 GFLOP).
+struct ConvTile {
+    FastDiv fpitch, frows, fgroups;  // by w + 1, h + 1 and the channel groups
+    unsigned positions;              // n (h + 1) (w + 1)
+    int halo, pieces;                // w + 2; pieces of a plane
+};
 template <class Op>
-cudaError_t launch_gemm(const Op& op, long long kchunk, int splits, int* err, cudaStream_t s) {
+ConvTile conv_tile(const Op& op) {
+    ConvTile t;
+    t.fpitch = FastDiv((unsigned)op.g.w + 1);
+    t.frows = FastDiv((unsigned)op.g.h + 1);
+    t.fgroups = FastDiv((unsigned)op.channels() / 8);
+    t.positions = (unsigned)op.g.n * (op.g.h + 1) * (op.g.w + 1);
+    t.halo = op.g.w + 2;
+    t.pieces = (UM + 2 * t.halo) | 1;
+    return t;
+}
+inline size_t conv_tile_smem(int pieces, int channels, int bn) {
+    return (size_t)(channels / 8) * (pieces + 9 * (bn + 1)) * 16 + 16;
+}
+
+template <class Op, int BN>
+__global__ void __launch_bounds__(kGemmThreads) conv_tile_kernel(const Op op, const ConvTile ct,
+                                                                 int* err) {
+    constexpr int TC = tmem_cols<BN>();
+    extern __shared__ __align__(1024) unsigned char sm[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int c = op.channels(), groups = c / 8;
+    const unsigned m0 = blockIdx.x * UM;
+    const int n0 = blockIdx.y * BN;
+    const unsigned a0 = smem_addr(sm), plane = (unsigned)ct.pieces * 16;
+    const unsigned b0 = a0 + groups * plane, bplane = (BN + 1) * 16;
+    const unsigned bar = b0 + 9 * groups * bplane, tslot = bar + 8;
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tslot),
+                     "n"(TC)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // position pos: its pixel, or -1 for padding
+    auto pixel = [&](unsigned pos) -> long long {
+        if (pos >= ct.positions) return -1;  // (positions below 0 too)
+        const unsigned row = ct.fpitch.div(pos), x = pos - row * ct.fpitch.d;
+        const unsigned nn = ct.frows.div(row), y = row - nn * ct.frows.d;
+        if (x == (unsigned)op.g.w || y == (unsigned)op.g.h) return -1;
+        return ((long long)nn * op.g.h + y) * op.g.w + x;
+    };
+    {
+        const bf16* in = op.pixels();
+        const int total = (UM + 2 * ct.halo) * groups;
+        for (int v = tid; v < total; v += kGemmThreads) {
+            const int px = (int)ct.fgroups.div((unsigned)v), cg = v - px * groups;
+            const long long p = pixel(m0 + (unsigned)px - (unsigned)ct.halo);
+            cp16(a0 + cg * plane + px * 16, in + p * c + cg * 8, in, p >= 0);
+        }
+    }
+    const bf16* wt = op.weights();
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+        for (int v = tid; v < BN * groups; v += kGemmThreads) {
+            const int r = (int)ct.fgroups.div((unsigned)v), cg = v - r * groups;
+            cp16(b0 + (t * groups + cg) * bplane + r * 16,
+                 wt + (long long)(n0 + r) * 9 * c + t * c + cg * 8, wt, n0 + r < op.N());
+        }
+        cp_commit();
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    unsigned taddr;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(taddr) : "r"(tslot) : "memory");
+    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+                               ((uint32_t)(UM >> 4) << 24);
+    auto tap = [&](int t) {  // after its cp.async group
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (tid != 0) return;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int shift = Op::kTap * ((t / 3 - 1) * (op.g.w + 1) + t % 3 - 1);
+        const unsigned at = a0 + (unsigned)(ct.halo + shift) * 16, bt = b0 + t * groups * bplane;
+        for (int k = 0; k < groups; k += 2) {
+            const uint64_t ad = smem_desc(at + k * plane, plane, 128);
+            const uint64_t bd = smem_desc(bt + k * bplane, bplane, 128);
+            const unsigned acc = t > 0 || k > 0 ? 1u : 0u;
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(taddr),
+                "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+                : "memory");
+        }
+        if (t == 8)
+            asm volatile(
+                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+                : "memory");
+    };
+    cp_wait<8>(); tap(0);
+    cp_wait<7>(); tap(1);
+    cp_wait<6>(); tap(2);
+    cp_wait<5>(); tap(3);
+    cp_wait<4>(); tap(4);
+    cp_wait<3>(); tap(5);
+    cp_wait<2>(); tap(6);
+    cp_wait<1>(); tap(7);
+    cp_wait<0>(); tap(8);
+    const bool ok = mbar_wait_parity(bar, 0);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const long long p = pixel(m0 + 32 * warp + lane);
+#pragma unroll 1
+    for (int c0 = 0; c0 < BN; c0 += 16) {
+        uint32_t r[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
+            "%13,%14,%15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+              "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+              "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(taddr + ((unsigned)(32 * warp) << 16) + (unsigned)c0));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        float v[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+        if (ok && p >= 0) {
+            op.store8(p, n0 + c0, v);
+            op.store8(p, n0 + c0 + 8, v + 8);
+        }
+    }
+    if (!ok && lane == 0) atomicExch(err, 1);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "n"(TC)
+                     : "memory");
+}
+
+template <class Op, int BN>
+cudaError_t launch_conv_bn(const Op& op, const ConvTile& t, int* err, cudaStream_t s) {
+    static bool configured = false;
+    if (!configured) {
+        cudaError_t e = cudaFuncSetAttribute(conv_tile_kernel<Op, BN>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kConvSmemMax);
+        if (e != cudaSuccess) return e;
+        configured = true;
+    }
+    const dim3 grid((t.positions + UM - 1) / UM, (op.N() + BN - 1) / BN);
+    conv_tile_kernel<Op, BN>
+        <<<grid, kGemmThreads, conv_tile_smem(t.pieces, op.channels(), BN), s>>>(op, t, err);
+    return cudaGetLastError();
+}
+
+// The tile width: the smallest UMMA N (16, 32, 64, 128, 256) that covers N,
+// 256 above; narrower ones, down to 32, while the tiles are fewer than `fill`.
+template <class Op>
+cudaError_t launch_gemm(const Op& op, long long kchunk, int splits, int fill, int* err,
+                        cudaStream_t s) {
     const int n = op.N();
-    if (n <= 16) return launch_umma_bn<Op, 16>(op, kchunk, splits, err, s);
-    if (n <= 32) return launch_umma_bn<Op, 32>(op, kchunk, splits, err, s);
-    if (n <= 64) return launch_umma_bn<Op, 64>(op, kchunk, splits, err, s);
-    if (n <= 128 || !LBM_GEMM_WIDE) return launch_umma_bn<Op, 128>(op, kchunk, splits, err, s);
-    return launch_umma_bn<Op, 256>(op, kchunk, splits, err, s);
+    const long long gm = (op.M() + UM - 1) / UM * splits;
+    int bn = n <= 16 ? 16 : n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : 256;
+    while (bn > 32 && gm * ((n + bn - 1) / bn) < fill) bn /= 2;
+    switch (bn) {
+    case 16: return launch_umma_bn<Op, 16>(op, kchunk, splits, err, s);
+    case 32: return launch_umma_bn<Op, 32>(op, kchunk, splits, err, s);
+    case 64: return launch_umma_bn<Op, 64>(op, kchunk, splits, err, s);
+    case 128: return launch_umma_bn<Op, 128>(op, kchunk, splits, err, s);
+    default: return launch_umma_bn<Op, 256>(op, kchunk, splits, err, s);
+    }
+}
+
+// A forward or input-gradient convolution: over tiles of pixels where the
+// channels come in steps of 16 and a tile with its weights fits a CTA's shared
+// memory (always the faster one then); else as a GEMM.  In columns that cover N,
+// or fewer, down to 32, while the tiles are fewer than the SMs: of a batch of 16
+// at 8 x 8 with 256 channels, eight tiles of 256 columns took 93 us, 64 of 32
+// columns 33 (both as GEMMs).
+template <class Op>
+cudaError_t launch_conv(const Op& op, int sms, int* err, cudaStream_t s) {
+    const int n = op.N(), c = op.channels();
+    const ConvTile t = conv_tile(op);
+    const double positions = (double)op.g.n * (op.g.h + 1) * (op.g.w + 1);
+    int bn = n <= 16 ? 16 : n <= 32 ? 32 : n <= 64 ? 64 : 128;
+    const long long gm = ((long long)t.positions + UM - 1) / UM;
+    while (bn > 32 && (gm * ((n + bn - 1) / bn) < sms ||
+                       conv_tile_smem(t.pieces, c, bn) > (size_t)kConvSmemMax))
+        bn /= 2;
+    if (c % 16 || positions >= 2147483648.0 ||
+        conv_tile_smem(t.pieces, c, bn) > (size_t)kConvSmemMax)
+        return launch_gemm(op, op.K(), 1, sms, err, s);
+    switch (bn) {
+    case 16: return launch_conv_bn<Op, 16>(op, t, err, s);
+    case 32: return launch_conv_bn<Op, 32>(op, t, err, s);
+    case 64: return launch_conv_bn<Op, 64>(op, t, err, s);
+    default: return launch_conv_bn<Op, 128>(op, t, err, s);
+    }
 }
 
 // ---- elementwise and reduction kernels ----
 
-// Eight channels of one pixel (16 bytes; channel counts are padded to
-// multiples of 8) at a time, with 32-bit index arithmetic: the scalar forms
-// spent most of their time on 64-bit divisions.
-struct Oct {
-    float v[8];
-};
-__device__ __forceinline__ Oct load8(const bf16* p) {
-    const uint4 q = *reinterpret_cast<const uint4*>(p);
-    const unsigned w[4] = {q.x, q.y, q.z, q.w};
-    Oct o;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        o.v[2 * k] = __uint_as_float(w[k] << 16);
-        o.v[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
-    }
-    return o;
-}
-__device__ __forceinline__ void store8(bf16* p, const Oct& o) {
-    unsigned w[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(o.v[2 * k], o.v[2 * k + 1]);
-        w[k] = *reinterpret_cast<const unsigned*>(&h);
-    }
-    *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-}
 // Octet i of an (n, h, w, 8 c8) tensor: its pixel and channel group.
 struct At {
     unsigned p, y, x, g;
@@ -536,7 +829,7 @@ pool_kernel(const bf16* in, bf16* out, unsigned total, FastDiv c8, FastDiv fwo, 
         Oct o;
 #pragma unroll
         for (int k = 0; k < 8; ++k) o.v[k] = 0.25f * (((a.v[k] + b.v[k]) + d.v[k]) + e.v[k]);
-        store8(out + t.off, o);
+        put8(out + t.off, o);
     }
 }
 
@@ -555,7 +848,7 @@ pool_back_kernel(const bf16* g, bf16* gin, unsigned total, FastDiv c8, FastDiv f
         Oct o;
 #pragma unroll
         for (int k = 0; k < 8; ++k) o.v[k] = 0.25f * a.v[k] + b.v[k];
-        store8(gin + t.off, o);
+        put8(gin + t.off, o);
     }
 }
 
@@ -585,7 +878,7 @@ up_back_kernel(const bf16* g, bf16* gin, unsigned total, FastDiv c8, FastDiv fw,
         Oct o;
 #pragma unroll
         for (int k = 0; k < 8; ++k) o.v[k] = ((a.v[k] + b.v[k]) + d.v[k]) + e.v[k];
-        store8(gin + t.off, o);
+        put8(gin + t.off, o);
     }
 }
 
@@ -597,7 +890,7 @@ add_kernel(const bf16* a, const bf16* b, bf16* out, unsigned total) {
         Oct o;
 #pragma unroll
         for (int k = 0; k < 8; ++k) o.v[k] = x.v[k] + y.v[k];
-        store8(out + 8ull * i, o);
+        put8(out + 8ull * i, o);
     }
 }
 
@@ -620,7 +913,7 @@ relu_bias_kernel(const bf16* out, const bf16* g, bf16* gpre, unsigned total, int
             const Oct o = load8(out + 8ull * i);
 #pragma unroll
             for (int k = 0; k < 8; ++k) x.v[k] = o.v[k] > 0.0f ? x.v[k] : 0.0f;
-            store8(gpre + 8ull * i, x);
+            put8(gpre + 8ull * i, x);
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) s.v[k] += x.v[k];
@@ -1202,7 +1495,7 @@ lbm_status forward(lbm_nn* nn, int n) {
             f.cin = c.cinp;
             f.cout = c.coutp;
             f.relu = c.relu;
-            e = launch_gemm(f, f.K(), 1, nn->gemm_err, s);
+            e = launch_conv(f, nn->sms, nn->gemm_err, s);
         } else if (op.k == lbm_nn::POOL) {
             const lbm_nn::Tensor& X = nn->t[op.a];
             const lbm_nn::Tensor& O = nn->t[op.out];
@@ -1302,7 +1595,7 @@ lbm_status backward(lbm_nn* nn, int n, float* loss) {
             wg.part = nn->part;
             wg.cin = c.cinp;
             wg.cout = c.coutp;
-            if ((e = launch_gemm(wg, kchunk, splits, nn->gemm_err, s)) != cudaSuccess) break;
+            if ((e = launch_gemm(wg, kchunk, splits, 0, nn->gemm_err, s)) != cudaSuccess) break;
             const long long nw = (long long)conv_wsize(c);
             split_sum_kernel<<<grid_of((nw + c.coutp + 64) * 8), kThreads, 0, s>>>(
                 nn->part, c.gw, splits, nw, nn->bpart, c.gb, bb, c.coutp);
@@ -1317,7 +1610,7 @@ lbm_status backward(lbm_nn* nn, int n, float* loss) {
                 dg.gin = G[c.in];
                 dg.cin = c.cinp;
                 dg.cout = c.coutp;
-                if ((e = launch_gemm(dg, dg.K(), 1, nn->gemm_err, s)) != cudaSuccess) break;
+                if ((e = launch_conv(dg, nn->sms, nn->gemm_err, s)) != cudaSuccess) break;
                 ++nn->launches;
             }
         } else if (op.k == lbm_nn::POOL) {
