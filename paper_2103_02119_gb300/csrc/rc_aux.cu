@@ -83,10 +83,10 @@ struct Tiles {
 // read-out kernels are bound by them, and by conversions, which take the same
 // lanes.  So they spend FP64 on what needs it and the rest on integers.
 // Measured on 2048 x 2047 FP32 cells with obstacles, against sums, conversions
-// and divisions in FP64: lbm_stress 558 against 2085 us, lbm_diagnostics after a
-// step 380 against 1260 us, lbm_get_f 84 against 146 us, lbm_set_f 91 against
+// and divisions in FP64: lbm_stress 516 against 2085 us (558 with the conversion
+// instruction for the sums), lbm_diagnostics after a step 335 against 1260 us (375), lbm_get_f 84 against 146 us, lbm_set_f 91 against
 // 143 us, lbm_moments 51 against 68 us; the residual check of a 96-lattice batch
-// 0.86 against 2.56 ms.
+// 0.80 against 2.56 ms (0.86).
 
 // float -> double, exact, on the integer pipe, without a branch (a conversion
 // instruction under a predicate takes its place in the FP64 pipe even where
@@ -166,11 +166,18 @@ __device__ __forceinline__ bool fixed_of(float f, long long& v) {
     if (m == 0u) v = 0;
     return m == 0u || (sh >= 0 && m < 0x40000000u);
 }
-// a nonzero integer multiple of 2^-kFixedShift as a double (one rounding)
+// an integer multiple of 2^-kFixedShift as a double (rounded to nearest even),
+// on the integer pipe: the conversion instruction takes FP64 lanes
 __device__ __forceinline__ double unfixed(long long v) {
-    const double d = __ll2double_rn(v);
-    const int hi = __double2hiint(d);
-    return __hiloint2double(v ? hi - (kFixedShift << 20) : 0, __double2loint(d));
+    const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = __clzll((long long)a);
+    const unsigned long long n = a << (lz & 63);  // leading bit at 63
+    // the 53 leading bits, the hidden one among them: it adds one to the exponent
+    unsigned long long m = n >> 11;
+    m += ((unsigned)n & 0x7FFu) + ((unsigned)m & 1u) > 0x400u ? 1u : 0u;
+    const unsigned e = (unsigned)(1023 + 63 - kFixedShift - 1 - lz) << 20;
+    const unsigned hi = ((unsigned)(m >> 32) + e) | ((unsigned)(v >> 32) & 0x80000000u);
+    return __hiloint2double(v ? (int)hi : 0, v ? (int)(unsigned)m : 0);
 }
 // fixed: d in the fixed point (valid when the result is true)
 __device__ __forceinline__ bool raw_sums(const float g[9], Raw& r, long long& fixed) {
