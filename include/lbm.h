@@ -135,9 +135,11 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
 /* Advance nsteps >= 0 time steps (collide + stream, Sec. 4), one kernel
  * launch per step; runs of 50 steps replay a CUDA graph the handle captures
  * once per starting buffer (on a stream of its own; lbm_set_force drops
- * it).  Small lattices run many steps per launch (lbm_set_small_path), large
- * FP32 ones (from 80,000 cells) two steps per launch but for the last one or
- * two of a call; the states are bit for bit the same.  Asynchronous: the
+ * it).  Small lattices run many steps per launch (lbm_set_small_path), and so
+ * do FP32 lattices below 200,000 cells in calls of at least 16 steps where a CTA's
+ * rows fit its shared memory (a cooperative launch of up to 1024 steps); larger
+ * FP32 ones (from 80,000 cells) take two steps per launch but for the last one
+ * or two of a call; the states are bit for bit the same.  Asynchronous: the
  * return value reports launch errors only. */
 lbm_status lbm_step(lbm_handle* h, int64_t nsteps);
 

@@ -64,6 +64,7 @@ struct lbm_handle {
     int diag_blocks = 0;
     int bx = 0, nbands = 0;
     int chain_bands = 0;       // bands of the two-step kernel (0: not used)
+    lbm::BandRun band;         // the many-step kernel of middle-sized lattices (ctas = 0: not used)
     int64_t steps = 0, launches = 0;
     uint8_t* bits = nullptr;   // small lattices: link bits of the nx * ny cells (device)
     bool small = false;        // steps run as one cluster launch (small_step.cu)
@@ -369,6 +370,9 @@ lbm_status device_inputs(lbm_handle* h, const double* const* in, int n, int on_d
 // Steps per captured graph of a single lattice (even, so a run starts and
 // ends on the same buffer).
 constexpr int kRunSteps = 50;
+// Shortest run of steps for the many-step kernel of middle-sized lattices, whose
+// launch reads and writes the state on top of its steps.
+constexpr int kBandSteps = 16;
 
 void drop_run_graphs(lbm_handle* h) {
     for (auto& g : h->graph)
@@ -429,6 +433,17 @@ lbm_status step_lattice(lbm_handle* h, int64_t nsteps) {
     }
     int64_t left = nsteps;
     if constexpr (sizeof(T) == 4) {
+        // many steps per launch
+        while (h->band.ctas && k.collide && left >= kBandSteps) {
+            const int n = left < kSmallRun ? (int)left : kSmallRun;
+            CK(h, lbm::launch_band_run((float*)h->f[0], (float*)h->f[1], k, h->cur, n, h->band,
+                                       h->stream),
+               "many-step kernel");
+            h->cur ^= n & 1;
+            h->launches += 1;
+            h->steps += n;
+            left -= n;
+        }
         // Two steps per launch; the last one or two are single steps, so that
         // the other buffer then holds the state one step earlier.
         while (h->chain_bands && k.collide && left >= 3) {
@@ -557,12 +572,27 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
     CKC(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
     h->diag_blocks = 2 * sms;
     CKC(lbm::dev_alloc(&h->part, sizeof(DiagPartial) * (h->diag_blocks + 1)), "cudaMalloc(diagnostics)");
-    CKC(lbm::dev_alloc(&h->status, sizeof(int)), "cudaMalloc(status)");
+    const bool f64 = p->precision == 64;
+    // Middle-sized FP32 lattices: many steps in one cooperative launch
+    // (band_run.cuh), wherever a band's rows fit a CTA's shared memory; us a step,
+    // that / the row-band or two-step kernel (calls of 61 steps, obstacles):
+    // 64 x 65 3.2 / 7.0, 100^2 3.8 / 6.4, 16 x 2000 3.2 / 20.6, 256^2 4.3 / 6.7,
+    // 100 x 1000 4.0 / 7.4, 300^2 5.3 / 8.3, 350^2 6.4 / 8.3.
+    if (!f64 && !kRowInterleaved && h->N > lbm::kSmallCells && h->N < 200000)
+        h->band = lbm::band_run_shape(p->nx, p->ny, sms);
+    // with the status word, in one allocation: its flags and mailboxes
+    const size_t flag_bytes = (size_t)h->band.ctas * 32 * sizeof(unsigned);
+    CKC(lbm::dev_alloc(&h->status, h->band.ctas ? 256 + flag_bytes + h->band.mail_bytes : sizeof(int)),
+        "cudaMalloc(status)");
+    if (h->band.ctas) {
+        unsigned char* q = reinterpret_cast<unsigned char*>(h->status) + 256;
+        h->band.flags = reinterpret_cast<unsigned*>(q);
+        h->band.mail = reinterpret_cast<float*>(q + flag_bytes);
+    }
     CKC(cudaMemsetAsync(h->status, 0, sizeof(int), h->stream), "cudaMemset");
 
     // Step kernel launch shape: one block per BX columns and per band of
     // rows, sized so that every block is resident at once (one wave).
-    const bool f64 = p->precision == 64;
     auto seg_width = [&](int b) {
         return f64 ? lbm::step_segment_width<double>(b) : lbm::step_segment_width<float>(b);
     };

@@ -56,6 +56,20 @@ inline bool chain2_takes(int nx, int ny, int pitch) {
 template <typename T>
 int step_occupancy(int bx, bool mask);
 
+// Middle-sized FP32 lattices: nsteps steps in one cooperative launch of a CTA
+// per band of rows (band_run.cuh), from buffer `from` (f0 or f1).
+constexpr int kBandThreads = 512;
+struct BandRun {
+    int ctas = 0, threads = 0;  // 0: the lattice cannot take it
+    // device buffers of the lattice:
+    size_t mail_bytes = 0;
+    float* mail = nullptr;      // mail_bytes
+    unsigned* flags = nullptr;  // 32 words a CTA
+};
+BandRun band_run_shape(int nx, int ny, int sms);
+cudaError_t launch_band_run(float* f0, float* f1, const KParams<float>& p, int from, int nsteps,
+                            const BandRun& b, cudaStream_t s);
+
 // Small lattices (at most kSmallCells cells): nsteps steps in one launch of
 // one thread-block cluster of min(ny, kSmallCluster) CTAs, from buffer
 // `from` (f0 or f1); bits: the link bits of the nx * ny cells (device).
