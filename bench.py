@@ -202,13 +202,17 @@ STEP_KERNEL_SOURCES = ("rc_step.cu", "rc_free_step.cu", "rnr_step.cu", "step_blo
                        "lbm_device.cuh")
 
 
-def step_kernel_hash(csrc=None):
+# the FP32 step's two-step kernel (large lattices)
+TWO_STEP_SOURCES = ("chain_step.cu", "chain_step.cuh", "lbm_device.cuh")
+
+
+def step_kernel_hash(csrc=None, sources=STEP_KERNEL_SOURCES):
     """Hash of the step kernels' code (comments and whitespace left out, so
     that only a change of the code itself invalidates recorded counters)."""
     import re
     csrc = csrc or os.path.join(ROOT, "paper_2103_02119_gb300", "csrc")
     h = hashlib.sha256()
-    for f in STEP_KERNEL_SOURCES:
+    for f in sources:
         with open(os.path.join(csrc, f)) as fh:
             code = fh.read()
         code = re.sub(r"/\*.*?\*/", " ", code, flags=re.S)
@@ -217,26 +221,27 @@ def step_kernel_hash(csrc=None):
     return h.hexdigest()[:16]
 
 
-def profiled(precision, key, mask=False):
+def profiled(precision, key, mask=False, two=False):
     """A per-cell figure of the committed ncu summary of the step kernel
-    (with a solid mask: its own entry), or None when the kernel has changed
-    since it was captured."""
+    (with a solid mask, and of the two-step kernel: their own entries), or
+    None when the kernel has changed since it was captured."""
     path = os.path.join(ROOT, "profiles", "rc_step_traffic.json")
     try:
         with open(path) as fh:
             d = json.load(fh)
     except (OSError, ValueError):
         return None
-    e = d.get(f"fp{precision}" + ("_mask" if mask else ""))
-    if not e or e.get("kernel_sha") != step_kernel_hash():
+    e = d.get(f"fp{precision}" + ("_mask" if mask else "") + ("_two_step" if two else ""))
+    sha = step_kernel_hash(sources=TWO_STEP_SOURCES) if two else step_kernel_hash()
+    if not e or e.get("kernel_sha") != sha:
         return None
     return e.get(key)
 
 
-def profiled_traffic(precision, cells, mask=False):
+def profiled_traffic(precision, cells, mask=False, two=False):
     """DRAM bytes per launch from the committed ncu summary, scaled to this
     grid, or None when the kernel has changed since it was captured."""
-    b = profiled(precision, "dram_bytes_per_cell", mask)
+    b = profiled(precision, "dram_bytes_per_cell", mask, two)
     return None if b is None else b * cells
 
 
@@ -736,17 +741,22 @@ def main():
     secs = max_over_ranks(secs, dist)
     cells = wl.cells
     value = world * cells * args.steps / secs / 1e6
-    per_launch = secs / args.steps
-    # a solid mask adds its link-mask byte to the algorithmic bytes
+    per_step = secs / args.steps
+    # A launch reads and writes the state once, whether it takes one step or
+    # two (large FP32 lattices; then mostly two); a solid mask adds its
+    # link-mask byte to the algorithmic bytes.
     bpc_main = BYTES_PER_CELL[args.precision] + (1 if args.mask else 0)
     algo_bytes = bpc_main * cells
+    two = launches < 0.75 * args.steps
     peak, peak_kind = measured_peaks()
-    achieved = algo_bytes / per_launch / 1e9
-    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak,
-                "traffic": profiled_traffic(args.precision, cells, args.mask),
+    achieved = algo_bytes * launches / secs / 1e9
+    kernel = "chain_kernel" if two else "rc_step_kernel"
+    roofline = {"bound": "fp32 issue" if two else "hbm", "achieved": achieved, "peak": peak,
+                "unit": "GB/s", "frac": achieved / peak,
+                "traffic": profiled_traffic(args.precision, cells, args.mask, two),
                 "peak_kind": peak_kind,
-                "kernel": f"rc_step_kernel<fp{args.precision}{', mask' if args.mask else ''}>",
+                "kernel": f"{kernel}<fp{args.precision}{', mask' if args.mask else ''}>",
+                "steps_per_launch": args.steps / launches,
                 "algorithmic_bytes_per_cell": bpc_main}
     e2e_res = None if args.no_e2e else e2e(lat, wl, torch, args.e2e_chunk, args.e2e_steps)
     peaks = None
@@ -792,15 +802,17 @@ def main():
         wm = with_obstacles(wl) if wl.mask is None else wl
         latm = Lattice.from_workload(wm, precision=args.precision, stream=stream)
         nm = max(100, args.steps // 10)
-        sm, _ = time_steps(latm, torch, nm, 10, barrier)
+        sm, lm = time_steps(latm, torch, nm, 10, barrier)
         latm.close()
         bpc = BYTES_PER_CELL[args.precision] + 1
-        am = bpc * cells / (sm / nm) / 1e9
+        am = bpc * cells * lm / sm / 1e9
+        two = lm < 0.75 * nm
         with_mask = {"value": cells * nm / sm / 1e6, "unit": "MLUPS", "steps": nm,
                      "solid_fraction": float(wm.mask.mean()),
-                     "roofline": {"bound": "hbm", "achieved": am, "peak": peak, "unit": "GB/s",
-                                  "frac": am / peak, "algorithmic_bytes_per_cell": bpc,
-                                  "traffic": profiled_traffic(args.precision, cells, True)}}
+                     "roofline": {"bound": "fp32 issue" if two else "hbm", "achieved": am,
+                                  "peak": peak, "unit": "GB/s", "frac": am / peak,
+                                  "steps_per_launch": nm / lm, "algorithmic_bytes_per_cell": bpc,
+                                  "traffic": profiled_traffic(args.precision, cells, True, two)}}
 
     batch = None
     if rank == 0 and not args.no_batch:
@@ -828,7 +840,7 @@ def main():
     if rank == 0:
         line = {
             "metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": world,
-            "steps": args.steps, "warmup": args.warmup, "ms_per_step": per_launch * 1e3,
+            "steps": args.steps, "warmup": args.warmup, "ms_per_step": per_step * 1e3,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
             "dtype": f"f{args.precision}", "data": "synthetic",
             "config": workload_config(args, wl), "roofline": roofline,
