@@ -301,6 +301,35 @@ template <typename T>
 KParams<T> kparams(const lbm_handle* h) { return kparams_of<T>(h->p, geometry(h)); }
 AuxParams aux(const lbm_handle* h) { return aux_of(h->p, geometry(h)); }
 
+// Bands of an FP64 lattice in blocks of one warp: the fewest microseconds by a
+// model fitted to 19 sizes (24 x 2816 to 1024 x 1024; 12 % rms, its choice
+// mostly within 8 % of the best shape measured): a block takes 12 us a
+// row alone on its SM, the SM's FP64 pipe 1.3 us per row of a warp; blocks that
+// are all resident end with the fullest SM, more of them even out but for the
+// last block.
+int short_bands(int nx, int ny, int width, int occupancy, int sms) {
+    const double nseg = (nx + width - 1) / width;
+    int best = ny;
+    double cost = 0.0;
+    for (int rows = 1; rows <= 32 && rows <= ny; ++rows) {
+        const int nb = (ny + rows / 2) / rows < 1 ? 1 : (ny + rows / 2) / rows;
+        const double per_sm = nseg * nb / sms, tall = (ny + nb - 1) / nb + 0.35;
+        const double march = 12.0 * tall;
+        double c;
+        if (per_sm <= occupancy) {
+            const double pipe = 1.3 * std::ceil(per_sm) * tall;
+            c = std::pow(std::pow(march, 2.2) + std::pow(pipe, 2.2), 1.0 / 2.2);
+        } else {
+            c = 1.3 * per_sm * ((double)ny / nb + 0.35) + 0.89 * march;
+        }
+        if (rows == 1 || c < cost) {
+            best = nb;
+            cost = c;
+        }
+    }
+    return best;
+}
+
 // Link mask of every cell (see lbm_device.cuh: bit i-1 = source of
 // direction i is a wall or solid node, 0xFF = solid cell).  Fluid cells
 // with no fluid neighbour become solid.  Returns the number of fluid cells.
@@ -596,11 +625,24 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
     auto seg_width = [&](int b) {
         return f64 ? lbm::step_segment_width<double>(b) : lbm::step_segment_width<float>(b);
     };
-    int bx = p->block_x;
+    int bx = p->block_x, nb = p->bands;
+    // Middle-sized FP64 lattices: many one-warp blocks of few rows, where the
+    // shapes below leave SMs with long marches or a second wave of few blocks;
+    // us a step, that / those: 192^2 24 / 29, 64 x 1000 33 / 99, 300^2 44 / 85,
+    // 300 x 700 87 / 171, 512^2 105 / 171, 600^2 142 / 158, 2000 x 200 150 / 171,
+    // 724^2 199 / 246, 850^2 274 / 308, 800 x 1300 365 / 445, 300 x 3000 354 / 530;
+    // but 1024 x 700 254 / 247, 1500 x 600 318 / 306, 1024^2 364 / 345 (not measured
+    // above 1.1 million cells).  A block per row and SM is already the shortest
+    // where there are no more rows: 128^2 23.1 / 20.8.
+    if (f64 && bx == 0 && nb == 0 && (h->N < 700000 || (h->N < 1100000 && p->nx < 900)) &&
+        (long long)((p->nx + seg_width(128) - 1) / seg_width(128)) * p->ny > sms) {
+        bx = 32;
+        nb = short_bands(p->nx, p->ny, seg_width(32),
+                         lbm::step_occupancy<double>(32, solid_mask != nullptr), sms);
+    }
     if (bx == 0) bx = p->nx <= seg_width(32) ? 32 : p->nx <= seg_width(64) ? 64 : 128;
     h->bx = bx;
     const int nseg = (p->nx + seg_width(bx) - 1) / seg_width(bx);
-    int nb = p->bands;
     if (nb == 0) {
         // Short bands (about 14 rows) keep the blocks that run at the same
         // time on nearby rows; enough of them to fill every SM, but bands of
