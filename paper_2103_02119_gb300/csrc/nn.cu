@@ -601,6 +601,10 @@ cudaError_t launch_umma_bn(const Op& op, long long kchunk, int splits, int* err,
 // and in narrower tiles where the tiles are few, 249 here; the 14 input gradients
 // 472, 342, 218.  What bounds it now is latency: a CTA's copies, nine taps and
 // read-out follow one another (9 to 29 us a convolution of 1.2 GFLOP).
+// (the copies are what the threads do: 256 of them take 729 us for a gradient pass
+// of 4 at 32 x 32 and 271 for a prediction at 64 x 64, 128 take 758 and 282; a pass of
+// 16 at 64 x 64 1,320 either way)
+constexpr int kConvThreads = 256;
 struct ConvTile {
     FastDiv fpitch, frows, fgroups;  // by w + 1, h + 1 and the channel groups
     unsigned positions;              // n (h + 1) (w + 1)
@@ -622,7 +626,7 @@ inline size_t conv_tile_smem(int pieces, int channels, int bn) {
 }
 
 template <class Op, int BN>
-__global__ void __launch_bounds__(kGemmThreads) conv_tile_kernel(const Op op, const ConvTile ct,
+__global__ void __launch_bounds__(kConvThreads) conv_tile_kernel(const Op op, const ConvTile ct,
                                                                  int* err) {
     constexpr int TC = tmem_cols<BN>();
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -654,7 +658,7 @@ __global__ void __launch_bounds__(kGemmThreads) conv_tile_kernel(const Op op, co
     {
         const bf16* in = op.pixels();
         const int total = (UM + 2 * ct.halo) * groups;
-        for (int v = tid; v < total; v += kGemmThreads) {
+        for (int v = tid; v < total; v += kConvThreads) {
             const int px = (int)ct.fgroups.div((unsigned)v), cg = v - px * groups;
             const long long p = pixel(m0 + (unsigned)px - (unsigned)ct.halo);
             cp16(a0 + cg * plane + px * 16, in + p * c + cg * 8, in, p >= 0);
@@ -663,7 +667,7 @@ __global__ void __launch_bounds__(kGemmThreads) conv_tile_kernel(const Op op, co
     const bf16* wt = op.weights();
 #pragma unroll
     for (int t = 0; t < 9; ++t) {
-        for (int v = tid; v < BN * groups; v += kGemmThreads) {
+        for (int v = tid; v < BN * groups; v += kConvThreads) {
             const int r = (int)ct.fgroups.div((unsigned)v), cg = v - r * groups;
             cp16(b0 + (t * groups + cg) * bplane + r * 16,
                  wt + (long long)(n0 + r) * 9 * c + t * c + cg * 8, wt, n0 + r < op.N());
@@ -710,9 +714,13 @@ __global__ void __launch_bounds__(kGemmThreads) conv_tile_kernel(const Op op, co
     cp_wait<0>(); tap(8);
     const bool ok = mbar_wait_parity(bar, 0);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const long long p = pixel(m0 + 32 * warp + lane);
+    // a warp reads the 32 rows of its place in its group of four, the second
+    // group of warps the upper half of the columns
+    constexpr int kCols = BN >= 32 ? BN / 2 : BN;
+    const int quarter = warp & 3, cbeg = (warp >> 2) * kCols;
+    const long long p = pixel(m0 + 32 * quarter + lane);
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 16) {
+    for (int c0 = cbeg; c0 < cbeg + kCols && c0 < BN; c0 += 16) {
         uint32_t r[16];
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,"
@@ -720,7 +728,7 @@ __global__ void __launch_bounds__(kGemmThreads) conv_tile_kernel(const Op op, co
             : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
               "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
               "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-            : "r"(taddr + ((unsigned)(32 * warp) << 16) + (unsigned)c0));
+            : "r"(taddr + ((unsigned)(32 * quarter) << 16) + (unsigned)c0));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         float v[16];
 #pragma unroll
@@ -750,7 +758,7 @@ cudaError_t launch_conv_bn(const Op& op, const ConvTile& t, int* err, cudaStream
     }
     const dim3 grid((t.positions + UM - 1) / UM, (op.N() + BN - 1) / BN);
     conv_tile_kernel<Op, BN>
-        <<<grid, kGemmThreads, conv_tile_smem(t.pieces, op.channels(), BN), s>>>(op, t, err);
+        <<<grid, kConvThreads, conv_tile_smem(t.pieces, op.channels(), BN), s>>>(op, t, err);
     return cudaGetLastError();
 }
 
