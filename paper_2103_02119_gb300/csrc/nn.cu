@@ -1221,15 +1221,32 @@ __global__ void weight_copies_kernel(const float* wm, bf16* wf, bf16* wd, int ci
     }
 }
 
-// The host's parameter order (dy, dx, cin, cout, then the biases) from or to a
-// convolution's device arrays w [coutp][9][cinp], b [coutp].  A block moves a
+// The host's parameter order (dy, dx, cin, cout, then the biases) from or to the
+// convolutions' device arrays w [coutp][9][cinp], b [coutp].  A block moves a
 // tile of 32 input by 32 output channels of one tap through shared memory, so
-// that both sides are read and written in rows.
+// that both sides are read and written in rows; all convolutions in one launch
+// (one launch each took 75 us more of a gradient pass of 16 at 64 x 64, now 1,250).
+constexpr int kMaxConvs = 23;  // of six levels
+struct ParamTable {
+    struct Entry {
+        float *w, *b;
+        long long at;               // in the host's order
+        int cin, cout, cinp, first; // first: its first block
+    } e[kMaxConvs];
+    int n;
+};
 template <bool TO_HOST>
 __global__ void __launch_bounds__(kThreads)
-param_order_kernel(float* host, float* w, float* b, int cin, int cout, int cinp) {
+param_order_kernel(float* vec, const __grid_constant__ ParamTable table) {
     __shared__ float t[32][33];
-    const int tap = blockIdx.z, ci0 = blockIdx.y * 32, co0 = blockIdx.x * 32;
+    int k = 0;
+    while (k + 1 < table.n && table.e[k + 1].first <= (int)blockIdx.x) ++k;
+    const ParamTable::Entry& c = table.e[k];
+    float* const host = vec + c.at;
+    float *const w = c.w, *const b = c.b;
+    const int cin = c.cin, cout = c.cout, cinp = c.cinp;
+    const int tx = (cout + 31) / 32, ty = (cin + 31) / 32, local = (int)blockIdx.x - c.first;
+    const int tap = local / (tx * ty), ci0 = local / tx % ty * 32, co0 = local % tx * 32;
     const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
     for (int r = y; r < 32; r += kThreads / 32) {
         if (TO_HOST) {  // rows of the device array: ci across
@@ -1250,11 +1267,11 @@ param_order_kernel(float* host, float* w, float* b, int cin, int cout, int cinp)
             if (co < cout && ci < cin) w[((long long)co * 9 + tap) * cinp + ci] = t[r][x];
         }
     }
-    if (tap == 0 && blockIdx.y == 0)
-        for (int k = threadIdx.x; k < 32 && co0 + k < cout; k += kThreads) {
-            float* hb = host + 9ll * cin * cout + co0 + k;
-            if (TO_HOST) *hb = b[co0 + k];
-            else b[co0 + k] = *hb;
+    if (tap == 0 && ci0 == 0)
+        for (int i = threadIdx.x; i < 32 && co0 + i < cout; i += kThreads) {
+            float* hb = host + 9ll * cin * cout + co0 + i;
+            if (TO_HOST) *hb = b[co0 + i];
+            else b[co0 + i] = *hb;
         }
 }
 
@@ -1906,19 +1923,19 @@ static lbm_status transfer_params(lbm_nn* nn, float* host, bool to_device, bool 
     if (to_device)
         NCK(nn, cudaMemcpyAsync(nn->flat, host, bytes, cudaMemcpyHostToDevice, nn->stream),
             "cudaMemcpyAsync(H2D)");
-    float* q = nn->flat;
+    ParamTable table;
+    table.n = 0;
+    long long at = 0;
+    int blocks = 0;
     for (auto& c : nn->conv) {
-        float* w = grads ? c.gw : c.wm;
-        float* b = grads ? c.gb : c.bm;
-        const dim3 g((c.cout + 31) / 32, (c.cin + 31) / 32, 9);
-        if (to_device)
-            param_order_kernel<false><<<g, kThreads, 0, nn->stream>>>(q, w, b, c.cin, c.cout, c.cinp);
-        else
-            param_order_kernel<true><<<g, kThreads, 0, nn->stream>>>(q, w, b, c.cin, c.cout, c.cinp);
-        NCK(nn, cudaGetLastError(), "parameter order");
-        ++nn->launches;
-        q += 9ull * c.cin * c.cout + c.cout;
+        table.e[table.n++] = {grads ? c.gw : c.wm, grads ? c.gb : c.bm, at, c.cin, c.cout, c.cinp, blocks};
+        at += 9ll * c.cin * c.cout + c.cout;
+        blocks += (c.cout + 31) / 32 * ((c.cin + 31) / 32) * 9;
     }
+    if (to_device) param_order_kernel<false><<<blocks, kThreads, 0, nn->stream>>>(nn->flat, table);
+    else param_order_kernel<true><<<blocks, kThreads, 0, nn->stream>>>(nn->flat, table);
+    NCK(nn, cudaGetLastError(), "parameter order");
+    ++nn->launches;
     if (!to_device)
         NCK(nn, cudaMemcpyAsync(host, nn->flat, bytes, cudaMemcpyDeviceToHost, nn->stream),
             "cudaMemcpyAsync(D2H)");
