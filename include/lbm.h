@@ -136,8 +136,9 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
  * launch per step; runs of 50 steps replay a CUDA graph the handle captures
  * once per starting buffer (on a stream of its own; lbm_set_force drops
  * it).  Small lattices run many steps per launch (lbm_set_small_path), and so
- * do FP32 lattices below 200,000 cells in calls of at least 16 steps where a CTA's
- * rows fit its shared memory (a cooperative launch of up to 1024 steps); larger
+ * do FP32 lattices below 200,000 cells in calls of at least 3 steps (14 up to
+ * 20,480 cells) where a CTA's rows fit its shared memory (a cooperative launch of
+ * up to 1024 steps); larger
  * FP32 ones (from 80,000 cells) take two steps per launch but for the last one
  * or two of a call; the states are bit for bit the same.  Asynchronous: the
  * return value reports launch errors only. */

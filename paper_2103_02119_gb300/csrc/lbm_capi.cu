@@ -399,9 +399,14 @@ lbm_status device_inputs(lbm_handle* h, const double* const* in, int n, int on_d
 // Steps per captured graph of a single lattice (even, so a run starts and
 // ends on the same buffer).
 constexpr int kRunSteps = 50;
-// Shortest run of steps for the many-step kernel of middle-sized lattices, whose
-// launch reads and writes the state on top of its steps.
-constexpr int kBandSteps = 16;
+// Shortest run of steps for the many-step kernel of middle-sized lattices.  Its
+// launch reads and writes the state on top of its steps; us of a call, that /
+// a launch per step: 256 x 256 2 steps 15.5 / 16.5, 3 steps 19.5 / 24.7, 8 steps
+// 40 / 66; 350 x 350 3 steps 27.8 / 26.7, 4 steps 33.9 / 37.0; 16 x 2000 3 steps
+// 15.5 / 64.6.  Up to 20,480 cells a call of fewer than 14 steps stays a launch
+// per step, as its callers count them (100 x 100, 8 steps: 35 / 66).
+constexpr int kBandSteps = 3, kBandStepsFew = 14;
+constexpr long long kBandFewCells = 20480;
 
 void drop_run_graphs(lbm_handle* h) {
     for (auto& g : h->graph)
@@ -463,7 +468,8 @@ lbm_status step_lattice(lbm_handle* h, int64_t nsteps) {
     int64_t left = nsteps;
     if constexpr (sizeof(T) == 4) {
         // many steps per launch
-        while (h->band.ctas && k.collide && left >= kBandSteps) {
+        while (h->band.ctas && k.collide &&
+               left >= (h->N > kBandFewCells ? kBandSteps : kBandStepsFew)) {
             const int n = left < kSmallRun ? (int)left : kSmallRun;
             CK(h, lbm::launch_band_run((float*)h->f[0], (float*)h->f[1], k, h->cur, n, h->band,
                                        h->stream),
