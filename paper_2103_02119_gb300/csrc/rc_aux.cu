@@ -83,10 +83,11 @@ struct Tiles {
 // read-out kernels are bound by them, and by conversions, which take the same
 // lanes.  So they spend FP64 on what needs it and the rest on integers.
 // Measured on 2048 x 2047 FP32 cells with obstacles, against sums, conversions
-// and divisions in FP64: lbm_stress 516 against 2085 us (558 with the conversion
-// instruction for the sums), lbm_diagnostics after a step 335 against 1260 us (375), lbm_get_f 84 against 146 us, lbm_set_f 91 against
-// 143 us, lbm_moments 51 against 68 us; the residual check of a 96-lattice batch
-// 0.80 against 2.56 ms (0.86).
+// and divisions in FP64: lbm_stress 455 against 2085 us (558 with the conversion
+// instruction for the sums, 516 with ten FP64 operations more in its algebra),
+// lbm_diagnostics after a step 335 against 1260 us (375), lbm_get_f 84 against 146 us,
+// lbm_set_f 91 against 143 us, lbm_moments 51 against 68 us; the residual check of a
+// 96-lattice batch 0.80 against 2.56 ms (0.86).
 
 // float -> double, exact, on the integer pipe, without a branch (a conversion
 // instruction under a predicate takes its place in the FP64 pipe even where
@@ -520,7 +521,10 @@ density_kernel(const T* __restrict__ f, const AuxParams p, double* __restrict__ 
 // reciprocals and products in place of the five divisions, and the constants
 // from the host.
 struct StressConst {
-    double a, a2, cs2, nu4, nu5, zeta, b1c, b2c, c1c, c2c, g1, g2, e5, hFx, hFy;
+    double a, a2, cs2, g1, g2, hFx, hFy;
+    double bc, cb, d, v, dv;  // (b1 + c1)/2, (c2 - b2)/2, (b1 - c1)/2, (b2 + c2)/2, d v
+    double e5, k5;            // xy strain rate and stress over the xy moment
+    double sp, sm;            // bulk plus and minus shear viscosity
 };
 template <typename T, bool MASK>
 __global__ void __launch_bounds__(kThreads)
@@ -533,7 +537,7 @@ stress_kernel(const T* __restrict__ f, const AuxParams p, const StressConst q,
         if (x >= p.nx || y >= p.ny) continue;
         const long long row = (long long)y * p.nx, c = row + x;
         const unsigned sb = link_bits<MASK>(p, x, y);
-        double e_xx = 0.0, e_yy = 0.0, e_xy = 0.0, s_m = 0.0, s_d = 0.0, s_xy = 0.0;
+        double e_xx = 0.0, e_yy = 0.0, e_xy = 0.0, s_xx = 0.0, s_yy = 0.0, s_xy = 0.0;
         if (sb != 0xFFu) {
             T g[9];
             pull(f, p, x, y, sb, g);
@@ -551,31 +555,33 @@ stress_kernel(const T* __restrict__ f, const AuxParams p, const StressConst q,
             const double ir = rcp64_ok(r) ? rcp64(r) : 1.0 / r;
             const double jx = s.jx + q.hFx, jy = fma(q.a, s.jy, q.hFy);
             const double ux = jx * ir, uy = jy * ir;
-            // non-equilibrium second-order moments m - m^eq
-            const double ux2 = ux * ux, uy2 = uy * uy;
+            // non-equilibrium second-order moments m - m^eq, and the gradient terms
             const double n20 = fma(-jx, ux, fma(-q.cs2, s.d, s.sxx));
             const double n02 = fma(-jy, uy, fma(-q.cs2, s.d, q.a2 * s.syy));
             const double n11 = fma(-jx, uy, q.a * s.sxy);
-            const double gx = q.g1 * ux * (rE - rW), gy = q.g2 * uy * (rN - rS);
-            const double m20 = n20 + gx, m02 = n02 + gy;
-            const double R3 = m20 + m02, R4 = m20 - m02;
-            const double B1 = fma(1.5, ux2, q.b1c), B2 = fma(1.5, uy2, q.b2c);
-            const double C1 = fma(1.5, ux2, q.c1c), C2 = fma(-1.5, uy2, q.c2c);
-            const double det = fma(B1, C2, -(B2 * C1));
-            const double id = (rcp64_ok(det) ? rcp64(det) : 1.0 / det) * ir;
-            e_xx = fma(C2, R3, -(B2 * R4)) * id;
-            e_yy = fma(B1, R4, -(C1 * R3)) * id;
-            const double e11 = q.e5 * n11;
-            s_xy = q.nu5 * e11;
-            e_xy = e11 * ir;
-            s_m = r * (q.zeta * (e_xx + e_yy));
-            s_d = r * (q.nu4 * (e_xx - e_yy));
+            const double m20 = fma(q.g1 * ux, rE - rW, n20), m02 = fma(q.g2 * uy, rN - rS, n02);
+            // With B1 = 3/2 ux^2 + b1, C1 = 3/2 ux^2 + c1, B2 = 3/2 uy^2 + b2, C2 = c2 -
+            // 3/2 uy^2, the strain rates are
+            //   rho dx ux = (C2 R3 - B2 R4) / det, rho dy uy = (B1 R4 - C1 R3) / det,
+            //   R3 = m20 + m02, R4 = m20 - m02, det = B1 C2 - B2 C1;
+            // in halves of sums and differences of the coefficients the products
+            // that cancel are gone (8 of 22 FP64 operations).
+            const double P = fma(1.5, ux * ux, q.bc), Q = fma(-1.5, uy * uy, q.cb);
+            const double det = fma(P, Q, q.dv);
+            const double id = rcp64_ok(det) ? rcp64(det) : 1.0 / det;
+            const double rxx = fma(Q, m20, q.v * m02) * id, ryy = fma(q.d, m20, -(P * m02)) * id;
+            e_xx = rxx * ir;
+            e_yy = ryy * ir;
+            e_xy = q.e5 * n11 * ir;
+            s_xx = fma(q.sp, rxx, q.sm * ryy);
+            s_yy = fma(q.sm, rxx, q.sp * ryy);
+            s_xy = q.k5 * n11;
         }
         if (dxux) dxux[c] = e_xx;
         if (dyuy) dyuy[c] = e_yy;
         if (sxy) sxy[c] = e_xy;
-        if (txx) txx[c] = s_m + s_d;
-        if (tyy) tyy[c] = s_m - s_d;
+        if (txx) txx[c] = s_xx;
+        if (tyy) tyy[c] = s_yy;
         if (txy) txy[c] = s_xy;
     }
 }
@@ -956,16 +962,23 @@ cudaError_t launch_stress(const T* f, const AuxParams& p, const double* rho, dou
     q.a = p.a;
     q.a2 = a2;
     q.cs2 = c;
-    q.nu4 = c * (1.0 / p.w4 - 0.5);
-    q.nu5 = c * (1.0 / p.w5 - 0.5);
-    q.zeta = c * (1.0 / p.w3 - 0.5);
-    q.b1c = -2.0 * c / p.w3 - 0.5 * (1.0 - 3.0 * c);
-    q.b2c = -2.0 * c / p.w3 - 0.5 * (a2 - 3.0 * c);
-    q.c1c = -2.0 * c / p.w4 - 0.5 * (1.0 - 3.0 * c);
-    q.c2c = 2.0 * c / p.w4 + 0.5 * (a2 - 3.0 * c);
+    const double nu4 = c * (1.0 / p.w4 - 0.5), nu5 = c * (1.0 / p.w5 - 0.5),
+                 zeta = c * (1.0 / p.w3 - 0.5);
+    const double b1 = -2.0 * c / p.w3 - 0.5 * (1.0 - 3.0 * c);
+    const double b2 = -2.0 * c / p.w3 - 0.5 * (a2 - 3.0 * c);
+    const double c1 = -2.0 * c / p.w4 - 0.5 * (1.0 - 3.0 * c);
+    const double c2 = 2.0 * c / p.w4 + 0.5 * (a2 - 3.0 * c);
+    q.bc = 0.5 * (b1 + c1);
+    q.cb = 0.5 * (c2 - b2);
+    q.d = 0.5 * (b1 - c1);
+    q.v = 0.5 * (b2 + c2);
+    q.dv = q.d * q.v;
     q.g1 = 0.25 * (1.0 - 3.0 * c);           // with the spacing 2 of the differences
     q.g2 = 0.25 * (a2 - 3.0 * c) / p.a;      // and 2a
     q.e5 = -p.w5 / c;
+    q.k5 = nu5 * q.e5;
+    q.sp = zeta + nu4;
+    q.sm = zeta - nu4;
     q.hFx = 0.5 * p.Fx;
     q.hFy = 0.5 * p.Fy;
     if (p.lmask)
