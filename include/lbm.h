@@ -242,7 +242,10 @@ lbm_status lbm_set_f(lbm_handle* h, const double* f, int on_device);
  *          conserves momentum): motion along them alternates every step and
  *          never decays, a residual between states an even number of steps
  *          apart is blind to it, and the two-step mean cancels it
- *   out[5] number of fluid cells with a non-finite rho or u
+ *   out[5] number of fluid cells with a non-finite rho or u, or with a stored
+ *          value (f_i - w_i rho0) of 32 or more in magnitude, where the exact
+ *          mass sum ends: a flow that holds one has long left the range of the
+ *          scheme.  Such cells stay out of out[1] .. out[4] and out[7]
  *   out[6] step counter n
  *   out[7] step-to-step change sqrt(sum |u(n) - u(n-1)|^2) / sqrt(sum
  *          |ubar(n)|^2), which such alternating motion keeps away from zero;

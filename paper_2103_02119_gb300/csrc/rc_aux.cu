@@ -587,7 +587,8 @@ stress_kernel(const T* __restrict__ f, const AuxParams p, const StressConst q,
 }
 
 // Adds v exactly (down to 2^-kMassShift) to a fixed-point number held as
-// 24-bit limbs.  Returns false when v is too large for the accumulator.
+// 24-bit limbs.  Returns false when v is too large for the accumulator (32 or more
+// in magnitude) or not finite.
 __device__ __forceinline__ bool add_fixed(long long limb[kMassLimbs], double v) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
     const int E = (int)((bits >> 52) & 0x7FF);
@@ -636,8 +637,9 @@ __device__ __forceinline__ bool add_mass(__int128& acc, long long limb[kMassLimb
     for (int i = 0; i < 9; ++i) ok &= add_fixed(limb, (double)g[i]);
     return ok;
 }
-// FP64 storage: each deviation in units of 2^-100, where it is zero or
-// between 2^-47 and 2^6 in magnitude (below 2^19 values a thread: < 2^125).
+// FP64 storage: each deviation in units of 2^-100, where it is between 2^-48 and
+// 2^5 in magnitude, which is also where add_fixed ends (a cell with a larger one
+// stays out of every sum); below 2^19 values a thread: < 2^124.
 __device__ __forceinline__ bool add_mass(__int128& acc, long long limb[kMassLimbs],
                                          const double g[9], bool, long long) {
     bool ok = true;
@@ -645,7 +647,7 @@ __device__ __forceinline__ bool add_mass(__int128& acc, long long limb[kMassLimb
     for (int i = 0; i < 9; ++i) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(g[i]);
         const int sh = (int)((b >> 52) & 0x7FF) - 975;  // exponent - 1075 + 100
-        if (sh >= 0 && sh < 1029 - 975) {
+        if (sh >= 0 && sh < 1028 - 975) {
             const __int128 v = (__int128)((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << sh;
             acc += (long long)b < 0 ? -v : v;
         } else {
