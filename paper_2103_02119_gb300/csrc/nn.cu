@@ -1028,16 +1028,17 @@ __global__ void out_smooth_kernel(const void* in, int icp, FL fluid, void* out, 
     }
 }
 
-// Block (j, k): sums over part j of the fluid cells of instance k of (-1)^x v1,
+// Block (k, j): sums over part j of the fluid cells of instance k of (-1)^x v1,
 // (-1)^y v2 and the cell count, in a fixed order, to sums[k][j][3].  (One block
-// per instance took 26 us for 16 instances of 64 x 64.)
+// per instance took 26 us for 16 instances of 64 x 64.  Instances go along x: a
+// batch may hold more of them than the 65,535 of a grid's y.)
 constexpr int kStaggerParts = 16;
 template <typename FL>
 __global__ void __launch_bounds__(kThreads) stagger_sum_kernel(const float* v, FL fluid,
                                                                double* sums, int h, int w) {
-    const long long hw = (long long)h * w, p0 = (long long)blockIdx.y * hw;
+    const long long hw = (long long)h * w, p0 = (long long)blockIdx.x * hw;
     double s1 = 0.0, s2 = 0.0, nf = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < hw;
+    for (long long i = blockIdx.y * (long long)blockDim.x + threadIdx.x; i < hw;
          i += kStaggerParts * (long long)blockDim.x) {
         const long long p = p0 + i;
         if (!fluid(p)) continue;
@@ -1050,22 +1051,22 @@ __global__ void __launch_bounds__(kThreads) stagger_sum_kernel(const float* v, F
     s2 = block_sum(s2);
     nf = block_sum(nf);
     if (threadIdx.x == 0) {
-        double* o = sums + 3 * ((long long)blockIdx.y * kStaggerParts + blockIdx.x);
+        double* o = sums + 3 * ((long long)blockIdx.x * kStaggerParts + blockIdx.y);
         o[0] = s1;
         o[1] = s2;
         o[2] = nf;
     }
 }
 
-// Block (j, k) applies the projection to part j of instance k.
+// Block (k, j) applies the projection to part j of instance k.
 template <typename FL>
 __global__ void __launch_bounds__(kThreads)
 stagger_apply_kernel(const float* v, FL fluid, const double* sums, float* out, int h, int w) {
     __shared__ float c[2];
     __shared__ int any;
-    const long long hw = (long long)h * w, p0 = (long long)blockIdx.y * hw;
+    const long long hw = (long long)h * w, p0 = (long long)blockIdx.x * hw;
     if (threadIdx.x == 0) {
-        const double* q = sums + 3 * (long long)blockIdx.y * kStaggerParts;
+        const double* q = sums + 3 * (long long)blockIdx.x * kStaggerParts;
         double s1 = 0.0, s2 = 0.0, nf = 0.0;
         for (int j = 0; j < kStaggerParts; ++j) {
             s1 += q[3 * j];
@@ -1077,8 +1078,8 @@ stagger_apply_kernel(const float* v, FL fluid, const double* sums, float* out, i
         c[1] = nf > 0.0 ? (float)(s2 / nf) : 0.0f;
     }
     __syncthreads();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < hw;
-         i += gridDim.x * (long long)blockDim.x) {
+    for (long long i = blockIdx.y * (long long)blockDim.x + threadIdx.x; i < hw;
+         i += kStaggerParts * (long long)blockDim.x) {
         const long long p = p0 + i;
         const unsigned y = (unsigned)i / (unsigned)w, x = (unsigned)i - y * (unsigned)w;
         float o1 = v[p * 3 + 1], o2 = v[p * 3 + 2];
@@ -1497,7 +1498,7 @@ void wgrad_splits(const lbm_nn* nn, const lbm_nn::Conv& c, long long P, int& spl
 lbm_status unstagger(lbm_nn* nn, int n, const float* v, float* out) {
     const lbm_nn::Tensor& X = nn->t[nn->x_id];
     const FluidIn fl{X.v, X.cp};
-    const dim3 g(kStaggerParts, n);
+    const dim3 g(n, kStaggerParts);
     stagger_sum_kernel<<<g, kThreads, 0, nn->stream>>>(v, fl, nn->ssum, X.h, X.w);
     NCK(nn, cudaGetLastError(), "staggered sums");
     stagger_apply_kernel<<<g, kThreads, 0, nn->stream>>>(v, fl, nn->ssum, out, X.h, X.w);
@@ -2020,7 +2021,7 @@ lbm_status lbm_nn_prolong(lbm_nn* nn, const float* y, int n, int factor, const u
     NCK(nn, cudaGetLastError(), "prolongation");
     out_smooth_kernel<false, false><<<grid_of(P), kThreads, 0, s>>>(f0, 3, fl, f1, 3, n, H, W);
     NCK(nn, cudaGetLastError(), "output smoothing (fine)");
-    const dim3 parts(kStaggerParts, n);
+    const dim3 parts(n, kStaggerParts);
     stagger_sum_kernel<<<parts, kThreads, 0, s>>>(f1, fl, nn->ssum, H, W);
     NCK(nn, cudaGetLastError(), "staggered sums (fine)");
     stagger_apply_kernel<<<parts, kThreads, 0, s>>>(f1, fl, nn->ssum, f0, H, W);
