@@ -1028,18 +1028,53 @@ __global__ void out_smooth_kernel(const void* in, int icp, FL fluid, void* out, 
     }
 }
 
-// Block (k, j): sums over part j of the fluid cells of instance k of (-1)^x v1,
-// (-1)^y v2 and the cell count, in a fixed order, to sums[k][j][3].  (One block
-// per instance took 26 us for 16 instances of 64 x 64.  Instances go along x: a
-// batch may hold more of them than the 65,535 of a grid's y.)
+// How the cells of an instance are shared out: 2^lg threads, as many as it has cells
+// and a block at most, and parts of kThreads cells, up to 16, for a block each.
+// Block (k, j) takes part j of the instances whose threads fit a block, from k
+// kThreads / 2^lg on.  (One block per instance took 26 us for 16 instances of
+// 64 x 64; 16 parts of every instance cost a batch of 300 of 8 x 8 50 us a pass.
+// Instances go along x: a batch may hold more than the 65,535 of a grid's y.)
 constexpr int kStaggerParts = 16;
+struct Stagger {
+    int n, lg, parts;
+    Stagger(int n_, long long cells) : n(n_), lg(0) {
+        while ((1 << lg) < kThreads && (1 << lg) < cells) ++lg;
+        const long long p = (cells + kThreads - 1) / kThreads;
+        parts = p < kStaggerParts ? (int)p : kStaggerParts;
+    }
+    dim3 grid() const {
+        const int each = kThreads >> lg;
+        return dim3((unsigned)(((long long)n + each - 1) / each), parts);
+    }
+};
+// v summed over each group of 2^lg threads, valid in its first one: over warps
+// by shuffles, then in order
+template <typename V>
+__device__ __forceinline__ V group_sum(V v, int lg) {
+    __shared__ V sh[kThreads / 32];
+    const int width = lg < 5 ? 1 << lg : 32;
+    for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o, width);
+    if (lg <= 5) return v;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    V s = V(0);
+    if ((threadIdx.x & ((1 << lg) - 1)) == 0)
+        for (int i = 0; i < 1 << (lg - 5); ++i) s += sh[(threadIdx.x >> 5) + i];
+    return s;
+}
+
+// Sums over part j of the fluid cells of instance k of (-1)^x v1, (-1)^y v2 and
+// the cell count, in a fixed order, to sums[k][j][3].
 template <typename FL>
-__global__ void __launch_bounds__(kThreads) stagger_sum_kernel(const float* v, FL fluid,
-                                                               double* sums, int h, int w) {
-    const long long hw = (long long)h * w, p0 = (long long)blockIdx.x * hw;
+__global__ void __launch_bounds__(kThreads)
+stagger_sum_kernel(const float* v, FL fluid, double* sums, int h, int w, const Stagger g) {
+    const int lane = threadIdx.x & ((1 << g.lg) - 1);
+    const int k = blockIdx.x * (kThreads >> g.lg) + (threadIdx.x >> g.lg);
+    const long long hw = (long long)h * w, p0 = k * hw;
     double s1 = 0.0, s2 = 0.0, nf = 0.0;
-    for (long long i = blockIdx.y * (long long)blockDim.x + threadIdx.x; i < hw;
-         i += kStaggerParts * (long long)blockDim.x) {
+    for (long long i = ((long long)blockIdx.y << g.lg) + lane; k < g.n && i < hw;
+         i += (long long)g.parts << g.lg) {
         const long long p = p0 + i;
         if (!fluid(p)) continue;
         const unsigned y = (unsigned)i / (unsigned)w, x = (unsigned)i - y * (unsigned)w;
@@ -1047,45 +1082,47 @@ __global__ void __launch_bounds__(kThreads) stagger_sum_kernel(const float* v, F
         s2 += (y & 1) ? -(double)v[p * 3 + 2] : (double)v[p * 3 + 2];
         nf += 1.0;
     }
-    s1 = block_sum(s1);
-    s2 = block_sum(s2);
-    nf = block_sum(nf);
-    if (threadIdx.x == 0) {
-        double* o = sums + 3 * ((long long)blockIdx.x * kStaggerParts + blockIdx.y);
+    s1 = group_sum(s1, g.lg);
+    s2 = group_sum(s2, g.lg);
+    nf = group_sum(nf, g.lg);
+    if (lane == 0 && k < g.n) {
+        double* o = sums + 3 * ((long long)k * g.parts + blockIdx.y);
         o[0] = s1;
         o[1] = s2;
         o[2] = nf;
     }
 }
 
-// Block (k, j) applies the projection to part j of instance k.
+// Applies the projection to part j of instance k.
 template <typename FL>
 __global__ void __launch_bounds__(kThreads)
-stagger_apply_kernel(const float* v, FL fluid, const double* sums, float* out, int h, int w) {
-    __shared__ float c[2];
-    __shared__ int any;
-    const long long hw = (long long)h * w, p0 = (long long)blockIdx.x * hw;
-    if (threadIdx.x == 0) {
-        const double* q = sums + 3 * (long long)blockIdx.x * kStaggerParts;
+stagger_apply_kernel(const float* v, FL fluid, const double* sums, float* out, int h, int w,
+                     const Stagger g) {
+    __shared__ float c[kThreads][2];
+    const int lane = threadIdx.x & ((1 << g.lg) - 1), sub = threadIdx.x >> g.lg;
+    const int k = blockIdx.x * (kThreads >> g.lg) + sub;
+    const long long hw = (long long)h * w, p0 = k * hw;
+    if (lane == 0 && k < g.n) {
+        const double* q = sums + 3 * (long long)k * g.parts;
         double s1 = 0.0, s2 = 0.0, nf = 0.0;
-        for (int j = 0; j < kStaggerParts; ++j) {
+        for (int j = 0; j < g.parts; ++j) {
             s1 += q[3 * j];
             s2 += q[3 * j + 1];
             nf += q[3 * j + 2];
         }
-        any = nf > 0.0;
-        c[0] = nf > 0.0 ? (float)(s1 / nf) : 0.0f;
-        c[1] = nf > 0.0 ? (float)(s2 / nf) : 0.0f;
+        // (without fluid cells nothing below uses them)
+        c[sub][0] = nf > 0.0 ? (float)(s1 / nf) : 0.0f;
+        c[sub][1] = nf > 0.0 ? (float)(s2 / nf) : 0.0f;
     }
     __syncthreads();
-    for (long long i = blockIdx.y * (long long)blockDim.x + threadIdx.x; i < hw;
-         i += kStaggerParts * (long long)blockDim.x) {
+    for (long long i = ((long long)blockIdx.y << g.lg) + lane; k < g.n && i < hw;
+         i += (long long)g.parts << g.lg) {
         const long long p = p0 + i;
         const unsigned y = (unsigned)i / (unsigned)w, x = (unsigned)i - y * (unsigned)w;
         float o1 = v[p * 3 + 1], o2 = v[p * 3 + 2];
-        if (any && fluid(p)) {
-            o1 -= (x & 1) ? -c[0] : c[0];
-            o2 -= (y & 1) ? -c[1] : c[1];
+        if (fluid(p)) {
+            o1 -= (x & 1) ? -c[sub][0] : c[sub][0];
+            o2 -= (y & 1) ? -c[sub][1] : c[sub][1];
         }
         out[p * 3] = v[p * 3];
         out[p * 3 + 1] = o1;
@@ -1498,10 +1535,10 @@ void wgrad_splits(const lbm_nn* nn, const lbm_nn::Conv& c, long long P, int& spl
 lbm_status unstagger(lbm_nn* nn, int n, const float* v, float* out) {
     const lbm_nn::Tensor& X = nn->t[nn->x_id];
     const FluidIn fl{X.v, X.cp};
-    const dim3 g(n, kStaggerParts);
-    stagger_sum_kernel<<<g, kThreads, 0, nn->stream>>>(v, fl, nn->ssum, X.h, X.w);
+    const Stagger g(n, (long long)X.h * X.w);
+    stagger_sum_kernel<<<g.grid(), kThreads, 0, nn->stream>>>(v, fl, nn->ssum, X.h, X.w, g);
     NCK(nn, cudaGetLastError(), "staggered sums");
-    stagger_apply_kernel<<<g, kThreads, 0, nn->stream>>>(v, fl, nn->ssum, out, X.h, X.w);
+    stagger_apply_kernel<<<g.grid(), kThreads, 0, nn->stream>>>(v, fl, nn->ssum, out, X.h, X.w, g);
     NCK(nn, cudaGetLastError(), "staggered projection");
     nn->launches += 3;  // with the smoothing launched beside it
     return LBM_OK;
@@ -1859,7 +1896,9 @@ lbm_status lbm_nn_create(int levels, const int* channels, int max_batch, int hei
     NCKC(lbm::dev_alloc(&nn->yout, Pmax * 3 * sizeof(float)), "cudaMalloc(outputs)");
     NCKC(lbm::dev_alloc(&nn->gout, Pmax * 3 * sizeof(float)), "cudaMalloc(output gradient)");
     NCKC(lbm::dev_alloc(&nn->tmp3, Pmax * 3 * sizeof(float)), "cudaMalloc(output stage)");
-    NCKC(lbm::dev_alloc(&nn->ssum, (size_t)nn->nb * kStaggerParts * 3 * sizeof(double)),
+    // (of the finest grid that lbm_nn_prolong takes: a factor of 16)
+    NCKC(lbm::dev_alloc(&nn->ssum, (size_t)nn->nb * Stagger(1, 256LL * nn->H * nn->W).parts * 3 *
+                                       sizeof(double)),
          "cudaMalloc(output sums)");
     NCKC(lbm::dev_alloc(&nn->gemm_err, sizeof(int)), "cudaMalloc(error word)");
     NCKC(cudaMemsetAsync(nn->gemm_err, 0, sizeof(int), nn->stream), "cudaMemset");
@@ -2021,10 +2060,10 @@ lbm_status lbm_nn_prolong(lbm_nn* nn, const float* y, int n, int factor, const u
     NCK(nn, cudaGetLastError(), "prolongation");
     out_smooth_kernel<false, false><<<grid_of(P), kThreads, 0, s>>>(f0, 3, fl, f1, 3, n, H, W);
     NCK(nn, cudaGetLastError(), "output smoothing (fine)");
-    const dim3 parts(n, kStaggerParts);
-    stagger_sum_kernel<<<parts, kThreads, 0, s>>>(f1, fl, nn->ssum, H, W);
+    const Stagger g(n, cells);
+    stagger_sum_kernel<<<g.grid(), kThreads, 0, s>>>(f1, fl, nn->ssum, H, W, g);
     NCK(nn, cudaGetLastError(), "staggered sums (fine)");
-    stagger_apply_kernel<<<parts, kThreads, 0, s>>>(f1, fl, nn->ssum, f0, H, W);
+    stagger_apply_kernel<<<g.grid(), kThreads, 0, s>>>(f1, fl, nn->ssum, f0, H, W, g);
     NCK(nn, cudaGetLastError(), "staggered projection (fine)");
     nn->launches += 4;
     NCK(nn, cudaMemcpyAsync(out, f0, P * 3 * sizeof(float), cudaMemcpyDeviceToHost, s),
