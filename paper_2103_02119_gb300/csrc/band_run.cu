@@ -13,16 +13,25 @@ size_t band_smem(int nx, int ny, int C) {
     return band_cells(R, P) + 16 + (size_t)kSmallTable * 4 * R * (P / 2) + (size_t)(R + 2) * P;
 }
 
+// Whether the current device takes `ctas` such CTAs at once.  Allows the kernel
+// its shared memory on this device as well: the setting belongs to the device, so it
+// is made with every lattice, not once for the process.
+template <int SCH>
+bool band_fits(int ctas, int threads, size_t smem, int sms) {
+    int n = 0;
+    if (cudaFuncSetAttribute(band_run_kernel<SCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kBandSmemMax) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, band_run_kernel<SCH>, threads, smem) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (long long)n * sms >= ctas;
+}
+
 template <int SCH>
 cudaError_t launch_band(float* f0, float* f1, const KParams<float>& p, int from, int nsteps,
                         const BandRun& b, cudaStream_t s) {
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(band_run_kernel<SCH>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmemMax);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
     cudaError_t e = cudaMemsetAsync(b.flags, 0, (size_t)b.ctas * 32 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
@@ -47,8 +56,13 @@ BandRun band_run_shape(int nx, int ny, int sms) {
     const int R = (ny + C - 1) / C, G = (nx + 1) / 2;
     if ((long long)(R + 2) * G >= 65536 || 2LL * kMailRows * G >= 65536) return b;
     const int n = ((R + 2) * G + 31) / 32 * 32;
+    const int threads = n < 64 ? 64 : n < kBandThreads ? n : kBandThreads;
+    const size_t smem = band_smem(nx, ny, C);
+    if (!(band_fits<0>(C, threads, smem, sms) && band_fits<1>(C, threads, smem, sms) &&
+          band_fits<3>(C, threads, smem, sms)))
+        return b;
     b.ctas = C;
-    b.threads = n < 64 ? 64 : n < kBandThreads ? n : kBandThreads;
+    b.threads = threads;
     b.mail_bytes = (size_t)C * 4 * kMailRows * small_row<float>(nx) * sizeof(float);
     return b;
 }

@@ -169,15 +169,10 @@ cudaLaunchConfig_t small_batch_config(const SmallBatch& b, int n, cudaStream_t s
     cfg.numAttrs = 1;
     return cfg;
 }
+// Allows the kernel its shared memory on the current device.
 cudaError_t configure_small_batch() {
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(
-            batch_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallSmemMax);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
-    return cudaSuccess;
+    return cudaFuncSetAttribute(batch_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kSmallSmemMax);
 }
 
 template <int BXT>
@@ -221,14 +216,16 @@ cudaError_t LBM_SLOT_NAME(batch_chain_launch_)(int parity, int chains, int raw, 
 
 cudaError_t LBM_SLOT_NAME(batch_small_launch_)(const SmallBatch& b, int n, int from, int nsteps,
                                                cudaStream_t s) {
-    if (cudaError_t e = configure_small_batch(); e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = small_batch_config(b, n, s, attr);
     return cudaLaunchKernelEx(&cfg, batch_small_kernel, from, nsteps);
 }
 
 bool LBM_SLOT_NAME(batch_small_fits_)(const SmallBatch& b) {
-    if (configure_small_batch() != cudaSuccess) return false;
+    if (configure_small_batch() != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = small_batch_config(b, 1, nullptr, attr);
     int n = 0;

@@ -66,6 +66,8 @@ struct BandRun {
     float* mail = nullptr;      // mail_bytes
     unsigned* flags = nullptr;  // 32 words a CTA
 };
+// The shape for a lattice on the current device, of `sms` SMs; ctas = 0 where the
+// rows do not fit a CTA or the device does not take the launch.
 BandRun band_run_shape(int nx, int ny, int sms);
 cudaError_t launch_band_run(float* f0, float* f1, const KParams<float>& p, int from, int nsteps,
                             const BandRun& b, cudaStream_t s);
@@ -79,7 +81,8 @@ constexpr int kSmallSmemMax = 227 * 1024;  // shared memory of one CTA
 template <typename T>
 cudaError_t launch_small_run(T* f0, T* f1, const uint8_t* bits, const KParams<T>& p, int from,
                              int nsteps, cudaStream_t s);
-// whether such a cluster launch fits this device (queried, no launch)
+// whether such a cluster launch fits the current device (queried, no launch);
+// called before the first launch on it
 template <typename T>
 bool small_run_fits(const KParams<T>& p);
 // columns of lattice one block of bx threads of the step kernel covers

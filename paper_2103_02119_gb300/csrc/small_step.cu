@@ -33,20 +33,15 @@ cudaLaunchConfig_t small_config(const KParams<T>& p, cudaStream_t s, cudaLaunchA
     return cfg;
 }
 
-// the largest CTA: one row of 1365 FP64 cells (3 x 1365 cells on three CTAs)
+// Allows the kernel its clusters and shared memory on the current device (of the
+// largest CTA: one row of 1365 FP64 cells, 3 x 1365 cells on three CTAs).
 template <typename T>
 cudaError_t configure_small() {
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(small_run_kernel<T>,
-                                             cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(small_run_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kSmallSmemMax);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
-    return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(small_run_kernel<T>,
+                                         cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(small_run_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kSmallSmemMax);
 }
 
 }  // namespace
@@ -79,7 +74,6 @@ template <typename T>
 cudaError_t launch_small_run(T* f0, T* f1, const uint8_t* bits, const KParams<T>& p, int from,
                              int nsteps, cudaStream_t s) {
     if (nsteps <= 0) return cudaSuccess;
-    if (cudaError_t e = configure_small<T>(); e != cudaSuccess) return e;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = small_config<T>(p, s, attr);
     return cudaLaunchKernelEx(&cfg, small_run_kernel<T>, f0, f1, bits, p, from, nsteps);
@@ -87,7 +81,10 @@ cudaError_t launch_small_run(T* f0, T* f1, const uint8_t* bits, const KParams<T>
 
 template <typename T>
 bool small_run_fits(const KParams<T>& p) {
-    if (configure_small<T>() != cudaSuccess) return false;
+    if (configure_small<T>() != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = small_config<T>(p, nullptr, attr);
     if (cfg.dynamicSmemBytes > (size_t)kSmallSmemMax) return false;
