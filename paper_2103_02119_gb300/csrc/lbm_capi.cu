@@ -1897,7 +1897,8 @@ lbm_status advance(lbm_batch* b, int64_t nsteps, bool graphs) {
     if (lbm_status s = ensure_tables(b); s != LBM_OK) return s;
     int64_t left = nsteps;
     int parity = b->parity;  // of the buffers that hold the state
-    while (b->small.cluster && left > 0) {  // one launch per group and run of steps
+    // (the tuner's steps depend on the launch shape: neither clusters nor two at once)
+    while (b->small.cluster && !b->tuning && left > 0) {  // one launch per group and run of steps
         const int n = left < kSmallRun ? (int)left : kSmallRun;
         for (int g = 0; g < b->ngroups; ++g)
             BCK(b, lbm::batch_small_launch(g, b->small, (int)b->gtab[g].size(), parity, n, b->stream),
