@@ -91,8 +91,15 @@ band_run_kernel(float* f0, float* f1, const __grid_constant__ KParams<float> p, 
 #pragma unroll
         for (int i = 0; i < 9; ++i) buf[i * plane + (r + 1) * P + x] = g[i];
     }
-    if (nx < P)  // the inactive last column counts as solid
+    if (nx < P) {
+        // the inactive last column counts as solid; its populations are zero, and
+        // nothing streams there
         for (int r = tid; r < rows + 2; r += nt) sbits[r * P + nx] = 0xFFu;
+        for (int r = tid; r < 18 * (rows + 2); r += nt) {
+            const int i = r / (rows + 2);
+            buf[i * plane + (r - i * (rows + 2)) * P + nx] = 0.0f;
+        }
+    }
     __syncthreads();
     // where each population of each pair of cells goes (small_step.cuh)
     const int own = rows * G, items = own + 2 * G;
@@ -228,7 +235,10 @@ band_run_kernel(float* f0, float* f1, const __grid_constant__ KParams<float> p, 
             if (global) {
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    if (x + j >= nx) continue;
+                    // (the row padding beside an odd width: as the row-band kernel
+                    // leaves it, untouched with a mask, else what the collision
+                    // makes of an empty cell)
+                    if (x + j >= nx && p.lmask) continue;
                     const long long o = (long long)y * p.rstride + x + j;
                     if (kChecked && !(y >= 0 && y < ny && x + j < p.rstride)) {
                         bad = true;
@@ -236,7 +246,8 @@ band_run_kernel(float* f0, float* f1, const __grid_constant__ KParams<float> p, 
                     }
 #pragma unroll
                     for (int i = 0; i < 9; ++i)
-                        fout[i * p.plane + o] = (j ? bb : ba) == 0xFFu ? 0.0f : g[j][i];
+                        fout[i * p.plane + o] =
+                            p.lmask && (j ? bb : ba) == 0xFFu ? 0.0f : g[j][i];
                 }
             }
             if (!last) {
