@@ -290,6 +290,7 @@ AuxParams aux_of(const lbm_params& q, const Geometry& g) {
     a.rho032 = (float)q.rho0;
     a.hFx32 = 0.5f * (float)q.Fx;
     a.hFy32 = 0.5f * (float)q.Fy;
+    a.inv_nx = ~0ull / (unsigned long long)q.nx + 1ull;  // (nx >= 3)
     a.lmask = g.lmask;
     return a;
 }

@@ -127,6 +127,7 @@ struct AuxParams {
     double wrest[9];          // rest weights times rho0
     double w3, w4, w5;        // relaxation rates of the second-order moments
     float a32, cs232, iah232, rho032, hFx32, hFy32;  // a, cs2, 1/(2a^2), rho0, F/2 in FP32
+    unsigned long long inv_nx;  // ceil(2^64 / nx)
     const uint8_t* __restrict__ lmask;
 };
 

@@ -56,28 +56,19 @@ struct Feq32 {
         for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < (p).nx;                  \
              x += gridDim.x * blockDim.x)
 
-// Cells in tiles of kThreads: one row of 256 columns, or 2, 4, 8 rows of 128,
-// 64, 32 on narrow lattices; a block takes tiles blockIdx.x, + gridDim.x, ...
-// (one division of a tile index, the same for the whole block, instead of
-// one of a cell index per thread).
-struct Tiles {
-    int sh, ntx, n;
-    __host__ __device__ Tiles(int nx, int ny) {
-        sh = nx <= 32 ? 5 : nx <= 64 ? 6 : nx <= 128 ? 7 : 8;
-        ntx = (nx + (1 << sh) - 1) >> sh;
-        const int rows = kThreads >> sh;
-        n = ntx * ((ny + rows - 1) / rows);
-    }
-    __device__ __forceinline__ int y(int t) const {
-        return t / ntx * (kThreads >> sh) + ((int)threadIdx.x >> sh);
-    }
-    __device__ __forceinline__ int x(int t) const {
-        return (t % ntx << sh) + ((int)threadIdx.x & ((1 << sh) - 1));
-    }
-};
-#define LBM_FOR_TILES(p, t)            \
-    const Tiles tiles((p).nx, (p).ny); \
-    for (int t = blockIdx.x; t < tiles.n; t += gridDim.x)
+// Cells c, consecutive over a block and from one row to the next, with their row and
+// column: the row by a multiplication with ceil(2^64 / nx), exact while nx times the
+// number of cells stays below 2^64.  (Tiles of one row of 256 columns, or of 2 to 8
+// rows of 128 to 32, need no multiplication but leave most threads of a narrow lattice
+// without a cell: 3 x 100000, lbm_get_f 62 us against 25, FP64 lbm_diagnostics 435 / 79;
+// 2049 x 2048 with obstacles, FP64, 123 / 112 and 578 / 550.)
+__device__ __forceinline__ int row_of(const AuxParams& p, long long c) {
+    return (int)__umul64hi((unsigned long long)c, p.inv_nx);
+}
+#define LBM_FOR_ALL_CELLS(p, c)                                                          \
+    for (long long c = blockIdx.x * (long long)kThreads + threadIdx.x,                   \
+                   n_ = (long long)(p).nx * (p).ny;                                      \
+         c < n_; c += gridDim.x * (long long)kThreads)
 
 // GB300 has two FP64 lanes per SM (against 128 FP32 and 64 integer ones): the
 // read-out kernels are bound by them, and by conversions, which take the same
@@ -232,10 +223,8 @@ __global__ void __launch_bounds__(kThreads)
 init_kernel(double* __restrict__ f, const AuxParams p, const double* __restrict__ rho,
             const double* __restrict__ ux, const double* __restrict__ uy) {
     const double iah2 = 0.5 / (p.a * p.a);
-    LBM_FOR_TILES(p, t) {
-        const int x = tiles.x(t), y = tiles.y(t);
-        if (x >= p.nx || y >= p.ny) continue;
-        const long long c = (long long)y * p.nx + x;
+    LBM_FOR_ALL_CELLS(p, c) {
+        const int y = row_of(p, c), x = (int)(c - (long long)y * p.nx);
         const long long o = (long long)y * p.rstride + x;
         const unsigned sb = link_bits<MASK>(p, x, y);
         if (sb == 0xFFu) {
@@ -379,10 +368,8 @@ template <typename T, bool MASK>
 __global__ void __launch_bounds__(kThreads)
 set_f_kernel(T* __restrict__ f, const AuxParams p, const double* __restrict__ fin) {
     const long long N = (long long)p.nx * p.ny;
-    LBM_FOR_TILES(p, t) {
-        const int x = tiles.x(t), y = tiles.y(t);
-        if (x >= p.nx || y >= p.ny) continue;
-        const long long c = (long long)y * p.nx + x;
+    LBM_FOR_ALL_CELLS(p, c) {
+        const int y = row_of(p, c), x = (int)(c - (long long)y * p.nx);
         const long long o = (long long)y * p.rstride + x;
         const unsigned sb = link_bits<MASK>(p, x, y);
         if (sb == 0xFFu) {
@@ -405,10 +392,8 @@ template <typename T, bool MASK>
 __global__ void __launch_bounds__(kThreads)
 get_f_kernel(const T* __restrict__ f, const AuxParams p, double* __restrict__ fout) {
     const long long N = (long long)p.nx * p.ny;
-    LBM_FOR_TILES(p, t) {
-        const int x = tiles.x(t), y = tiles.y(t);
-        if (x >= p.nx || y >= p.ny) continue;
-        const long long c = (long long)y * p.nx + x;
+    LBM_FOR_ALL_CELLS(p, c) {
+        const int y = row_of(p, c), x = (int)(c - (long long)y * p.nx);
         const unsigned sb = link_bits<MASK>(p, x, y);
         if (sb == 0xFFu) {
 #pragma unroll
@@ -493,9 +478,8 @@ __global__ void moments_kernel(const T* __restrict__ f, const AuxParams p,
 template <typename T, bool MASK>
 __global__ void __launch_bounds__(kThreads)
 density_kernel(const T* __restrict__ f, const AuxParams p, double* __restrict__ rho) {
-    LBM_FOR_TILES(p, t) {
-        const int x = tiles.x(t), y = tiles.y(t);
-        if (x >= p.nx || y >= p.ny) continue;
+    LBM_FOR_ALL_CELLS(p, c) {
+        const int y = row_of(p, c), x = (int)(c - (long long)y * p.nx);
         const unsigned sb = link_bits<MASK>(p, x, y);
         double r = 0.0;
         if (sb != 0xFFu) {
@@ -506,7 +490,7 @@ density_kernel(const T* __restrict__ f, const AuxParams p, double* __restrict__ 
             raw_sums(g, s, fixed);
             r = p.rho0 + s.d;
         }
-        rho[(long long)y * p.nx + x] = r;
+        rho[c] = r;
     }
 }
 
@@ -532,10 +516,9 @@ stress_kernel(const T* __restrict__ f, const AuxParams p, const StressConst q,
               const double* __restrict__ rho,
               double* __restrict__ dxux, double* __restrict__ dyuy, double* __restrict__ sxy,
               double* __restrict__ txx, double* __restrict__ tyy, double* __restrict__ txy) {
-    LBM_FOR_TILES(p, t) {
-        const int x = tiles.x(t), y = tiles.y(t);
-        if (x >= p.nx || y >= p.ny) continue;
-        const long long row = (long long)y * p.nx, c = row + x;
+    LBM_FOR_ALL_CELLS(p, c) {
+        const int y = row_of(p, c), x = (int)(c - (long long)y * p.nx);
+        const long long row = c - x;
         const unsigned sb = link_bits<MASK>(p, x, y);
         double e_xx = 0.0, e_yy = 0.0, e_xy = 0.0, s_xx = 0.0, s_yy = 0.0, s_xy = 0.0;
         if (sb != 0xFFu) {
@@ -724,10 +707,8 @@ diag_kernel(const T* __restrict__ f, const T* __restrict__ fprev, const AuxParam
     const long long N = (long long)p.nx * p.ny;
     DiagPartial d = {};
     __int128 acc = 0;
-    LBM_FOR_TILES(p, t) {
-        const int x = tiles.x(t), y = tiles.y(t);
-        if (x >= p.nx || y >= p.ny) continue;
-        const long long c = (long long)y * p.nx + x;
+    LBM_FOR_ALL_CELLS(p, c) {
+        const int y = row_of(p, c), x = (int)(c - (long long)y * p.nx);
         const unsigned sb = link_bits<MASK>(p, x, y);
         if (sb == 0xFFu) continue;
         // every read first: one latency a cell
@@ -812,8 +793,8 @@ __device__ void res_block_reduce(ResPartial& d, ResPartial* out) {
     }
 }
 
-// Block w sums reduction chunk w - rbegin[j] of active lattice j: its tiles
-// chunk, chunk + nchunk, ...
+// Block w sums reduction chunk w - rbegin[j] of active lattice j: its runs of
+// kThreads cells chunk, chunk + nchunk, ...
 __global__ void __launch_bounds__(kThreads)
 batch_res_kernel(const BatchLattice<float>* __restrict__ lat, const BatchAux* __restrict__ aux,
                  const int* __restrict__ active, const int* __restrict__ rbegin,
@@ -837,11 +818,9 @@ batch_res_kernel(const BatchLattice<float>* __restrict__ lat, const BatchAux* __
     const long long N = (long long)p.nx * p.ny;
     double* __restrict__ up = B.uprev;
     ResPartial d = {};
-    const Tiles tiles(p.nx, p.ny);
-    for (int t = chunk; t < tiles.n; t += B.nchunk) {
-        const int x = tiles.x(t), y = tiles.y(t);
-        if (x >= p.nx || y >= p.ny) continue;
-        const long long c = (long long)y * p.nx + x;
+    for (long long c = chunk * (long long)kThreads + threadIdx.x; c < N;
+         c += B.nchunk * (long long)kThreads) {
+        const int y = row_of(p, c), x = (int)(c - (long long)y * p.nx);
         const unsigned sb = link_bits<true>(p, x, y);
         if (sb == 0xFFu) continue;
         float g[9], q[9];
@@ -889,10 +868,10 @@ batch_res_final(const BatchAux* __restrict__ aux, const int* __restrict__ active
     res_block_reduce(d, out + k);
 }
 
-// blocks of LBM_FOR_TILES, at most `most`
-int tile_grid(const AuxParams& p, int most = 4096) {
-    const int n = Tiles(p.nx, p.ny).n;
-    return n < most ? n : most;
+// blocks of LBM_FOR_ALL_CELLS, at most `most`
+int cell_grid(const AuxParams& p, int most = 4096) {
+    const long long n = ((long long)p.nx * p.ny + kThreads - 1) / kThreads;
+    return n < most ? (int)n : most;
 }
 
 // grid of LBM_FOR_CELLS: blocks across a row, rows down the grid, at most
@@ -914,7 +893,7 @@ cudaError_t launch_init(T* f, const AuxParams& p, const double* rho, const doubl
         if (p.lmask) init32_kernel<true><<<g, kInitThreads, 0, s>>>(f, p, rho, ux, uy, rows);
         else init32_kernel<false><<<g, kInitThreads, 0, s>>>(f, p, rho, ux, uy, rows);
     } else {
-        const int g = tile_grid(p);
+        const int g = cell_grid(p);
         if (p.lmask) init_kernel<true><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
         else init_kernel<false><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
     }
@@ -923,7 +902,7 @@ cudaError_t launch_init(T* f, const AuxParams& p, const double* rho, const doubl
 
 template <typename T>
 cudaError_t launch_set_f(T* f, const AuxParams& p, const double* fin, cudaStream_t s) {
-    const int g = tile_grid(p);
+    const int g = cell_grid(p);
     if (p.lmask) set_f_kernel<T, true><<<g, kThreads, 0, s>>>(f, p, fin);
     else set_f_kernel<T, false><<<g, kThreads, 0, s>>>(f, p, fin);
     return cudaGetLastError();
@@ -931,7 +910,7 @@ cudaError_t launch_set_f(T* f, const AuxParams& p, const double* fin, cudaStream
 
 template <typename T>
 cudaError_t launch_get_f(const T* f, const AuxParams& p, double* fout, cudaStream_t s) {
-    const int g = tile_grid(p);
+    const int g = cell_grid(p);
     if (p.lmask) get_f_kernel<T, true><<<g, kThreads, 0, s>>>(f, p, fout);
     else get_f_kernel<T, false><<<g, kThreads, 0, s>>>(f, p, fout);
     return cudaGetLastError();
@@ -948,7 +927,7 @@ cudaError_t launch_moments(const T* f, const AuxParams& p, double* rho, double* 
 
 template <typename T>
 cudaError_t launch_density(const T* f, const AuxParams& p, double* rho, cudaStream_t s) {
-    const int g = tile_grid(p);
+    const int g = cell_grid(p);
     if (p.lmask) density_kernel<T, true><<<g, kThreads, 0, s>>>(f, p, rho);
     else density_kernel<T, false><<<g, kThreads, 0, s>>>(f, p, rho);
     return cudaGetLastError();
@@ -958,7 +937,7 @@ template <typename T>
 cudaError_t launch_stress(const T* f, const AuxParams& p, const double* rho, double* dxux,
                           double* dyuy, double* sxy, double* txx, double* tyy, double* txy,
                           cudaStream_t s) {
-    const int g = tile_grid(p);
+    const int g = cell_grid(p);
     const double a2 = p.a * p.a, c = p.cs2;
     StressConst q;
     q.a = p.a;
@@ -994,7 +973,7 @@ template <typename T>
 cudaError_t launch_diag(const T* f, const T* fprev, const AuxParams& p, double* uprev,
                         int have_prev, DiagPartial* part, int nblocks, const int* status,
                         cudaStream_t s) {
-    const int n = tile_grid(p, nblocks);
+    const int n = cell_grid(p, nblocks);
     if (p.lmask)
         diag_kernel<T, true><<<n, kThreads, 0, s>>>(f, fprev, p, uprev, have_prev, part);
     else
