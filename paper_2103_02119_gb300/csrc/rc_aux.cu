@@ -347,6 +347,40 @@ init32_kernel(float* __restrict__ f, const AuxParams p, const double* __restrict
     }
 }
 
+// The same for narrow lattices, a cell a thread: each reads its nine neighbours' fields
+// (from L1 and L2: a row is a few sectors) and evaluates the same expressions.  Up to
+// 48 columns, where a block's march leaves most of its threads without a column, and
+// from the rows on that make it march more than one (init_rows); us with obstacles,
+// cells / march: 3 x 100000 23 / 199, 17 x 100000 78 / 238, 40 x 40000 64 / 113,
+// 33 x 10000 19 / 28; but 33 x 1000 9.7 / 9.8, 17 x 1000 9.0 / 9.7 (without obstacles
+// 9.6 / 8.6), 64 x 30000 without obstacles 68 / 59, 2049 x 2048 163 / 86.
+constexpr int kInitNarrow = 48, kInitTall = 2432;
+template <bool MASK>
+__global__ void __launch_bounds__(kThreads)
+init32_narrow_kernel(float* __restrict__ f, const AuxParams p, const double* __restrict__ rho,
+                     const double* __restrict__ ux, const double* __restrict__ uy) {
+    const Feq32 feq{p.cs232, p.a32, p.iah232, p.rho032};
+    LBM_FOR_ALL_CELLS(p, c) {
+        const int y = row_of(p, c), x = (int)(c - (long long)y * p.nx);
+        const long long o = (long long)y * p.rstride + x;
+        const unsigned sb = link_bits<MASK>(p, x, y);
+        if (sb == 0xFFu) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i * p.plane + o] = 0.0f;
+            continue;
+        }
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            // the cell that pulls the slot, or this one as the opposite direction
+            const bool back = i > 0 && ((sb >> (opp(i) - 1)) & 1u);
+            const long long t = back || i == 0 ? c : target(p, x, y, i);
+            const float dr = narrow((rho ? rho[t] : 1.0) - p.rho0);
+            const float u = narrow(ux ? ux[t] : 0.0), v = narrow(uy ? uy[t] : 0.0);
+            f[i * p.plane + o] = back ? feq(opp(i), dr, u, v) : feq(i, dr, u, v);
+        }
+    }
+}
+
 // Rows of an init32_kernel band: kInitRows where the blocks then fill the
 // GPU (about eight 256-thread blocks on each of 152 SMs), fewer on smaller
 // lattices, down to one.
@@ -888,6 +922,12 @@ template <typename T>
 cudaError_t launch_init(T* f, const AuxParams& p, const double* rho, const double* ux,
                         const double* uy, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
+        if (p.nx <= kInitNarrow && p.ny >= kInitTall) {
+            const int g = cell_grid(p);
+            if (p.lmask) init32_narrow_kernel<true><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
+            else init32_narrow_kernel<false><<<g, kThreads, 0, s>>>(f, p, rho, ux, uy);
+            return cudaGetLastError();
+        }
         const int rows = init_rows(p.nx, p.ny);
         const dim3 g((p.nx + kThreads - 1) / kThreads, (p.ny + rows - 1) / rows);
         if (p.lmask) init32_kernel<true><<<g, kInitThreads, 0, s>>>(f, p, rho, ux, uy, rows);

@@ -77,3 +77,44 @@ def test_a_narrow_lattice_costs_what_its_cells_cost(precision):
         g.close()
     for name, (wide, narrow) in times.items():
         assert narrow <= 4.0 * wide, (name, times)
+
+
+@pytest.mark.parametrize("masked", [False, True])
+def test_setting_up_a_narrow_lattice(masked):
+    """lbm_init_fields of 3 x 100000 FP32 cells against 1000 x 300: at most six times the
+    time (as for the read-out, and a cell reads its nine neighbours' fields)."""
+    import torch
+    times = []
+    for nx, ny in ((1000, 300), (3, 100000)):
+        m = np.zeros((ny, nx), np.uint8) if masked else None
+        if masked:
+            m[ny // 2, nx // 2] = 1
+        g = _lattice(nx, ny, 32, m)
+        q = [torch.full((ny, nx), v, dtype=torch.float64, device="cuda") for v in (1.0, 0.01, -0.02)]
+        best = 1e9
+        for _ in range(6):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            torch.cuda.synchronize()
+            e[0].record()
+            for _ in range(20):
+                g.init_fields(*q)
+            e[1].record()
+            torch.cuda.synchronize()
+            best = min(best, e[0].elapsed_time(e[1]))
+        times.append(best)
+        g.close()
+    assert times[1] <= 6.0 * times[0], times
+
+
+@pytest.mark.parametrize("kind", ["periodic", "force", "side_walls", "walls", "walls_mask", "periodic_mask"])
+@pytest.mark.parametrize("nx,ny", [(3, 2432), (48, 2432), (48, 2431), (49, 2432), (17, 5001)])
+def test_setup_at_the_edges_of_the_narrow_form(orc, nx, ny, kind):
+    """Both forms of the FP32 set-up around the line between them, against the oracle's
+    equilibria (within a few FP32 roundings of the deviations, as in
+    test_gpu_parity.test_fp32_setup_and_readout)."""
+    from gpu_common import gpu_of, oracle_of
+    from test_gpu_chain import _flow
+    wl = _flow(nx, ny, kind)
+    o, g = oracle_of(orc, wl), gpu_of(wl, 32)
+    assert float(np.abs(g.get_f() - o.get_f()).max()) <= 1e-7
+    g.close()
