@@ -1890,6 +1890,19 @@ lbm_status lbm_batch_get_shape(const lbm_batch* b, int* block_x, int* rows_per_b
 }  // extern "C"
 
 namespace {
+// Whether a call of nsteps steps goes by the clusters.  Their launch reads and writes the
+// state on top of its steps, so a call of one step is a row-band step where
+// the shape has short bands, and one of up to three where the clusters queue for the
+// SMs, one CTA each; us a step, row-band kernel in its best shape / clusters:
+// calls of one step 16 of 64 x 64 11 / 17, 128 of 64 x 64 21 / 38, 700 of 64 x 64
+// 117 / 222; of two 128 of 64 x 64 21 / 26, 700 of 512 x 8 114 / 169; of three 114 / 143,
+// 700 of 64 x 64 116 / 114; but 16 of 64 x 64 in bands of 16 rows 37 / 17, 700 of 16 x 16
+// 58 / 42.  (The tuner's steps depend on the launch shape: never clusters.)
+bool cluster_call(const lbm_batch* b, int64_t nsteps) {
+    if (!b->small.cluster || b->tuning) return false;
+    return !(nsteps <= 3 && (b->small.queues || (nsteps == 1 && b->rows <= 8)));
+}
+
 // nsteps steps of every active lattice; runs of kGraphSteps replay a graph
 // when `graphs` is set, the rest are launched one by one.
 lbm_status advance(lbm_batch* b, int64_t nsteps, bool graphs) {
@@ -1898,8 +1911,7 @@ lbm_status advance(lbm_batch* b, int64_t nsteps, bool graphs) {
     if (lbm_status s = ensure_tables(b); s != LBM_OK) return s;
     int64_t left = nsteps;
     int parity = b->parity;  // of the buffers that hold the state
-    // (the tuner's steps depend on the launch shape: neither clusters nor two at once)
-    while (b->small.cluster && !b->tuning && left > 0) {  // one launch per group and run of steps
+    while (cluster_call(b, nsteps) && left > 0) {  // one launch per group and run of steps
         const int n = left < kSmallRun ? (int)left : kSmallRun;
         for (int g = 0; g < b->ngroups; ++g)
             BCK(b, lbm::batch_small_launch(g, b->small, (int)b->gtab[g].size(), parity, n, b->stream),

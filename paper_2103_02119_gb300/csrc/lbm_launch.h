@@ -124,6 +124,7 @@ constexpr int kBatchTableCap = 62000 / (int)sizeof(BatchTableLattice);
 struct SmallBatch {
     int cluster = 0, threads = 0;
     size_t smem = 0;
+    bool queues = false;  // one CTA an SM, and more CTAs than SMs
 };
 // The shape for lattices of these sizes (at most kSmallCells cells each;
 // cluster = 0 when they do not fit), for a device of `sms` SMs.

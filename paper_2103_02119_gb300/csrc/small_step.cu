@@ -67,6 +67,7 @@ SmallBatch small_batch_shape(const int* nx, const int* ny, int n, int sms) {
         if (best.cluster && (long long)n * C > 2LL * sms) break;
         best = b;
     }
+    best.queues = (long long)n * best.cluster > sms && 2 * best.smem > (size_t)kSmallSmemMax;
     return best;
 }
 

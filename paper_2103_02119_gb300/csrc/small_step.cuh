@@ -84,9 +84,15 @@ __device__ __forceinline__ void cluster_st(unsigned addr, float v) {
 __device__ __forceinline__ void cluster_st(unsigned addr, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
 }
+__device__ __forceinline__ void cluster_arrive() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
-                     : "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 
 // pull() with loads that bypass L1 (the buffers are written later in the launch)
@@ -119,6 +125,12 @@ __device__ __forceinline__ void pull_l2(const S* fin, const P& p, int x, int y, 
         }
         f[i] = __ldcg(fin + idx[i]);
     }
+}
+
+// the deviations of a cell summed in step_block's order
+template <typename T>
+__device__ __forceinline__ T density(const T g[9]) {
+    return ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
 }
 
 // nsteps steps of one lattice from buffer `from` (f0 or f1), by the CTAs of
@@ -162,22 +174,45 @@ __device__ __forceinline__ void small_run(const PT& p, T* f0, T* f1,
         if (kChecked && !(owner >= 0 && owner < C && yy - first >= 0 && yy - first < R)) bad = true;
     }
 
-    // the state: pulled from global memory once
+    // the state: pulled from global memory once, the cells of a group together
+    // (their reads in flight at once); an inactive last column counts as solid.  A
+    // single step pulls the rows either side too, for their densities, and then needs
+    // no neighbour CTA.
+    const int own = rows * G, items = own + 2 * G;
+    const bool one = nsteps == 1;
     {
         const T* fin = from ? f1 : f0;
-        for (int c = tid; c < rows * nx; c += nt) {
-            const int r = c / nx, x = c - r * nx;
-            const long long mi = (long long)(y0 + r) * bpitch + x;
-            const unsigned sb = bits[mi];
-            sbits[r * P + x] = (uint8_t)sb;
-            if (sb == 0xFFu) continue;
-            T g[9];
-            pull_l2(fin, p, x, y0 + r, sb, g, bad);
+        for (int it = tid; it < (one ? items : own); it += nt) {
+            const int r = (int)__umulhi((unsigned)it, inv), x = (it - r * G) * VC;
+            int y = y0 + r;
+            if (r >= rows) {  // the row below the band, or the one above it
+                if (!(r == rows ? hv[0] : hv[1])) continue;
+                y = r == rows ? y0 - 1 : y1;
+                y = y < 0 ? ny - 1 : y >= ny ? 0 : y;
+            }
+            unsigned sb[VC];
+            T g[VC][9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) buf[i * plane + r * P + x] = g[i];
+            for (int j = 0; j < VC; ++j)
+                sb[j] = x + j >= nx ? 0xFFu
+                        : p.lmask   ? bits[(long long)y * bpitch + x + j]
+                                    : link_bits<false>(p, x + j, y);
+#pragma unroll
+            for (int j = 0; j < VC; ++j)
+                if (sb[j] != 0xFFu) pull_l2(fin, p, x + j, y, sb[j], g[j], bad);
+#pragma unroll
+            for (int j = 0; j < VC; ++j) {
+                if (r >= rows) {
+                    if (sb[j] != 0xFFu)
+                        dens[(r == rows ? 0 : rows + 1) * P + x + j] = density(g[j]);
+                    continue;
+                }
+                sbits[r * P + x + j] = (uint8_t)sb[j];
+                if (sb[j] == 0xFFu) continue;
+#pragma unroll
+                for (int i = 0; i < 9; ++i) buf[i * plane + r * P + x + j] = g[j][i];
+            }
         }
-        if (nx < P)  // the inactive last column counts as solid
-            for (int r = tid; r < rows; r += nt) sbits[r * P + nx] = 0xFFu;
     }
     __syncthreads();
     // FP32: where each population of each pair of cells goes: byte offsets in
@@ -185,8 +220,7 @@ __device__ __forceinline__ void small_run(const PT& p, T* f0, T* f1,
     // word for solid cells), so that a step pushes without a test.  What they
     // cost instead, tests of nine links and two edges a cell, was half of a
     // step.
-    const int own = rows * G, items = own + 2 * G;
-    if constexpr (VC == 2) {
+    if (VC == 2 && !one) {  // (a single step pushes nothing)
         const unsigned self = cluster_map(base, (unsigned)rank);
         const unsigned dump = self + (unsigned)((unsigned char*)(table - 4) - smem) + 1u;
         for (int it = tid; it < own; it += nt) {
@@ -218,13 +252,13 @@ __device__ __forceinline__ void small_run(const PT& p, T* f0, T* f1,
             }
         }
     }
-    cluster_barrier();
+    if (!one) cluster_barrier();
 
     for (int s = 0; s < nsteps; ++s) {
         const T* cur = buf + (s & 1) * bufn;
         const int nxt = ((s & 1) ^ 1) * bufn;
         // 1. densities
-        for (int it = tid; it < items; it += nt) {
+        for (int it = tid; it < (one ? own : items); it += nt) {
             const int r = (int)__umulhi((unsigned)it, inv), x = (it - r * G) * VC;
             T g[9][VC];
             T* dst = dens;
@@ -251,6 +285,8 @@ __device__ __forceinline__ void small_run(const PT& p, T* f0, T* f1,
         __syncthreads();
         // 3. collide and push
         const bool last = s + 1 == nsteps, global = s + 2 >= nsteps;
+        // (the last step reads nothing more from its neighbours and pushes nothing)
+        if (last && !one) cluster_arrive();
         T* fout = ((from + s) & 1) ? f0 : f1;
         for (int it = tid; it < own; it += nt) {
             const int r = (int)__umulhi((unsigned)it, inv), x = (it - r * G) * VC, y = y0 + r;
@@ -397,7 +433,8 @@ __device__ __forceinline__ void small_run(const PT& p, T* f0, T* f1,
                 }
             }
         }
-        cluster_barrier();
+        if (!last) cluster_arrive();
+        if (!one) cluster_wait();
     }
     if (kChecked && bad) atomicOr(p.status, kStatusBounds);
 }
