@@ -323,11 +323,14 @@ const char* lbm_last_error(const lbm_handle* h);
  * scheme reads the parameters from a table in global memory (slower: they
  * then take vector registers).  Runs of 50 steps replay a captured CUDA
  * graph.  When every active lattice has at most 4096 cells (and they fit the
- * constant-memory tables), each steps on a thread-block cluster of its own
- * that keeps its state in shared memory, up to 1024 steps per launch and
- * group.  Else, when every one collides and has at least 64 x 16 cells, a
+ * constant-memory tables, and no more than half of them are wider than 512
+ * columns), each steps on a thread-block cluster of its own that keeps its state
+ * in shared memory, up to 1024 steps per launch and group; but for calls of one step
+ * with bands of up to 8 rows, and of up to 3 where the clusters outnumber the SMs and
+ * fill them.  Else, when every one collides and has at least 64 x 16 cells, a
  * launch per group takes two steps, but for the last one or two of a call.  The
- * launch shape does not matter to either.  Lattices can be retired (made inactive) and brought back; an inactive lattice keeps
+ * choice changes the schedule only, never the results.  Lattices can be retired
+ * (made inactive) and brought back; an inactive lattice keeps
  * its state and is not stepped.  Conventions as for lbm_handle; work is
  * issued on the stream given to lbm_batch_create.
  * ------------------------------------------------------------------------ */
@@ -392,8 +395,8 @@ int lbm_batch_is_active(const lbm_batch* b, int k);
 
 /* Launch shape of the batch step: threads per block along x (32, 64 or 128;
  * a block covers 2 x block_x columns) and target rows per band (1 .. 65536;
- * lattice k gets max(1, round(ny_k / rows_per_band)) bands), for single
- * steps.  The shape changes the schedule only, never the results.  Default 32, 16. */
+ * lattice k gets max(1, round(ny_k / rows_per_band)) bands), for the launches of one
+ * step.  The shape changes the schedule only, never the results.  Default 32, 16. */
 lbm_status lbm_batch_set_shape(lbm_batch* b, int block_x, int rows_per_band);
 lbm_status lbm_batch_get_shape(const lbm_batch* b, int* block_x, int* rows_per_band);
 
@@ -435,7 +438,7 @@ lbm_status lbm_batch_diagnostics(lbm_batch* b, int k, double out[LBM_DIAG_COUNT]
 int64_t lbm_batch_step_count(const lbm_batch* b, int k);
 
 /* Batch step kernel launches issued so far: one per group of lattices and
- * step, or two steps, or (active lattices of at most 4096 cells) run of up to 1024 steps. */
+ * step, or two steps, or (clusters) run of up to 1024 steps. */
 int64_t lbm_batch_launch_count(const lbm_batch* b);
 
 /* Message of the last error on b (or of the last failed lbm_batch_create

@@ -1495,7 +1495,13 @@ void plan_groups(lbm_batch* b) {
                 nx.push_back(b->p[k].nx);
                 ny.push_back(b->p[k].ny);
             }
-        if ((int)nx.size() == b->n_active) {
+        // but for a majority of wide, flat ones, whose CTAs hold a row or two: what they
+        // exchange outweighs what they compute.  us a step of calls of 50, row-band
+        // kernel in its best shape / clusters: 16 of 700 x 3 8.3 / 13, 128 of 682 x 6
+        // 19 / 22, 16 of 1024 x 4 9.1 / 16, 128 of 1365 x 3 15 / 39; but 128 of 512 x 4
+        // 13 / 7.2, 700 of 512 x 8 103 / 89
+        const auto wide = std::count_if(nx.begin(), nx.end(), [](int w) { return w > 512; });
+        if ((int)nx.size() == b->n_active && 2 * wide <= b->n_active) {
             b->small = lbm::small_batch_shape(nx.data(), ny.data(), b->n_active, b->sms);
             for (int g = 0; b->small.cluster && g < b->ngroups; ++g)
                 if (!lbm::batch_small_fits(g, b->small)) b->small = lbm::SmallBatch{};

@@ -2,6 +2,8 @@
 // thread-block cluster (the work is in small_step.cuh).
 #include "small_step.cuh"
 
+#include <algorithm>
+
 namespace lbm {
 
 namespace {
@@ -47,13 +49,15 @@ cudaError_t configure_small() {
 }  // namespace
 
 // CTAs per lattice of a batch: as many (1, 2, 4, 8) as shared memory asks for,
-// and more while the batch makes at most two CTAs per SM.  Us a step with a
+// and more while the batch makes at most two CTAs per SM and the tallest lattice has
+// two rows for each.  Us a step with a
 // target of one / two / four CTAs per SM (and of the band kernel, one launch a
 // step): 64 lattices of 16-32 cells a side 1.89 / 1.83 / 1.94 (11.0), 32 of 60-64
 // 2.80 / 2.64 / 2.64 (11.9), 128 of 16-64 4.34 / 4.35 / 6.55 (24.5).
 SmallBatch small_batch_shape(const int* nx, const int* ny, int n, int sms) {
     SmallBatch best;
     // (a CTA past a lattice's last row has none and only joins the barriers)
+    const int tallest = n ? *std::max_element(ny, ny + n) : 0;
     for (int C = 1; C <= 8; C *= 2) {
         SmallBatch b;
         b.cluster = C;
@@ -64,7 +68,7 @@ SmallBatch small_batch_shape(const int* nx, const int* ny, int n, int sms) {
             if (t > b.threads) b.threads = t;
         }
         if (b.smem > (size_t)kSmallSmemMax) continue;
-        if (best.cluster && (long long)n * C > 2LL * sms) break;
+        if (best.cluster && ((long long)n * C > 2LL * sms || 2 * C > tallest)) break;
         best = b;
     }
     best.queues = (long long)n * best.cluster > sms && 2 * best.smem > (size_t)kSmallSmemMax;
