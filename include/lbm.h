@@ -137,11 +137,12 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
  * once per starting buffer (on a stream of its own; lbm_set_force drops
  * it).  Small lattices run many steps per launch (lbm_set_small_path), and so
  * do FP32 lattices below 200,000 cells in calls of at least 3 steps (14 up to
- * 20,480 cells) where a CTA's rows fit its shared memory (a cooperative launch of
- * up to 1024 steps); larger
- * FP32 ones (from 80,000 cells) take two steps per launch but for the last one
- * or two of a call; the states are bit for bit the same.  Asynchronous: the
- * return value reports launch errors only. */
+ * 20,480 cells) where a CTA's rows, two or more of them, fit its shared memory (up to
+ * 596 columns) and the device takes the launch: a cooperative one of up to 1024 steps.
+ * Larger FP32 ones (from 80,000 cells; from 380,000 where at most 64 columns lie
+ * between walls at rest none) take two steps per launch but for the last one or two of a
+ * call.  The states are bit for bit the same.  Asynchronous: the return value reports
+ * launch errors only. */
 lbm_status lbm_step(lbm_handle* h, int64_t nsteps);
 
 /* Replace the uniform body force density F (Sec. 4: it shifts the velocity
@@ -327,9 +328,10 @@ const char* lbm_last_error(const lbm_handle* h);
  * columns), each steps on a thread-block cluster of its own that keeps its state
  * in shared memory, up to 1024 steps per launch and group; but for calls of one step
  * with bands of up to 8 rows, and of up to 3 where the clusters outnumber the SMs and
- * fill them.  Else, when every one collides and has at least 64 x 16 cells, a
- * launch per group takes two steps, but for the last one or two of a call.  The
- * choice changes the schedule only, never the results.  Lattices can be retired
+ * fill them.  Else, when every one collides and has at least 64 x 16 cells (and, with
+ * bands of up to 8 rows, no more than half of the cells lie in lattices of 64
+ * columns between walls at rest), a launch per group takes two steps, but for the
+ * last one or two of a call.  The choice changes the schedule only, never the results.  Lattices can be retired
  * (made inactive) and brought back; an inactive lattice keeps
  * its state and is not stepped.  Conventions as for lbm_handle; work is
  * issued on the stream given to lbm_batch_create.

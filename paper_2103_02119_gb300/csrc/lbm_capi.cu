@@ -675,7 +675,13 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
     //   10.4 / 16.0, 200 x 6000 21.6 / 25.2, 2048 x 8192 162 / 209;
     //   cavities with obstacles 256^2 7.2 / 6.7, 300^2 7.3 / 7.6, 1001 x 2003
     //   27.8 / 33.8, 1543 x 3001 54 / 79, 2048 x 8192 165 / 215.
-    if (!f64 && !kRowInterleaved && h->N >= 80000)
+    // But a lattice that fills one 64-column segment of the row-band kernel, between
+    // walls at rest, takes two strips of the two-step kernel: tall ones are slower, calls
+    // of 100 steps 64 x 6000 18.4 / 16.8, 64 x 10000 24.5 / 20.8, of 40 64 x 20000
+    // 38 / 31, 64 x 65000 98 / 90 (but 64 x 4000 14.5 / 18.2; 64 x 65000 periodic along
+    // x 74 / 104, with moving walls 105 / 121).
+    const bool one_segment = lbm::one_segment(kparams<float>(h));
+    if (!f64 && !kRowInterleaved && h->N >= 80000 && !(one_segment && h->N >= 380000))
         h->chain_bands = lbm::chain2_bands(p->nx, p->ny, h->pitch, sms);
     // small lattices: all the steps of an lbm_step call in one launch of one
     // thread-block cluster, when the device can hold it
@@ -1364,12 +1370,23 @@ bool g_table_fresh[64] = {};
 // of one height, when the kernel was slower by other causes).
 void plan_chains(lbm_batch* b) {
     b->chains = b->ngroups > 0 && b->small.cluster == 0;
+    double cells = 0.0, narrow = 0.0;
     for (int g = 0; g < b->ngroups; ++g) {
         b->gchain[g].assign(b->gtab[g].size() + 1, 0);
-        for (const lbm::BatchTableLattice& L : b->gtab[g])  // (36 plane: offsets of 32 bits)
+        for (const lbm::BatchTableLattice& L : b->gtab[g]) {  // (36 plane: offsets of 32 bits)
             b->chains &= L.kp.collide && lbm::chain2_takes(L.kp.nx, L.kp.ny, L.kp.pitch) &&
                          36.0 * (double)L.kp.plane < 4294967296.0;
+            cells += (double)L.kp.nx * L.kp.ny;
+            if (lbm::one_segment(L.kp)) narrow += (double)L.kp.nx * L.kp.ny;
+        }
     }
+    // Lattices of 64 columns between walls at rest take two strips each, where the
+    // row-band kernel takes one segment: with short bands (the tuned shapes) it is the
+    // faster one for batches of mostly such lattices, us a step, two-step / row-band kernel
+    // in bands of 4 rows: 1 of 64 x 65 8.5 / 13 (of 1 row 8.2 / 6.7), 4 of 64 x 1000
+    // 16 / 14, 20 of 64 x 1000 45 / 35, 312 of 64 x 65 57 / 52; in bands of 16 45 / 44 and
+    // 59 / 81.
+    if (b->rows <= 8 && 2.0 * narrow > cells) b->chains = false;
     if (!b->chains) return;
     const double full = 8.0 * b->sms;  // chains in flight
     auto strips = [](const lbm::BatchTableLattice& L) {

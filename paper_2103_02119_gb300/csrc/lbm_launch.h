@@ -53,6 +53,12 @@ constexpr int kChainColumns = 56;
 inline bool chain2_takes(int nx, int ny, int pitch) {
     return nx >= 64 && ny >= 16 && 4.0 * pitch * ny < 4294967296.0;
 }
+// Whether a lattice is one 64-column segment of the row-band kernel between walls at
+// rest along x (no wall moves).
+template <typename PT>
+bool one_segment(const PT& k) {
+    return k.nx <= 64 && !k.px && !k.moving;
+}
 template <typename T>
 int step_occupancy(int bx, bool mask);
 
