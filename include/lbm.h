@@ -137,8 +137,10 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
  * once per starting buffer (on a stream of its own; lbm_set_force drops
  * it).  Small lattices run many steps per launch (lbm_set_small_path), and so
  * do FP32 lattices below 200,000 cells in calls of at least 3 steps (14 up to
- * 20,480 cells) where a CTA's rows, two or more of them, fit its shared memory (up to
- * 596 columns) and the device takes the launch: a cooperative one of up to 1024 steps.
+ * 20,480 cells, else 4 above 450 columns) where a CTA's rows, two or more of them, fit
+ * its shared memory (up to 596 columns; 560 without a mask where 200 rows or fewer make
+ * more than 20,480 cells) and the device takes the launch: a cooperative one of up to
+ * 1024 steps.
  * Larger FP32 ones (from 80,000 cells; from 380,000 where at most 64 columns lie
  * between walls at rest none) take two steps per launch but for the last one or two of a
  * call.  The states are bit for bit the same.  Asynchronous: the return value reports

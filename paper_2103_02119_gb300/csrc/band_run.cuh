@@ -21,8 +21,8 @@
 // of step s - 2.  The launch is cooperative (all CTAs resident); every wait
 // is bounded, and one that runs out ends the CTA with bit 0 of the status word.
 //
-// What bounds it: latency, 3 to 6 us a step (256 x 256: 4.3 against 6.7 with a
-// launch per step; 16 x 2000 3.2 / 20.6; 100 x 1000 4.0 / 7.4): the exchange
+// What bounds it: latency, 3 to 8 us a step (256 x 256: 4.1 against 7.1 with a
+// launch per step; 16 x 2000 3.0 / 18; 100 x 1000 3.7 / 18): the exchange
 // through the L2 (a release, a neighbour's acquire, its reads of the mailbox),
 // about half of it, and the dependent instructions of a collision by two warps a
 // scheduler.  A fence before the release, which the block barrier makes

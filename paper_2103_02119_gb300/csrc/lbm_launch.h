@@ -64,7 +64,9 @@ int step_occupancy(int bx, bool mask);
 
 // Middle-sized FP32 lattices: nsteps steps in one cooperative launch of a CTA
 // per band of rows (band_run.cuh), from buffer `from` (f0 or f1).
-constexpr int kBandThreads = 512;
+// (640 threads: a pair of cells each for two rows of up to 640 columns, where 512 left a
+// second pass of a few; 596 x 100 8.6 -> 7.8 us a step; 96 registers a thread, no spills)
+constexpr int kBandThreads = 640;
 struct BandRun {
     int ctas = 0, threads = 0;  // 0: the lattice cannot take it
     // device buffers of the lattice:
