@@ -84,9 +84,11 @@ typedef struct {
                               or top wall                                        */
     int32_t use_iso_corr;  /* 1: isotropy correction m^{eq,s} (Eq. 23-24)       */
     int32_t use_gi_corr;   /* 1: Galilean-invariance correction (Eq. 25-26)     */
-    int32_t block_x;       /* step kernel tuning: threads per block along x,
-                              0 = automatic, else one of 32, 64, 128, 256        */
-    int32_t bands;         /* step kernel tuning: number of row bands,
+    int32_t block_x;       /* row-band kernel tuning: threads per block along x,
+                              0 = automatic, else one of 32, 64, 128, 256.  The
+                              kernels that take several steps per launch
+                              (lbm_step) have shapes of their own               */
+    int32_t bands;         /* row-band kernel tuning: number of row bands,
                               0 = automatic                                     */
     int32_t scheme;        /* 0: RC-LBM collision (Sec. 4); 1: raw-moment
                               collision (RNR-LBM, Sec. 3: Eq. 10-13 with the

@@ -1,9 +1,11 @@
 """Launch-shape tuning with a JSON cache (library plumbing; the paper has no
 tuner).
 
-The single-lattice step kernel takes a block width (32, 64, 128 or 256
-threads, two cells each) and a number of row bands; the batch kernel takes a
-block width and rows per band.  A tuner times candidate shapes on the GPU and
+The row-band kernel of a single lattice takes a block width (32, 64, 128 or 256
+threads, two cells each) and a number of row bands; that of a batch takes a
+block width and rows per band.  (The kernels that take several steps per launch have
+shapes of their own: for FP32 lattices above 4096 cells the shape is that of calls of
+a step or two and of the last steps of longer ones.)  A tuner times candidate shapes on the GPU and
 keeps the fastest; the result goes to a JSON cache keyed by (nx, ny,
 precision, layout, mask) -- for a batch, by its multiset of lattice sizes --
 so that a later run of the same size takes the shape without measuring.
