@@ -302,27 +302,44 @@ template <typename T>
 KParams<T> kparams(const lbm_handle* h) { return kparams_of<T>(h->p, geometry(h)); }
 AuxParams aux(const lbm_handle* h) { return aux_of(h->p, geometry(h)); }
 
-// Bands of an FP64 lattice in blocks of one warp: the fewest microseconds by a
-// model fitted to 19 sizes (24 x 2816 to 1024 x 1024; 12 % rms, its choice
-// mostly within 8 % of the best shape measured): a block takes 12 us a
-// row alone on its SM, the SM's FP64 pipe 1.3 us per row of a warp; blocks that
-// are all resident end with the fullest SM, more of them even out but for the
-// last block.
+// Microseconds of a step of an FP64 lattice in blocks of `width` columns (64 a warp) and nb
+// bands, by a model fitted to 19 sizes (24 x 2816 to 1024 x 1024; 12 % rms): a
+// block takes 12 us a row alone on its SM, the SM's FP64 pipe 1.3 us per row of a warp;
+// blocks that are all resident end with the fullest SM, more of them even out but for
+// the last block.  Blocks go to the SMs in turn, segments first: where the number of
+// segments and of SMs share a factor, an SM holds blocks of the same few segments, and
+// the last one is lighter (whole warps past the lattice skip the collision, a warp of
+// one column half of it).
+double shape_cost(int nx, int ny, int width, int nb, int occupancy, int sms) {
+    const int nseg = (nx + width - 1) / width;
+    auto warps = [&](int seg) {  // of a segment
+        const int c = std::min(width, nx - seg * width);
+        return c / 64 + (c % 64 == 0 ? 0.0 : c % 64 == 1 ? 0.5 : 1.0);
+    };
+    int share = nseg;  // the greatest common divisor
+    for (int a = sms; a != 0;) {
+        const int t = share % a;
+        share = a;
+        a = t;
+    }
+    const double all = (nseg - 1) * warps(0) + warps(nseg - 1);
+    // the fullest SM's blocks: full segments alone if there are as many classes
+    const double most = share == 1 ? all / nseg : warps(0);
+    const double per_sm = (double)nseg * nb / sms, tall = (ny + nb - 1) / nb + 0.35;
+    const double march = 12.0 * tall;
+    if (per_sm <= occupancy) {
+        const double pipe = 1.3 * std::ceil(per_sm) * tall * most;
+        return std::pow(std::pow(march, 2.2) + std::pow(pipe, 2.2), 1.0 / 2.2);
+    }
+    return 1.3 * per_sm * (all / nseg) * ((double)ny / nb + 0.35) + 0.89 * march;
+}
+// Its bands in blocks of one warp: the cheapest of 1 to 32 rows.
 int short_bands(int nx, int ny, int width, int occupancy, int sms) {
-    const double nseg = (nx + width - 1) / width;
     int best = ny;
     double cost = 0.0;
     for (int rows = 1; rows <= 32 && rows <= ny; ++rows) {
-        const int nb = (ny + rows / 2) / rows < 1 ? 1 : (ny + rows / 2) / rows;
-        const double per_sm = nseg * nb / sms, tall = (ny + nb - 1) / nb + 0.35;
-        const double march = 12.0 * tall;
-        double c;
-        if (per_sm <= occupancy) {
-            const double pipe = 1.3 * std::ceil(per_sm) * tall;
-            c = std::pow(std::pow(march, 2.2) + std::pow(pipe, 2.2), 1.0 / 2.2);
-        } else {
-            c = 1.3 * per_sm * ((double)ny / nb + 0.35) + 0.89 * march;
-        }
+        const int nb = std::max(1, (ny + rows / 2) / rows);
+        const double c = shape_cost(nx, ny, width, nb, occupancy, sms);
         if (rows == 1 || c < cost) {
             best = nb;
             cost = c;
@@ -641,22 +658,8 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
         return f64 ? lbm::step_segment_width<double>(b) : lbm::step_segment_width<float>(b);
     };
     int bx = p->block_x, nb = p->bands;
-    // Middle-sized FP64 lattices: many one-warp blocks of few rows, where the
-    // shapes below leave SMs with long marches or a second wave of few blocks;
-    // us a step, that / those: 192^2 24 / 29, 64 x 1000 33 / 99, 300^2 44 / 85,
-    // 300 x 700 87 / 171, 512^2 105 / 171, 600^2 142 / 158, 2000 x 200 150 / 171,
-    // 724^2 199 / 246, 850^2 274 / 308, 800 x 1300 365 / 445, 300 x 3000 354 / 530;
-    // but 1024 x 700 254 / 247, 1500 x 600 318 / 306, 1024^2 364 / 345 (not measured
-    // above 1.1 million cells).  A block per row and SM is already the shortest
-    // where there are no more rows: 128^2 23.1 / 20.8.
-    if (f64 && bx == 0 && nb == 0 && (h->N < 700000 || (h->N < 1100000 && p->nx < 900)) &&
-        (long long)((p->nx + seg_width(128) - 1) / seg_width(128)) * p->ny > sms) {
-        bx = 32;
-        nb = short_bands(p->nx, p->ny, seg_width(32),
-                         lbm::step_occupancy<double>(32, solid_mask != nullptr), sms);
-    }
+    const bool automatic = bx == 0 && nb == 0;
     if (bx == 0) bx = p->nx <= seg_width(32) ? 32 : p->nx <= seg_width(64) ? 64 : 128;
-    h->bx = bx;
     const int nseg = (p->nx + seg_width(bx) - 1) / seg_width(bx);
     if (nb == 0) {
         // Short bands (about 14 rows) keep the blocks that run at the same
@@ -673,7 +676,34 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
         if (nb < 1) nb = 1;
     }
     if (nb > p->ny) nb = p->ny;
+    // Middle-sized FP64 lattices: many one-warp blocks of few rows, where the
+    // shape above leaves SMs with long marches or a second wave of few blocks;
+    // us a step, that / this: 192^2 24 / 29, 64 x 1000 33 / 99, 300^2 44 / 85,
+    // 300 x 700 87 / 171, 512^2 105 / 171, 600^2 142 / 158, 2000 x 200 150 / 171,
+    // 724^2 199 / 246, 850^2 274 / 308, 800 x 1300 365 / 445, 300 x 3000 354 / 530;
+    // but 1024 x 700 254 / 247, 1500 x 600 318 / 306, 1024^2 364 / 345 (not measured
+    // above 1.1 million cells).  A block per row and SM is already the shortest
+    // where there are no more rows: 128^2 23.1 / 20.8.  And only where the model says
+    // 10 % less (20 % beside a last segment of one column, which it knows least): over
+    // 220 sizes from 20 x 301 to 850 x 1177, with and without obstacles, that takes 0.87
+    // of the time of the shape above in the mean, and none more than 1.06 of it; the
+    // choice by size alone took 0.88, but 1.29 at 65 x 10616, 1.15 at 129 x 3101 and
+    // 1.07 at 500 x 2001.
+    if (f64 && automatic && (h->N < 700000 || (h->N < 1100000 && p->nx < 900)) &&
+        (long long)((p->nx + seg_width(128) - 1) / seg_width(128)) * p->ny > sms) {
+        const bool mask = solid_mask != nullptr;
+        const int occ = lbm::step_occupancy<double>(32, mask);
+        const int bands = short_bands(p->nx, p->ny, seg_width(32), occ, sms);
+        const double least = p->nx % seg_width(32) == 1 ? 0.8 : 0.9;
+        if (shape_cost(p->nx, p->ny, seg_width(32), bands, occ, sms) <
+            least * shape_cost(p->nx, p->ny, seg_width(bx), nb,
+                               lbm::step_occupancy<double>(bx, mask), sms)) {
+            bx = 32;
+            nb = bands;
+        }
+    }
     if (nb > 65535) nb = 65535;  // grid.y limit
+    h->bx = bx;
     h->nbands = nb;
     // Two steps per launch (chain_step.cuh) where that is faster than the
     // row-band kernel; us a step, two-step / row-band kernel:
