@@ -143,10 +143,12 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
  * its shared memory (up to 596 columns; 560 without a mask where 200 rows or fewer make
  * more than 20,480 cells) and the device takes the launch: a cooperative one of up to
  * 1024 steps.
- * Larger FP32 ones (from 80,000 cells; from 380,000 where at most 64 columns lie
- * between walls at rest none) take two steps per launch but for the last one or two of a
- * call.  The states are bit for bit the same.  Asynchronous: the return value reports
- * launch errors only. */
+ * Larger FP32 ones (from 80,000 cells) take two steps per launch but for the last one
+ * or two of a call; but not where the replayed graph of the row-band kernel is the
+ * faster one: lattices of at most 64 columns between walls at rest from 380,000 cells
+ * on, and below 200,000 cells some with walls along x or moving walls, for runs of 50
+ * steps or for all.  The states are bit for bit the same.  Asynchronous: the return
+ * value reports launch errors only. */
 lbm_status lbm_step(lbm_handle* h, int64_t nsteps);
 
 /* Replace the uniform body force density F (Sec. 4: it shifts the velocity

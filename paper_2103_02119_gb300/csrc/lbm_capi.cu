@@ -64,6 +64,7 @@ struct lbm_handle {
     int diag_blocks = 0;
     int bx = 0, nbands = 0;
     int chain_bands = 0;       // bands of the two-step kernel (0: not used)
+    bool runs_first = false;   // runs of kRunSteps by the row-band kernel, the rest by that one
     lbm::BandRun band;         // the many-step kernel of middle-sized lattices (ctas = 0: not used)
     int64_t steps = 0, launches = 0;
     uint8_t* bits = nullptr;   // small lattices: link bits of the nx * ny cells (device)
@@ -501,18 +502,24 @@ lbm_status step_lattice(lbm_handle* h, int64_t nsteps) {
             h->steps += n;
             left -= n;
         }
-        // Two steps per launch; the last one or two are single steps, so that
-        // the other buffer then holds the state one step earlier.
-        while (h->chain_bands && k.collide && left >= 3) {
-            CK(h, lbm::launch_chain2((const float*)h->f[h->cur], (float*)h->f[h->cur ^ 1], k,
-                                     h->chain_bands, h->stream),
-               "two-step kernel");
-            h->cur ^= 1;
-            h->launches += 1;
-            h->steps += 2;
-            left -= 2;
-        }
     }
+    // Two steps per launch; the last one or two of a call are single steps, so that
+    // the other buffer then holds the state one step earlier.
+    auto chain = [&]() -> lbm_status {
+        if constexpr (sizeof(T) == 4)
+            while (h->chain_bands && k.collide && left >= 3) {
+                CK(h, lbm::launch_chain2((const float*)h->f[h->cur], (float*)h->f[h->cur ^ 1], k,
+                                         h->chain_bands, h->stream),
+                   "two-step kernel");
+                h->cur ^= 1;
+                h->launches += 1;
+                h->steps += 2;
+                left -= 2;
+            }
+        return LBM_OK;
+    };
+    if (!h->runs_first)
+        if (lbm_status st = chain(); st != LBM_OK) return st;
     while (left >= kRunSteps) {
         if (lbm_status st = ensure_run_graph<T>(h, k, h->cur); st != LBM_OK) return st;
         CK(h, cudaGraphLaunch(h->graph[h->cur], h->stream), "cudaGraphLaunch");
@@ -520,6 +527,7 @@ lbm_status step_lattice(lbm_handle* h, int64_t nsteps) {
         h->launches += kRunSteps;
         h->steps += kRunSteps;
     }
+    if (lbm_status st = chain(); st != LBM_OK) return st;
     CK(h, launch_steps_of<T>(h, k, h->cur, (int)left, h->stream), "step kernel");
     h->cur ^= (int)(left & 1);
     h->launches += left;
@@ -721,6 +729,27 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
     const bool one_segment = lbm::one_segment(kparams<float>(h));
     if (!f64 && !kRowInterleaved && h->N >= 80000 && !(one_segment && h->N >= 380000))
         h->chain_bands = lbm::chain2_bands(p->nx, p->ny, h->pitch, sms);
+    // Below 200,000 cells the row-band kernel's bands are of a row or two, and a replayed run
+    // of it is as fast as the two-step kernel, or faster where that has walls along x
+    // or an odd width (its outer strips) or moving walls to do and no link bits to read;
+    // us a step of calls of 100, two-step / row-band kernel: walls at rest 900 x 90
+    // 7.2 / 6.1, 900 x 178 9.2 / 7.3, a moving lid 2500 x 65 9.2 / 7.7, moving side walls
+    // 600 x 135 9.2 / 6.8, with obstacles 9.3 / 8.7, a channel 1393 x 94 8.2 / 7.6; but
+    // channels 600 x 135 7.2 / 7.3, walls at rest with obstacles 8.2 / 8.4, and in bands
+    // of two rows 1393 x 133 9.3 / 11.2 (moving side walls 900 x 206 11.2 / 10.1).
+    // Launched one by one the row-band kernel is the slower one (calls of 10, 900 x 90
+    // 7.5 / 8.3, a lid 7.7 / 8.4), but with moving side walls and no obstacles
+    // (9.1 / 8.5).
+    if (h->chain_bands && h->N < 200000) {
+        const KParams<float> k = kparams<float>(h);
+        const int rows = (p->ny + nb - 1) / nb;  // of a band
+        const bool mask = solid_mask != nullptr;
+        const bool sides = !p->periodic_x && lbm::moving_sides(k);
+        h->runs_first =
+            (rows == 1 && (mask ? sides : !p->periodic_x || k.moving || p->nx % 2 == 1)) ||
+            (rows == 2 && sides && !mask);
+        if (rows == 1 && sides && !mask) h->chain_bands = 0;
+    }
     // small lattices: all the steps of an lbm_step call in one launch of one
     // thread-block cluster, when the device can hold it
     if (h->N <= lbm::kSmallCells && !kRowInterleaved) {

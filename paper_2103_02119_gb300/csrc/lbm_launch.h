@@ -59,6 +59,14 @@ template <typename PT>
 bool one_segment(const PT& k) {
     return k.nx <= 64 && !k.px && !k.moving;
 }
+// Whether a wall along x moves.
+template <typename PT>
+bool moving_sides(const PT& k) {
+    for (int w = 0; w < 2; ++w)
+        for (int j = 0; j < 3; ++j)
+            if (k.wall_odd[w][j] != 0) return true;
+    return false;
+}
 template <typename T>
 int step_occupancy(int bx, bool mask);
 

@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny,kind,steps,launches", [
     (450, 100, "walls", 3, 1), (451, 100, "walls", 3, 3), (451, 100, "walls", 4, 1), (451, 100, "walls_mask", 3, 3),
     (560, 60, "periodic", 60, 1), (561, 60, "periodic", 9, 9), (561, 60, "periodic_mask", 9, 1),
-    (596, 200, "walls", 9, 5), (596, 202, "walls", 9, 1), (590, 8, "periodic", 14, 1)])
+    (596, 200, "force", 9, 5), (596, 202, "force", 9, 1), (590, 8, "periodic", 14, 1)])
 def test_route_and_states(nx, ny, kind, steps, launches):
     from paper_2103_02119_gb300.lbm import Lattice
     wl = _flow(nx, ny, kind)
