@@ -303,36 +303,42 @@ template <typename T>
 KParams<T> kparams(const lbm_handle* h) { return kparams_of<T>(h->p, geometry(h)); }
 AuxParams aux(const lbm_handle* h) { return aux_of(h->p, geometry(h)); }
 
-// Microseconds of a step of an FP64 lattice in blocks of `width` columns (64 a warp) and nb
+// Warps that a row of an FP64 lattice keeps busy in blocks of `width` columns (64 a warp;
+// whole warps past the lattice skip the collision, a warp of one column half of it).
+// Blocks go to the SMs in turn, segments first: where the numbers of segments and of SMs
+// share a factor, an SM holds blocks of the same few segments, and the last one is
+// lighter.
+struct RowWarps {
+    double mean, most;  // of a block, and of one on the fullest SM
+    RowWarps(int nx, int width, int sms) {
+        const int nseg = (nx + width - 1) / width, c = nx - (nseg - 1) * width;
+        const double full = width / 64;
+        const double last = c / 64 + (c % 64 == 0 ? 0.0 : c % 64 == 1 ? 0.5 : 1.0);
+        mean = ((nseg - 1) * full + last) / nseg;
+        int share = nseg;  // the greatest common divisor
+        for (int a = sms; a != 0;) {
+            const int t = share % a;
+            share = a;
+            a = t;
+        }
+        most = nseg == 1 ? last : share == 1 ? mean : full;
+    }
+};
+// Microseconds of a step of an FP64 lattice in blocks of `width` columns and nb
 // bands, by a model fitted to 19 sizes (24 x 2816 to 1024 x 1024; 12 % rms): a
 // block takes 12 us a row alone on its SM, the SM's FP64 pipe 1.3 us per row of a warp;
 // blocks that are all resident end with the fullest SM, more of them even out but for
-// the last block.  Blocks go to the SMs in turn, segments first: where the number of
-// segments and of SMs share a factor, an SM holds blocks of the same few segments, and
-// the last one is lighter (whole warps past the lattice skip the collision, a warp of
-// one column half of it).
+// the last block.
 double shape_cost(int nx, int ny, int width, int nb, int occupancy, int sms) {
+    const RowWarps w(nx, width, sms);
     const int nseg = (nx + width - 1) / width;
-    auto warps = [&](int seg) {  // of a segment
-        const int c = std::min(width, nx - seg * width);
-        return c / 64 + (c % 64 == 0 ? 0.0 : c % 64 == 1 ? 0.5 : 1.0);
-    };
-    int share = nseg;  // the greatest common divisor
-    for (int a = sms; a != 0;) {
-        const int t = share % a;
-        share = a;
-        a = t;
-    }
-    const double all = (nseg - 1) * warps(0) + warps(nseg - 1);
-    // the fullest SM's blocks: full segments alone if there are as many classes
-    const double most = share == 1 ? all / nseg : warps(0);
     const double per_sm = (double)nseg * nb / sms, tall = (ny + nb - 1) / nb + 0.35;
     const double march = 12.0 * tall;
     if (per_sm <= occupancy) {
-        const double pipe = 1.3 * std::ceil(per_sm) * tall * most;
+        const double pipe = 1.3 * std::ceil(per_sm) * tall * w.most;
         return std::pow(std::pow(march, 2.2) + std::pow(pipe, 2.2), 1.0 / 2.2);
     }
-    return 1.3 * per_sm * (all / nseg) * ((double)ny / nb + 0.35) + 0.89 * march;
+    return 1.3 * per_sm * w.mean * ((double)ny / nb + 0.35) + 0.89 * march;
 }
 // Its bands in blocks of one warp: the cheapest of 1 to 32 rows.
 int short_bands(int nx, int ny, int width, int occupancy, int sms) {
@@ -708,6 +714,21 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
                                lbm::step_occupancy<double>(bx, mask), sms)) {
             bx = 32;
             nb = bands;
+        }
+    }
+    // FP64: not a few blocks more than one wave.  The second wave then takes almost as
+    // long as the first, by how blocks happen to end (the same shape went from 710 to
+    // 875 us a step at 619 x 2512 with another build of the kernel).  In place of one to two
+    // waves, one, 2048 x 879 729 -> 606 us, 2500 x 461 520 -> 407, 1024 x 2930
+    // 1060 -> 975; or, where the last segment is the lighter one, four waves of shorter
+    // bands, which even out, 619 x 2262 638 -> 529, 300 x 6001 862 -> 770, 800 x 1751
+    // 704 -> 542, 850 x 2706 888 -> 848.
+    if (f64 && automatic && bx == 128) {
+        const int segs = (p->nx + seg_width(bx) - 1) / seg_width(bx);
+        const long long wave = (long long)sms * lbm::step_occupancy<double>(bx, solid_mask != nullptr);
+        if ((long long)segs * nb > wave && (long long)segs * nb < 2 * wave && segs <= wave) {
+            const bool light = RowWarps(p->nx, seg_width(bx), sms).mean < seg_width(bx) / 64;
+            nb = (int)std::min<long long>((light ? 4 : 1) * wave / segs, std::max(nb, p->ny / 3));
         }
     }
     if (nb > 65535) nb = 65535;  // grid.y limit

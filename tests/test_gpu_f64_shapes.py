@@ -30,3 +30,28 @@ def test_automatic_shape_is_no_slower(nx, ny, block_x):
         times.append(best)
         g.close()
     assert times[0] <= 1.08 * times[1], times
+
+
+@pytest.mark.parametrize("nx,ny,bands", [(619, 2512, 152), (2048, 879, 57), (2500, 461, 45), (619, 2262, 152)])
+def test_no_short_second_wave(nx, ny, bands):
+    """A few blocks more than one wave against bands that make one (three blocks of 128
+    threads on each of 152 SMs): at most 1.08 times."""
+    import torch
+    from paper_2103_02119_gb300.lbm import Lattice
+    wl = _flow(nx, ny, "periodic")
+    times = []
+    for kw in ({}, dict(block_x=128, bands=bands)):
+        g = Lattice.from_workload(wl, precision=64, stream=torch.cuda.current_stream(), **kw)
+        g.step(5)
+        best = 1e9
+        for _ in range(6):
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            torch.cuda.synchronize()
+            e[0].record()
+            g.step(10)
+            e[1].record()
+            torch.cuda.synchronize()
+            best = min(best, e[0].elapsed_time(e[1]))
+        times.append(best)
+        g.close()
+    assert times[0] <= 1.08 * times[1], times
