@@ -139,10 +139,10 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
  * once per starting buffer (on a stream of its own; lbm_set_force drops
  * it).  Small lattices run many steps per launch (lbm_set_small_path), and so
  * do FP32 lattices below 200,000 cells in calls of at least 3 steps (14 up to
- * 20,480 cells, else 4 above 450 columns) where a CTA's rows, two or more of them, fit
- * its shared memory (up to 596 columns; 560 without a mask where 200 rows or fewer make
- * more than 20,480 cells) and the device takes the launch: a cooperative one of up to
- * 1024 steps.
+ * 20,480 cells, else 5 above 400 columns by up to 304 rows) where a CTA's rows, two
+ * or more of them, fit its shared memory (up to 596 columns; 560 without a mask
+ * where 200 rows or fewer make more than 20,480 cells) and the device takes the
+ * launch: a cooperative one of up to 1024 steps.
  * Larger FP32 ones (from 80,000 cells) take two steps per launch but for the last one
  * or two of a call; but not where the replayed graph of the row-band kernel is the
  * faster one: lattices of at most 64 columns between walls at rest from 380,000 cells

@@ -427,15 +427,20 @@ constexpr int kRunSteps = 50;
 // Shortest run of steps for the many-step kernel of a middle-sized lattice.  Its
 // launch reads and writes the state on top of its steps; us of a call, that /
 // a launch per step: 256 x 256 2 steps 15.5 / 16.5, 3 steps 19.5 / 24.7, 8 steps
-// 40 / 66; 16 x 2000 3 steps 15.5 / 64.6; 350 x 350 3 steps 26.4 / 31.5; but the wide
-// rows of 500 x 100 3 steps 28.2 / 26.1, 4 steps 34 / 34, of 596 x 100 31.8 / 28.8 and
-// 38 / 38.  Up to 20,480 cells calls of fewer than 14 steps stay a launch per step
-// although 100 x 100 takes 35 / 66 for 8: the comparisons of the row-band kernel with the
-// oracle step such lattices 7 and 13 at a time and count the launches.
-constexpr int kBandSteps = 3, kBandStepsWide = 4, kBandWide = 450, kBandStepsFew = 14;
+// 40 / 66; 16 x 2000 3 steps 15.5 / 64.6; 350 x 350 3 steps 26.4 / 31.5, 440 x 440
+// 31.8 / 38.1; but the wide rows of flat lattices, which the row-band kernel steps by a block
+// a row, 500 x 100 3 steps 28.2 / 26.1, 4 steps 34 / 34, 411 x 69 28.2 / 25.2 and
+// 35.6 / 33.6, 437 x 67 30.9 / 25.8 and 36.8 / 33.6 (an odd number of rows leaves a CTA
+// three), 596 x 100 31.8 / 28.8 and 38 / 38.  Up to 20,480 cells calls of fewer
+// than 14 steps stay a launch per step although 100 x 100 takes 35 / 66 for 8: the
+// comparisons of the row-band kernel with the oracle step such lattices 7 and 13 at a
+// time and count the launches.
+constexpr int kBandSteps = 3, kBandStepsFlat = 5, kBandStepsFew = 14;
+constexpr int kFlatColumns = 400, kFlatRows = 304;
 constexpr long long kBandFewCells = 20480;
 int band_steps(const lbm_handle* h) {
-    return h->N <= kBandFewCells ? kBandStepsFew : h->p.nx > kBandWide ? kBandStepsWide : kBandSteps;
+    if (h->N <= kBandFewCells) return kBandStepsFew;
+    return h->p.nx > kFlatColumns && h->p.ny <= kFlatRows ? kBandStepsFlat : kBandSteps;
 }
 
 void drop_run_graphs(lbm_handle* h) {

@@ -9,7 +9,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("nx,ny,kind,steps,launches", [
-    (450, 100, "walls", 3, 1), (451, 100, "walls", 3, 3), (451, 100, "walls", 4, 1), (451, 100, "walls_mask", 3, 3),
+    (400, 100, "walls", 3, 1), (401, 100, "walls", 4, 4), (401, 100, "walls", 5, 1), (401, 100, "walls_mask", 4, 4),
+    (440, 180, "periodic", 4, 4), (440, 304, "periodic", 4, 3), (440, 306, "periodic", 3, 1), (437, 67, "periodic", 4, 4),
     (560, 60, "periodic", 60, 1), (561, 60, "periodic", 9, 9), (561, 60, "periodic_mask", 9, 1),
     (596, 200, "force", 9, 5), (596, 202, "force", 9, 1), (590, 8, "periodic", 14, 1)])
 def test_route_and_states(nx, ny, kind, steps, launches):
