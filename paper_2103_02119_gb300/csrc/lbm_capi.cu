@@ -292,6 +292,13 @@ AuxParams aux_of(const lbm_params& q, const Geometry& g) {
     a.hFx32 = 0.5f * (float)q.Fx;
     a.hFy32 = 0.5f * (float)q.Fy;
     a.inv_nx = ~0ull / (unsigned long long)q.nx + 1ull;  // (nx >= 3)
+    if ((long long)q.nx * q.ny < (1LL << 31)) {
+        // exact below 2^31: the error of div_mul / 2^div_shift is below 2^-31 / nx
+        int bits = 0;
+        while ((1LL << bits) < q.nx) ++bits;
+        a.div_shift = 31 + bits;
+        a.div_mul = (unsigned)(((1ull << a.div_shift) + q.nx - 1) / q.nx);
+    }
     a.lmask = g.lmask;
     return a;
 }

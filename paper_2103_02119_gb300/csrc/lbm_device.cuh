@@ -128,6 +128,8 @@ struct AuxParams {
     double w3, w4, w5;        // relaxation rates of the second-order moments
     float a32, cs232, iah232, rho032, hFx32, hFy32;  // a, cs2, 1/(2a^2), rho0, F/2 in FP32
     unsigned long long inv_nx;  // ceil(2^64 / nx)
+    unsigned div_mul;           // below 2^31 cells ceil(2^div_shift / nx) (else div_shift = 0)
+    int div_shift;
     const uint8_t* __restrict__ lmask;
 };
 

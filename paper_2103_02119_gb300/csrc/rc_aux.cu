@@ -57,12 +57,15 @@ struct Feq32 {
              x += gridDim.x * blockDim.x)
 
 // Cells c, consecutive over a block and from one row to the next, with their row and
-// column: the row by a multiplication with ceil(2^64 / nx), exact while nx times the
-// number of cells stays below 2^64.  (Tiles of one row of 256 columns, or of 2 to 8
+// column: the row by a multiplication with the reciprocal of nx, one of 32 by 32 bits
+// below 2^31 cells, else of 64 by 64 with ceil(2^64 / nx), exact while nx times the
+// number of cells stays below 2^64 (the latter at every size cost the read-outs of a
+// 2048 x 2047 lattice 2 %).  Tiles of one row of 256 columns, or of 2 to 8
 // rows of 128 to 32, need no multiplication but leave most threads of a narrow lattice
 // without a cell: 3 x 100000, lbm_get_f 62 us against 25, FP64 lbm_diagnostics 435 / 79;
-// 2049 x 2048 with obstacles, FP64, 123 / 112 and 578 / 550.)
+// 2049 x 2048 with obstacles, FP64, 123 / 112 and 578 / 550.
 __device__ __forceinline__ int row_of(const AuxParams& p, long long c) {
+    if (p.div_shift) return (int)((unsigned long long)(unsigned)c * p.div_mul >> p.div_shift);
     return (int)__umul64hi((unsigned long long)c, p.inv_nx);
 }
 #define LBM_FOR_ALL_CELLS(p, c)                                                          \
