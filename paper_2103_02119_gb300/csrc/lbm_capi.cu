@@ -491,6 +491,15 @@ lbm_status ensure_run_graph(lbm_handle* h, const KParams<T>& k, int from) {
     return LBM_OK;
 }
 
+// Whether runs of steps can be replayed on the stream: not while it is being captured,
+// which takes the launches themselves but no launch of a graph.
+cudaError_t replayable(cudaStream_t s, bool& yes) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(s, &st);
+    yes = st == cudaStreamCaptureStatusNone;
+    return e;
+}
+
 template <typename T>
 lbm_status step_lattice(lbm_handle* h, int64_t nsteps) {
     const KParams<T> k = kparams<T>(h);
@@ -536,9 +545,11 @@ lbm_status step_lattice(lbm_handle* h, int64_t nsteps) {
             }
         return LBM_OK;
     };
+    bool runs = left >= kRunSteps;
+    if (runs) CK(h, replayable(h->stream, runs), "cudaStreamIsCapturing");
     if (!h->runs_first)
         if (lbm_status st = chain(); st != LBM_OK) return st;
-    while (left >= kRunSteps) {
+    while (runs && left >= kRunSteps) {
         if (lbm_status st = ensure_run_graph<T>(h, k, h->cur); st != LBM_OK) return st;
         CK(h, cudaGraphLaunch(h->graph[h->cur], h->stream), "cudaGraphLaunch");
         left -= kRunSteps;
@@ -546,10 +557,14 @@ lbm_status step_lattice(lbm_handle* h, int64_t nsteps) {
         h->steps += kRunSteps;
     }
     if (lbm_status st = chain(); st != LBM_OK) return st;
-    CK(h, launch_steps_of<T>(h, k, h->cur, (int)left, h->stream), "step kernel");
-    h->cur ^= (int)(left & 1);
-    h->launches += left;
-    h->steps += left;
+    while (left > 0) {
+        const int n = left < (1 << 20) ? (int)left : (1 << 20);
+        CK(h, launch_steps_of<T>(h, k, h->cur, n, h->stream), "step kernel");
+        h->cur ^= n & 1;
+        h->launches += n;
+        h->steps += n;
+        left -= n;
+    }
     return LBM_OK;
 }
 
@@ -2053,6 +2068,8 @@ lbm_status advance(lbm_batch* b, int64_t nsteps, bool graphs) {
         parity ^= 1;
         left -= 2;
     }
+    graphs = graphs && left >= kGraphSteps;
+    if (graphs) BCK(b, replayable(b->stream, graphs), "cudaStreamIsCapturing");
     while (graphs && left >= kGraphSteps) {
         if (lbm_status s = ensure_graph(b, parity); s != LBM_OK) return s;
         BCK(b, cudaGraphLaunch(b->graph[parity], b->stream), "cudaGraphLaunch");
