@@ -77,10 +77,10 @@ __device__ __forceinline__ int row_of(const AuxParams& p, long long c) {
 // read-out kernels are bound by them, and by conversions, which take the same
 // lanes.  So they spend FP64 on what needs it and the rest on integers.
 // Measured on 2048 x 2047 FP32 cells with obstacles, against sums, conversions
-// and divisions in FP64: lbm_stress 455 against 2085 us (558 with the conversion
+// and divisions in FP64: lbm_stress 445 against 2010 us (558 with the conversion
 // instruction for the sums, 516 with ten FP64 operations more in its algebra),
-// lbm_diagnostics after a step 335 against 1260 us (375), lbm_get_f 84 against 146 us,
-// lbm_set_f 91 against 143 us, lbm_moments 51 against 68 us; the residual check of a
+// lbm_diagnostics after a step 337 against 1153 us (375), lbm_get_f 105 against 145 us,
+// lbm_set_f 95 against 146 us, lbm_moments 52 against 69 us; the residual check of a
 // 96-lattice batch 0.80 against 2.56 ms (0.86).
 
 // float -> double, exact, on the integer pipe, without a branch (a conversion
@@ -425,8 +425,9 @@ set_f_kernel(T* __restrict__ f, const AuxParams p, const double* __restrict__ fi
     }
 }
 
+// (six blocks an SM: at 44 registers, five, FP64 1000 x 1000 took 26.4 us, at 40 24.7)
 template <typename T, bool MASK>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 6)
 get_f_kernel(const T* __restrict__ f, const AuxParams p, double* __restrict__ fout) {
     const long long N = (long long)p.nx * p.ny;
     LBM_FOR_ALL_CELLS(p, c) {
