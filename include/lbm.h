@@ -137,8 +137,9 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
 /* Advance nsteps >= 0 time steps (collide + stream, Sec. 4), one kernel
  * launch per step; runs of 50 steps replay a CUDA graph the handle captures
  * once per starting buffer (on a stream of its own; lbm_set_force drops
- * it).  Small lattices run many steps per launch (lbm_set_small_path), and so
- * do FP32 lattices below 200,000 cells in calls of at least 3 steps (14 up to
+ * it; on a stream that is being captured the steps are launched one by one).
+ * Small lattices run many steps per launch (lbm_set_small_path), and so do
+ * FP32 lattices below 200,000 cells in calls of at least 3 steps (14 up to
  * 20,480 cells, else 5 above 400 columns by up to 304 rows) where a CTA's rows, two
  * or more of them, fit its shared memory (up to 596 columns; 560 without a mask
  * where 200 rows or fewer make more than 20,480 cells) and the device takes the

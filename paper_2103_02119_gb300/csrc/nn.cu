@@ -13,12 +13,17 @@
 //                partial sums added in a fixed order), transposed so that the
 //                taps and input channels fill the 128 rows of the MMA:
 //                A[(tap, ci)][p] = in(p + s(tap))[ci], B[co][p] = g(p)[co]
-// with s(tap) = (dy - 1, dx - 1) and zeros outside the grid.  A CTA of 128
-// threads computes a 128 x N tile (N = 16 .. 256): the threads gather K
-// chunks of 64 into two shared-memory buffers in the tensor core's K-major
-// core-matrix layout, one thread issues the MMAs of a chunk and commits them
-// to the buffer's mbarrier, and each warp reads its 32 rows of the
-// accumulator back with tcgen05.ld.
+// with s(tap) = (dy - 1, dx - 1) and zeros outside the grid.
+// Forward and input gradient go over tiles of pixels (conv_tile_kernel) where the
+// channels come in steps of 16 and the tile fits shared memory: a CTA of 256 threads
+// copies 128 positions and their neighbours once, a tap's operand A is a start
+// address in that tile, and one thread issues the MMAs of a tap as its weights land.
+// The weight gradient, and the convolutions that the tiles do not take, go by
+// umma_gemm_kernel: a CTA of 128 threads computes a 128 x N tile (N = 16 .. 256);
+// the threads copy K chunks of 64 (cp.async) into a ring of three or four
+// shared-memory stages in the tensor core's core-matrix layout, and one thread issues
+// the MMAs of a chunk and commits them to the stage's mbarrier.  In both each warp
+// reads its rows of the accumulator back with tcgen05.ld.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
