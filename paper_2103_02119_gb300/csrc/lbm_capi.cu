@@ -798,6 +798,25 @@ lbm_status lbm_create(const lbm_params* p, const uint8_t* solid_mask, void* cuda
             (rows == 2 && sides && !mask);
         if (rows == 1 && sides && !mask) h->chain_bands = 0;
     }
+    // And a lattice of 169 to 192 or 225 to 256 columns between walls at rest without
+    // obstacles: one segment of three or four full warps of the row-band kernel, but four or
+    // five strips of the two-step kernel, the last one nearly empty, while the state stays in
+    // the L2 and halving its traffic saves nothing; us a step of calls of 100, two-step /
+    // row-band kernel: 172 x 3488 17.8 / 15.5, 184 x 3532 18.4 / 15.7, 192 x 5208 21.5 / 19.4,
+    // 232 x 2586 16.4 / 13.9, 250 x 2600 16.4 / 14.7, but 232 x 3232 16.5 / 17.4 (either
+    // side is the faster one by how its bands fill the SMs; 140 such lattices in
+    // the range take 1.03 times the row-band kernel's time in the two-step kernel in the
+    // mean, 1.17 at most); below 480,000 cells 184 x 2500 14.1 / 15.0, 232 x 1982 12.6 /
+    // 14.9 (178 x 2584 9 % the other way), above 1.5 million 184 x 8423 28.4 / 28.8.
+    // With 193 to 224 columns, with obstacles, moving walls or periodic along x the two-step
+    // kernel is the faster one throughout, and in calls of fewer than 50 steps.
+    if (h->chain_bands && automatic && !solid_mask && h->N >= 480000 && h->N <= 1500000 &&
+        bx == 128 && p->nx > 128 && p->nx <= seg_width(128)) {
+        const KParams<float> k = kparams<float>(h);
+        const int strips = (p->nx + lbm::kChainColumns - 1) / lbm::kChainColumns;
+        h->runs_first |= !k.px && !k.moving &&
+                         strips * lbm::kChainColumns > (p->nx + 63) / 64 * 64;
+    }
     // small lattices: all the steps of an lbm_step call in one launch of one
     // thread-block cluster, when the device can hold it
     if (h->N <= lbm::kSmallCells && !kRowInterleaved) {
