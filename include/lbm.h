@@ -147,8 +147,9 @@ lbm_status lbm_init_fields(lbm_handle* h, const double* rho, const double* ux,
  * Larger FP32 ones (from 80,000 cells) take two steps per launch but for the last one
  * or two of a call; but not where the replayed graph of the row-band kernel is the
  * faster one: lattices of at most 64 columns between walls at rest from 380,000 cells
- * on, and below 200,000 cells some with walls along x or moving walls, for runs of 50
- * steps or for all.  The states are bit for bit the same.  Asynchronous: the return
+ * on, of 169 to 192 or 225 to 256 of 0.48 to 1.5 million cells without a mask (runs of
+ * 50 steps), and below 200,000 cells some with walls along x or moving walls, for runs
+ * of 50 steps or for all.  The states are bit for bit the same.  Asynchronous: the return
  * value reports launch errors only. */
 lbm_status lbm_step(lbm_handle* h, int64_t nsteps);
 
